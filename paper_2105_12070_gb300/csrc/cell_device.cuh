@@ -13,12 +13,14 @@
 
 #include "../../include/chemgpu.h"
 #include "chem_internal.h"
+#include "fixed_math.cuh"
 
 using namespace chemgpu;
 namespace {
 
 constexpr double kRu = 8.314462618e7;  // erg/(mol K)
 constexpr double kPatm = 1.01325e6;    // dyn/cm^2
+constexpr int64_t kFxLog2PatmRu = -28636412686642908LL;  // log2(Patm / Ru) * 2^52
 constexpr double kLnPatmRu = -4.4074185890025275;  // ln(Patm / Ru), Patm/Ru in mol K / cm^3
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -159,17 +161,21 @@ struct Grp {
     for (int i = 1; i < G; ++i) s += r[i];
     return s;
   }
-  // two sums at once (one exchange)
+  // two sums at once (one exchange): the first exchange leaves a's partial sums in the lower half
+  // of the warp and b's in the upper, so both take 5 additions instead of 10
   __device__ void sum2(double& a, double& b) const {
+    const bool upper = lane() >= 16;
+    double v = (upper ? b : a) + __shfl_xor_sync(kFull, upper ? a : b, 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(kFull, a, o);
-      b += __shfl_xor_sync(kFull, b, o);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    if (G == 1) {
+      a = __shfl_sync(kFull, v, 0);
+      b = __shfl_sync(kFull, v, 16);
+      return;
     }
-    if (G == 1) return;
     double* r = red + (parity & 1) * 3 * G;
     parity++;
-    if (lane() == 0) { r[2 * warp()] = a; r[2 * warp() + 1] = b; }
+    if ((lane() & 15) == 0) r[2 * warp() + (upper ? 1 : 0)] = v;
     sync();
     a = r[0];
     b = r[1];
@@ -344,7 +350,7 @@ __device__ inline EvalMem<double> eval_mem(const CellMem& w) {
 
 template <class S>
 struct CellScalarsT {
-  S T, invT, lnT, rho, inv_rho, Wbar, cp, dcp_dT, fT;
+  S T, invT, rho, inv_rho, Wbar, cp, inv_cp, dcp_dT, fT;
 };
 using CellScalars = CellScalarsT<double>;
 
@@ -498,23 +504,60 @@ __device__ inline void troe(const double* fo, S T, S invT, S Pr, S& F, S& dlF, S
   }
 }
 
+// The same in FP64 with the exponentials and logarithms in fixed point: fd[i * n] = 1 - alpha, alpha,
+// log2(e)/T3, log2(e)/T1, T2 log2(e).  A centre or reduced pressure that is not a positive normal
+// number takes the library logarithm (minus infinity or NaN, as there).
+static __device__ __noinline__ double log10_wide(double x) { return log10(x); }
+__device__ inline double log10_fx(double x) {
+  return fx_log2_takes(x) ? fx_value(fx_log2(x)) * 0.30102999566398119521 : log10_wide(x);
+}
+__device__ inline void troe_fx(const double* fd, int n, double T, double invT, double Pr, double& F, double& dlF,
+                               double& dlnF_dT, bool jac) {
+  const double oma = fd[0], a = fd[n], iT3 = fd[2 * n], iT1 = fd[3 * n], T2 = fd[4 * n];
+  const double e3 = fx_exp2_of(-T * iT3), e1 = fx_exp2_of(-T * iT1), e2 = fx_exp2_of(-T2 * invT);
+  const double Fcent = fma(oma, e3, fma(a, e1, e2));
+  const double L = log10_fx(Fcent);
+  const double nn = fma(-1.27, L, 0.75);
+  const double xc = log10_fx(Pr) + fma(-0.67, L, -0.4);
+  const double den = fma(-0.14, xc, nn);
+  const double iden = rcp_newton(den);
+  const double f1 = xc * iden;
+  const double ig = rcp_newton(fma(f1, f1, 1.0));
+  const double Lg = L * ig;
+  F = fx_exp2_of(Lg * 3.3219280948873623479);
+  if (jac) {
+    const double t = f1 * ig * Lg;  // L f1 / g^2
+    const double iden2 = iden * iden;
+    dlF = -2.0 * t * (nn * iden2);
+    // d Fcent / dT; the table's exponents carry log2(e): times ln 2
+    const double dFc = 0.69314718055994530942 * (T2 * (invT * invT) * e2 - (oma * iT3 * e3 + a * iT1 * e1));
+    const double dL = dFc * rcp_newton(Fcent);  // ln(10) dL/dT
+    const double df1_dL = fma(-0.67, den, xc * (1.27 - 0.14 * 0.67)) * iden2;
+    dlnF_dT = fma(-2.0 * t, df1_dL, ig) * dL;
+  }
+}
+
 // Evaluates f(y) into f[0..N).  With jac, also leaves per-reaction derivative data in
-// scr[u * R + r], u = 0..7: {dq/dC at the 4 distinct slot species, phi (coefficient of the
-// efficiencies), sum_j dq/dC_j C_j, dq/dT at fixed C, reaction enthalpy (erg/mol)} (rows of R,
-// so that the threads of consecutive reactions store to consecutive words), and the species
-// production rates in w.omega.
+// scr[u * R + r], u = 0..6: {dq/dC through each of the 4 slots (an empty slot's entry is not read),
+// phi (coefficient of the efficiencies; pressure-dependent reactions only), sum_j dq/dC_j C_j,
+// dq/dT at fixed C} (rows of R, so that the threads of consecutive reactions store to consecutive
+// words), and the species production rates in w.omega.
 // With kP (adjoint use, requires jac) it also writes P[r] = v . d f / d ln A_r for the weight
 // vector v = vP (N): with q'_r = d q_r / d ln A_r (q_r for elementary and third-body
 // reactions; q_r (Pr/(1+Pr) - d ln F/d ln Pr) for fall-off reactions, whose A is that of
 // k_inf), P_r = (q'_r / rho) (sum_{k<K} nu_kr W_k v_Yk - v_T dH_r / cp).
+//
+// This is the general form: any scalar type and any state.  FP64 states inside the mechanism's
+// fixed-point range take cell_rates_fx below.
 template <int G, class S, bool kP = false>
-__device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
-                                      const EvalMem<S>& w, S* scr, bool jac, const double* vP = nullptr,
-                                      S* P = nullptr) {
+__device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
+                                          const EvalMem<S>& w, S* scr, bool jac, const double* vP = nullptr,
+                                          S* P = nullptr) {
   constexpr int NT = Grp<G>::NT;
   const int K = m.K, d = K - 1;
   CellScalarsT<S> s;
   s.T = y[0];
+  S lnT;
   // mass fractions, mean molar mass, density, concentrations, thermo
   S ysum = cst<S>(0.0), yw = cst<S>(0.0);
   for (int k = g.t; k < d; k += NT) {
@@ -539,13 +582,13 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     }
     g.sync();
     s.invT = w.bc[0];
-    s.lnT = w.bc[1];
+    lnT = w.bc[1];
     s.Wbar = w.bc[2];
     s.rho = w.bc[3];
     s.inv_rho = w.bc[4];
   } else {
     s.invT = 1.0 / s.T;
-    s.lnT = log(s.T);
+    lnT = log(s.T);
     s.Wbar = 1.0 / yw;
     s.rho = p * s.Wbar / (kRu * s.T);
     s.inv_rho = yw * kRu * s.T / p;
@@ -557,7 +600,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     w.C[k] = s.rho * Yk * sp[1];
     const double* a = (val(s.T) <= sp[2]) ? sp + 3 : sp + 10;
     S cpR, hRT, sR, dcpR;
-    nasa7(a, s.T, s.invT, s.lnT, cpR, hRT, sR, dcpR);
+    nasa7(a, s.T, s.invT, lnT, cpR, hRT, sR, dcpR);
     w.cpR[k] = cpR;
     w.hRT[k] = hRT;
     w.gRT[k] = hRT - sR;
@@ -567,6 +610,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
   }
   g.sum2(cp, dcp);
   s.cp = cp * kRu;
+  s.inv_cp = 1.0 / s.cp;
   s.dcp_dT = dcp * kRu;
   g.sync();
   // third-body concentrations [M]_r = sum_k eff_rk C_k of the pressure-dependent reactions
@@ -585,7 +629,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     w.M[r] = (a0 + a1) + (a2 + a3);
   }
   g.sync();
-  const S ln_patm_rut = kLnPatmRu - s.lnT;  // ln(Patm / (Ru T))
+  const S ln_patm_rut = kLnPatmRu - lnT;  // ln(Patm / (Ru T))
   // reactions: warp 0 takes [0, split) (the fall-off reactions, whose Troe branch is long, lead
   // the device order), the other warps [split, R); the split balances the warps' iteration costs
   // (split 0: reaction r goes to thread r mod 32 G)
@@ -604,7 +648,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     const S Ca0 = w.C[a0], Ca1 = (a1 >= 0) ? w.C[a1] : cst<S>(1.0);
     const S Cp0 = w.C[p0], Cp1 = (p1 >= 0) ? w.C[p1] : cst<S>(1.0);
     const S pf = Ca0 * Ca1, pr = Cp0 * Cp1;
-    const S lkinf = fma(rd[1], s.lnT, rd[0]) - rd[2] * s.invT;
+    const S lkinf = fma(rd[1], lnT, rd[0]) - rd[2] * s.invT;
     S kf = exp_fast(lkinf);
     S dG = w.gRT[p0] - w.gRT[a0];
     if (p1 >= 0) dG += w.gRT[p1];
@@ -622,7 +666,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     if (fo) {
       fop = m.fo + (size_t)r * kFoDoubles;
       // k0 / k_inf as one exponential of the difference of the logarithms (no quotient)
-      const S ratio = exp_fast(fma(fop[1], s.lnT, fop[0]) - fop[2] * s.invT - lkinf);
+      const S ratio = exp_fast(fma(fop[1], lnT, fop[0]) - fop[2] * s.invT - lkinf);
       k0 = ratio * kf;
       Pr = ratio * Mr;
       if (fop[7] != 0.0) troe(fop, s.T, s.invT, Pr, F, dlF, dlnF_dT, jac);
@@ -652,23 +696,16 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
         phi = kf * pf - kr * pr;
       }
       const S dqdT = mfac * (kf * dlnk * pf - kr * (dlnk - dlnKc_dT) * pr);
-      S DC = phi * Mr;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = ii[4 + u];
-        S D = cst<S>(0.0);
-        if (j >= 0) {
-          const S dpf = (a0 == j ? Ca1 : cst<S>(0.0)) + (a1 == j ? Ca0 : cst<S>(0.0));
-          const S dpr = (p0 == j ? Cp1 : cst<S>(0.0)) + (p1 == j ? Cp0 : cst<S>(0.0));
-          D = mfac * (kf * dpf - kr * dpr);
-          DC = fma(D, w.C[j], DC);
-        }
-        o[u * R] = D;
-      }
+      // q = R_f - R_r, each proportional to the concentrations of its side's slots
+      const S kfm = mfac * kf, krm = mfac * kr;
+      const S Rf = kfm * pf, Rr = krm * pr;
+      o[0] = kfm * Ca1;
+      o[R] = kfm * Ca0;
+      o[2 * R] = -krm * Cp1;
+      o[3 * R] = -krm * Cp0;
       o[4 * R] = phi;
-      o[5 * R] = DC;
+      o[5 * R] = fma(phi, Mr, ((a1 >= 0) ? Rf + Rf : Rf) - ((p1 >= 0) ? Rr + Rr : Rr));
       o[6 * R] = dqdT;
-      o[7 * R] = dH * kRu * s.T;
       if (kP) {
         double gw = 0.0;  // sum over the species rows of nu_kr W_k v_Yk
 #pragma unroll
@@ -677,7 +714,7 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
           if (k >= 0) gw = fma(rd[3 + u] * m.sp[k * kSpDoubles], vP[1 + k], gw);
         }
         const S dq = fo ? q * (Pr * inv1p - dlF) : q;
-        P[r] = dq * s.inv_rho * (gw - vP[0] * (o[7 * R] / s.cp));
+        P[r] = dq * s.inv_rho * (gw - vP[0] * (dH * kRu * s.T * s.inv_cp));
       }
     }
   }
@@ -700,10 +737,232 @@ __device__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double 
     if (k < d) f[1 + k] = m.sp[k * kSpDoubles] * om * s.inv_rho;
   }
   const S Q = g.sum(Qp) * kRu * s.T;
-  s.fT = -Q * s.inv_rho / s.cp;
+  s.fT = -Q * s.inv_rho * s.inv_cp;
   if (g.t == 0) f[0] = s.fT;
   g.sync();
   return s;
+}
+
+// The same evaluation for FP64 states whose temperature lies in the mechanism's fixed-point range:
+// the logarithms of the rate and equilibrium constants are summed in 64-bit fixed point and the
+// exponentials and logarithms evaluated there (fixed_math.cuh), from tables with the constant
+// factors multiplied in.  Bound by FP64 issue (64 clocks per warp instruction and sub-partition):
+// a plain reaction takes 5 FP64 instructions here against 39 in the general form, a species' thermo
+// 17 against about 45.
+// The tables are laid out so that consecutive threads read consecutive words: at this pace the
+// strided records of the general form would be bound by L1 wavefronts.
+template <int G, bool kP>
+__device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p, const double* y, double* f,
+                                     const EvalMem<double>& w, double* scr, bool jac, const double* vP, double* P) {
+  constexpr int NT = Grp<G>::NT;
+  const int K = m.K, R = m.R, d = K - 1, npd = m.n_pd, nfo = m.n_fo;
+  const double* sp = m.spf;
+  CellScalars s;
+  s.T = y[0];
+  double ysum = 0.0, yw = 0.0;
+  for (int k = g.t; k < d; k += NT) {
+    const double Yk = y[1 + k];
+    ysum += Yk;
+    yw = fma(Yk, sp[K + k], yw);
+  }
+  g.sum2(ysum, yw);
+  const double Yd = 1.0 - ysum;
+  yw = fma(Yd, sp[K + d], yw);
+  // the reciprocals of T, yw and p on three lanes of each warp: one Newton iteration for all three
+  const int third = g.lane() & 3;
+  const double a3 = third == 0 ? s.T : third == 1 ? yw : p;
+  uint64_t rT;
+  const double rcp = fx_rcp(a3, rT);
+  s.invT = __shfl_sync(kFull, rcp, 0);
+  s.Wbar = __shfl_sync(kFull, rcp, 1);
+  const double invp = __shfl_sync(kFull, rcp, 2);
+  s.rho = (p * s.Wbar) * (s.invT * (1.0 / kRu));
+  s.inv_rho = (yw * s.T) * (kRu * invp);
+  const fx_t L2 = fx_log2(s.T);
+  // 1/T in units of 2^-70, with the reciprocal's 62 bits (T in (128, 8192): exponent 7 to 12)
+  const int64_t iT = (int64_t)(__shfl_sync(kFull, (unsigned long long)rT, 0) >>
+                               ((int)(__double_as_longlong(s.T) >> 52) - 1029));
+  const int64_t L2s = L2 << 7;
+  double cp = 0.0, dcp = 0.0;
+  int64_t* g2 = reinterpret_cast<int64_t*>(w.gRT);  // (g/RT) / ln 2 as fx
+  for (int k = g.t; k < K; k += NT) {
+    const double Yk = (k < d) ? y[1 + k] : Yd;
+    const double yiw = Yk * sp[K + k];
+    const double* a = sp + (size_t)(3 + (s.T <= sp[2 * K + k] ? 0 : kSpfRange)) * K + k;
+    auto c = [&](int i) { return a[(size_t)i * K]; };
+    const double T = s.T;
+    const double cpR = fma(T, fma(T, fma(T, fma(T, c(4), c(3)), c(2)), c(1)), c(0));
+    const double hRT = fma(T, fma(T, fma(T, fma(T, c(8), c(7)), c(6)), c(5)), fma(c(9), s.invT, c(0)));
+    auto cx = [&](int i) { return __double_as_longlong(c(i)); };
+    const double gT = T * fma(T, fma(T, fma(T, c(16), c(15)), c(14)), c(13));
+    w.C[k] = s.rho * yiw;
+    w.cpR[k] = cpR;
+    w.hRT[k] = hRT;
+    g2[k] = cx(10) + fx_mulhi(cx(11), L2s) + 2 * fx_mulhi(cx(12), iT) + fx_of(gT);
+    cp = fma(yiw, cpR, cp);
+    if (jac) {
+      const double dcpR = fma(T, fma(T, fma(T, c(19), c(18)), c(17)), c(1));
+      dcp = fma(yiw, dcpR, dcp);
+    }
+  }
+  if (jac) g.sum2(cp, dcp);
+  else cp = g.sum(cp);
+  s.cp = cp * kRu;
+  s.inv_cp = rcp_newton(s.cp);
+  s.dcp_dT = dcp * kRu;
+  if (G == 1) g.sync();  // (with several warps the reduction's barrier has published C and the thermo)
+  for (int r = g.t; r < npd; r += NT) {
+    const double* e = m.eff_t + r;
+    double a0 = 0.0, a1 = 0.0;
+    int k = 0;
+    for (; k + 1 < K; k += 2) {
+      a0 = fma(e[(size_t)k * npd], w.C[k], a0);
+      a1 = fma(e[(size_t)(k + 1) * npd], w.C[k + 1], a1);
+    }
+    if (k < K) a0 = fma(e[(size_t)k * npd], w.C[k], a0);
+    w.M[r] = a0 + a1;
+  }
+  g.sync();
+  const int64_t P2 = kFxLog2PatmRu - L2;  // log2(Patm / (Ru T))
+  const int split = (G == 1) ? 0 : m.rx_split[G == 2 ? 1 : G == 4 ? 2 : 3];
+  const int r_first = (split == 0) ? g.t : (g.warp() == 0) ? g.lane() : split + g.t - 32;
+  const int r_end = (split == 0 || g.warp() != 0) ? R : split;
+  const int r_step = (split == 0) ? NT : (g.warp() == 0) ? 32 : NT - 32;
+  for (int r = r_first; r < r_end; r += r_step) {
+    const uint32_t slots = m.rx4[r];
+    const int a0 = slots & 255, a1 = (slots >> 8) & 255, p0 = (slots >> 16) & 255, p1 = slots >> 24;
+    const bool two_r = a1 != 255, two_p = p1 != 255;
+    const double Ca0 = w.C[a0], Ca1 = two_r ? w.C[a1] : 1.0;
+    const double Cp0 = w.C[p0], Cp1 = two_p ? w.C[p1] : 1.0;
+    const double pf = Ca0 * Ca1, pr = Cp0 * Cp1;
+    // log2 of the forward constant, and of 1/Kc = exp(sum nu g/RT - dnu ln(Patm/(Ru T))); sums that
+    // wrap on the way are right modulo 2^64
+    const int64_t Xf = m.fxk[r] + fx_mulhi(m.fxk[R + r], L2s) - fx_mulhi(m.fxk[2 * R + r], iT);
+    const int dnu = (int)two_p - (int)two_r;
+    uint64_t Xc = (uint64_t)g2[p0] - (uint64_t)g2[a0];
+    if (two_p) Xc += (uint64_t)g2[p1];
+    if (two_r) Xc -= (uint64_t)g2[a1];
+    if (dnu != 0) Xc = dnu > 0 ? Xc - (uint64_t)P2 : Xc + (uint64_t)P2;
+    const bool pd = r < npd, fo = r < nfo;
+    double kf = fx_exp2(Xf), kr;
+    // reverse constant: directly from the summed logarithm, except for fall-off reactions
+    const double er = fx_exp2((fx_t)(fo ? Xc : Xc + (uint64_t)Xf));
+    double Mr = 1.0, mfac = 1.0;
+    double F = 1.0, dlF = 0.0, dlnF_dT = 0.0, dk_dM = 0.0, inv1p = 1.0, Pr = 0.0;
+    if (pd) Mr = w.M[r];
+    if (fo) {
+      const int64_t X0 = m.fxo[r] + fx_mulhi(m.fxo[nfo + r], L2s) - fx_mulhi(m.fxo[2 * nfo + r], iT);
+      const double ratio = fx_exp2(X0 - Xf);  // k0 / k_inf
+      Pr = ratio * Mr;
+      if (m.fo[(size_t)r * kFoDoubles + 7] != 0.0) troe_fx(m.fod + r, nfo, s.T, s.invT, Pr, F, dlF, dlnF_dT, jac);
+      inv1p = rcp_newton(1.0 + Pr);
+      const double kF = kf * (F * inv1p);
+      if (jac) dk_dM = ratio * kF * (inv1p + dlF);
+      kf = kF * Pr;
+      kr = kf * er;
+    } else {
+      kr = er;
+      if (pd) mfac = Mr;
+    }
+    double Rr = kr * pr;
+    if (!jac) {
+      double q = fma(kf, pf, -Rr);
+      if (pd) q *= mfac;
+      w.q[r] = q;
+    } else {
+      double Rf = kf * pf;
+      double q = Rf - Rr;
+      double* o = scr + r;  // o[u * R]
+      double DC = 0.0;
+      if (pd) {
+        double phi = q;  // plain third body: q / [M]
+        if (fo) {
+          phi = dk_dM * fma(-er, pr, pf);
+        } else {
+          kf *= mfac;
+          kr *= mfac;
+          Rf *= mfac;
+          Rr *= mfac;
+          q *= mfac;
+        }
+        o[4 * R] = phi;
+        DC = phi * Mr;
+      }
+      w.q[r] = q;
+      double dH = w.hRT[p0] - w.hRT[a0];
+      if (two_p) dH += w.hRT[p1];
+      if (two_r) dH -= w.hRT[a1];
+      const double dHn = dnu == 0 ? dH : dH - (dnu > 0 ? 1.0 : -1.0);
+      const double dlnKc_dT = dHn * s.invT;
+      double dlnk = fma(m.rxd_t[R + r], s.invT, m.rxd_t[r]) * s.invT;  // d ln k_inf / dT
+      if (fo) {
+        const double dlnk0 = fma(m.fo[(size_t)r * kFoDoubles + 2], s.invT, m.fo[(size_t)r * kFoDoubles + 1]) * s.invT;
+        dlnk = fma(inv1p + dlF, dlnk0 - dlnk, dlnk) + dlnF_dT;
+      }
+      o[0] = kf * Ca1;
+      o[R] = kf * Ca0;
+      o[2 * R] = -(kr * Cp1);
+      o[3 * R] = -(kr * Cp0);
+      // R_f and R_r are homogeneous in the concentrations of their side's slots
+      o[5 * R] = DC + ((two_r ? Rf + Rf : Rf) - (two_p ? Rr + Rr : Rr));
+      o[6 * R] = fma(q, dlnk, Rr * dlnKc_dT);
+      if (kP) {
+        const int* ii = m.rxi + r * kRxInts;
+        const double* rd = m.rxd + r * kRxDoubles;
+        double gw = 0.0;  // sum over the species rows of nu_kr W_k v_Yk
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = ii[8 + u];
+          if (k >= 0) gw = fma(rd[3 + u] * sp[k], vP[1 + k], gw);
+        }
+        const double dq = fo ? q * (Pr * inv1p - dlF) : q;
+        P[r] = dq * s.inv_rho * (gw - vP[0] * (dH * kRu * s.T * s.inv_cp));
+      }
+    }
+  }
+  g.sync();
+  // species production rates and the source term
+  double Qp = 0.0;
+  for (int k = g.t; k < K; k += NT) {
+    double om = 0.0;
+    const int len = m.sr_ptr[k + 1] - m.sr_ptr[k];
+    const uint32_t* e = m.srx + k;
+    for (int i = 0; i < len; ++i) {
+      const uint32_t v = e[(size_t)i * K];
+      om = fma(__hiloint2double((int)(v & 0xffff0000u), 0), w.q[v & 0xffffu], om);
+    }
+    w.omega[k] = om;
+    Qp = fma(w.hRT[k], om, Qp);
+    if (k < d) f[1 + k] = sp[k] * om * s.inv_rho;
+  }
+  const double Q = g.sum(Qp) * (kRu * s.T);
+  s.fT = -Q * s.inv_rho * s.inv_cp;
+  if (g.t == 0) f[0] = s.fT;
+  g.sync();
+  return s;
+}
+
+// The general form as a call (states outside the fixed-point range, rare in the solve): its code is
+// kept out of the kernels' loop, and its arguments are passed by value so that the caller's stay in registers.
+template <int G, bool kP>
+__device__ __noinline__ CellScalars cell_rates_wide(const DevMech& m, Grp<G> g, double p, const double* y, double* f,
+                                                    EvalMem<double> w, double* scr, bool jac, const double* vP,
+                                                    double* P) {
+  return cell_rates_any<G, double, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+}
+
+// f(y) and, with jac, the per-reaction derivative data (see cell_rates_any).
+template <int G, class S, bool kP = false>
+__device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
+                                                      const EvalMem<S>& w, S* scr, bool jac, const double* vP = nullptr,
+                                                      S* P = nullptr) {
+  if constexpr (std::is_same<S, double>::value) {
+    const double T = y[0];
+    if (T > m.fx_T[0] && T < m.fx_T[1]) return cell_rates_fx<G, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+    return cell_rates_wide<G, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+  } else {
+    return cell_rates_any<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+  }
 }
 
 // Assemble the analytical Jacobian (Sec. 2.3) at the state of the preceding cell_rates(jac)
@@ -845,8 +1104,8 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
     w.ccol[k] = -s.Wbar * (m.sp[k * kSpDoubles + 1] - invWd);
   }
   g.sync();
-  const S inv_rhocp = s.inv_rho / s.cp;
-  const S inv_cp = 1.0 / s.cp;
+  const S inv_cp = s.inv_cp;
+  const S inv_rhocp = s.inv_rho * inv_cp;
   const S fT = s.fT;
   // temperature row and column, then the species block (J now overwrites the scratch)
   const S ZQd = Z[d * N + d];
@@ -980,8 +1239,8 @@ __device__ void cell_jacobian_vjp(const DevMech& m, const Grp<G>& g, const CellS
   cpw = cpw * kRu;
   sB = sB * s.inv_rho;
   g.sync();
-  const S inv_rhocp = s.inv_rho / s.cp;
-  const S inv_cp = 1.0 / s.cp;
+  const S inv_cp = s.inv_cp;
+  const S inv_rhocp = s.inv_rho * inv_cp;
   const S fT = s.fT;
   const S sA = invWd * t[d];
   const S ZQd = zq[d];
@@ -1654,8 +1913,9 @@ __device__ void warp_lu_solve_s(const T* A, int N, const int* perm, const T* inv
   __syncwarp();
 }
 
+// (a call: the solves of a step share one copy of this code per factor type)
 template <typename T>
-__device__ void warp_lu_solve_any(const T* A, int N, const int* perm, const T* invdiag, const int* er, const int* ec,
+__device__ __noinline__ void warp_lu_solve_any(const T* A, int N, const int* perm, const T* invdiag, const int* er, const int* ec,
                                   const double* b, double* x) {
   if (N <= 32) warp_lu_solve_s<1, T>(A, N, perm, invdiag, er, ec, b, x);
   else if (N <= 64) warp_lu_solve_s<2, T>(A, N, perm, invdiag, er, ec, b, x);

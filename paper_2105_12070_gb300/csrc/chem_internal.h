@@ -13,7 +13,7 @@ enum : int { kElementary = 0, kThirdBody = 1, kLindemann = 2, kTroe = 3 };
 
 // Per-reaction integer record (16 ints).
 //   [0..3]  slot species: reactant 0, reactant 1, product 0, product 1 (-1 = empty)
-//   [4..7]  distinct slot species (the columns where dq/dC is non-zero without [M]), -1 pads
+//   [4..7]  distinct slot species, -1 pads
 //   [8..11] rows: distinct species k < K-1 with non-zero net coefficient, -1 pads
 //   [12..15] net coefficients of those rows
 constexpr int kRxInts = 16;
@@ -27,6 +27,17 @@ constexpr int kFoDoubles = 10;
 
 // Per species doubles: W, 1/W, Tmid, NASA low a1..a7, NASA high a1..a7
 constexpr int kSpDoubles = 17;
+
+// Rows of the per-species table of the fixed-point rate evaluation, [kSpfRows][K] (consecutive
+// threads read consecutive words): W, 1/W, Tmid, then kSpfRange rows for each range (low, high), all
+// with their constant factors multiplied in on the host:
+//   cp/R = sum a_n T^n:                           [0..4]  a1 .. a5
+//   h/RT = a1 + T (..) + a6/T:                    [5..8]  a2/2, a3/3, a4/4, a5/5   [9] a6
+//   (g/RT) / ln 2 = [10] + [11] log2 T + [12]/T + T ([13] + T ([14] + T ([15] + T [16]))), the first
+//     three as the bits of int64: * 2^52, * 2^57, * 2^45 (the largest terms are summed in fixed point)
+//   d(cp/R)/dT:                                   [17..19] 2 a3, 3 a4, 4 a5
+constexpr int kSpfRange = 20;
+constexpr int kSpfRows = 3 + 2 * kSpfRange;
 
 struct HostMech {
   int K = 0, R = 0, E = 0;
@@ -42,6 +53,19 @@ struct HostMech {
   std::vector<int> sr_ptr;             // [K + 1]
   std::vector<int> sr_idx;             // reaction index (device order)
   std::vector<double> sr_nu;           // net coefficient of the species in that reaction
+  // Tables of the fixed-point rate evaluation (build_fx_tables).  Logarithms base 2.
+  std::vector<double> fx_T;            // {lo, hi}: it takes temperatures inside (equal: none), chosen
+                                       // so that every exponent stays inside the fixed-point range
+  std::vector<uint32_t> rx4;           // [R] slot species, one byte each (255 = empty)
+  std::vector<int64_t> fxk;            // [3][R] log2 A * 2^52, b * 2^57, Ea/(Rc ln 2) * 2^46
+  std::vector<int64_t> fxo;            // [3][n_fo] the same of the low-pressure limit
+  std::vector<double> fod;             // [5][n_fo] 1 - alpha, alpha, log2(e)/T3, log2(e)/T1, T2 log2(e)
+  std::vector<double> spf;             // [kSpfRows][K]
+  std::vector<double> rxd_t;           // [2][R] b, Ea/Rc
+  std::vector<double> eff_t;           // [K][n_pd] efficiencies, transposed
+  // species production lists, entry e of species k at [e * K + k]: reaction index in the low half,
+  // the top 16 bits of the net coefficient as a double in the high half (small integers have no others)
+  std::vector<uint32_t> srx;
   // Jacobian gather plan (mass-action part).  Z entries (species row k < K-1, column j) that
   // receive contributions, each a list of (per-reaction scratch index src, coefficient):
   // Z[dst] = sum coef * s[src].  (src2 is kept for the layout and is always -1.)
@@ -63,6 +87,9 @@ struct HostMech {
   std::vector<int> cl_src;
   std::vector<int> cl_rx;
 };
+
+// (Re)build the tables of the fixed-point rate evaluation from the others (after a change of ln A too).
+void build_fx_tables(HostMech& m);
 
 // Parse the mechanism text file; false + message on error.
 bool parse_mechanism(const char* path, HostMech& m, std::string& err);
@@ -99,6 +126,16 @@ struct DevMech {
   const int* cl_ptr;
   const int* cl_src;
   const int* cl_rx;
+  // fixed-point rate evaluation (see HostMech)
+  const double* fx_T;  // (in device memory: a captured launch sees chem_set_lnA's change)
+  const uint32_t* rx4;
+  const int64_t* fxk;
+  const int64_t* fxo;
+  const double* fod;
+  const double* spf;
+  const double* rxd_t;
+  const double* eff_t;
+  const uint32_t* srx;
 };
 
 }  // namespace chemgpu

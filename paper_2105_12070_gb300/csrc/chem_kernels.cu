@@ -606,6 +606,15 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   const size_t o_clp = place(h.cl_ptr.size() * sizeof(int));
   const size_t o_cls = place(std::max<size_t>(1, h.cl_src.size()) * sizeof(int));
   const size_t o_clr = place(std::max<size_t>(1, h.cl_rx.size()) * sizeof(int));
+  const size_t o_fxT = place(h.fx_T.size() * sizeof(double));
+  const size_t o_rx4 = place(h.rx4.size() * sizeof(uint32_t));
+  const size_t o_fxk = place(h.fxk.size() * sizeof(int64_t));
+  const size_t o_fxo = place(h.fxo.size() * sizeof(int64_t));
+  const size_t o_fod = place(h.fod.size() * sizeof(double));
+  const size_t o_spf = place(h.spf.size() * sizeof(double));
+  const size_t o_rdt = place(h.rxd_t.size() * sizeof(double));
+  const size_t o_eft = place(h.eff_t.size() * sizeof(double));
+  const size_t o_srx = place(h.srx.size() * sizeof(uint32_t));
   const size_t total = off;
   std::vector<char> img(total, 0);
   auto put = [&](size_t o, const void* src, size_t bytes) { if (bytes) std::memcpy(img.data() + o, src, bytes); };
@@ -632,6 +641,15 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   put(o_clp, h.cl_ptr.data(), h.cl_ptr.size() * sizeof(int));
   put(o_cls, h.cl_src.data(), h.cl_src.size() * sizeof(int));
   put(o_clr, h.cl_rx.data(), h.cl_rx.size() * sizeof(int));
+  put(o_fxT, h.fx_T.data(), h.fx_T.size() * sizeof(double));
+  put(o_rx4, h.rx4.data(), h.rx4.size() * sizeof(uint32_t));
+  put(o_fxk, h.fxk.data(), h.fxk.size() * sizeof(int64_t));
+  put(o_fxo, h.fxo.data(), h.fxo.size() * sizeof(int64_t));
+  put(o_fod, h.fod.data(), h.fod.size() * sizeof(double));
+  put(o_spf, h.spf.data(), h.spf.size() * sizeof(double));
+  put(o_rdt, h.rxd_t.data(), h.rxd_t.size() * sizeof(double));
+  put(o_eft, h.eff_t.data(), h.eff_t.size() * sizeof(double));
+  put(o_srx, h.srx.data(), h.srx.size() * sizeof(uint32_t));
   e = cudaMalloc(&m->dbuf, total);
   if (e == cudaSuccess) e = cudaMemcpy(m->dbuf, img.data(), total, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_totals, 4 * sizeof(unsigned long long));
@@ -668,6 +686,15 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   d.cl_ptr = reinterpret_cast<const int*>(b + o_clp);
   d.cl_src = reinterpret_cast<const int*>(b + o_cls);
   d.cl_rx = reinterpret_cast<const int*>(b + o_clr);
+  d.fx_T = reinterpret_cast<const double*>(b + o_fxT);
+  d.rx4 = reinterpret_cast<const uint32_t*>(b + o_rx4);
+  d.fxk = reinterpret_cast<const int64_t*>(b + o_fxk);
+  d.fxo = reinterpret_cast<const int64_t*>(b + o_fxo);
+  d.fod = reinterpret_cast<const double*>(b + o_fod);
+  d.spf = reinterpret_cast<const double*>(b + o_spf);
+  d.rxd_t = reinterpret_cast<const double*>(b + o_rdt);
+  d.eff_t = reinterpret_cast<const double*>(b + o_eft);
+  d.srx = reinterpret_cast<const uint32_t*>(b + o_srx);
   d.n_pairs = (int)h.pr_pd.size();
   d.n_prows = (int)h.pr_rows.size();
   {
@@ -1053,10 +1080,13 @@ int chem_set_lnA(chem_mech* m, const double* lnA) {
   for (int r = 0; r < h.R; ++r)
     if (!std::isfinite(lnA[r])) return set_err(CHEM_EINVAL, "chem_set_lnA: non-finite value");
   for (int dr = 0; dr < h.R; ++dr) h.rxd[(size_t)dr * kRxDoubles] = lnA[h.order[dr]];
+  build_fx_tables(h);
   // the device tables are read by kernels in flight on any stream: wait for them first
   CK(cudaDeviceSynchronize());
   CK(cudaMemcpy(const_cast<double*>(m->dev.rxd), h.rxd.data(), h.rxd.size() * sizeof(double),
                 cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(const_cast<int64_t*>(m->dev.fxk), h.fxk.data(), h.fxk.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(const_cast<double*>(m->dev.fx_T), h.fx_T.data(), h.fx_T.size() * sizeof(double), cudaMemcpyHostToDevice));
   return CHEM_OK;
 }
 

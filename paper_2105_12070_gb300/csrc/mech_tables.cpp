@@ -20,6 +20,145 @@
 
 namespace chemgpu {
 
+// Fixed-point value v * 2^bits, rounded; 0 and ok = false if it does not fit in 63 bits.
+static int64_t to_fixed(long double v, int bits, bool& ok) {
+  const long double x = std::ldexp(v, bits);
+  if (!(std::fabs(x) < 9.2e18L)) {
+    ok = false;
+    return 0;
+  }
+  return (int64_t)std::llround(x);
+}
+
+void build_fx_tables(HostMech& m) {
+  const int K = m.K, R = m.R, nf = m.n_fo, npd = m.n_tb + m.n_fo;
+  const long double log2e = 1.0L / std::log(2.0L);
+  bool ok = K < 255 && R < 65536;
+  m.rx4.assign(R, 0xffffffffu);
+  m.fxk.assign((size_t)3 * R, 0);
+  m.rxd_t.assign((size_t)2 * R, 0.0);
+  m.fxo.assign((size_t)3 * std::max(nf, 1), 0);
+  m.fod.assign((size_t)5 * std::max(nf, 1), 0.0);
+  for (int r = 0; r < R; ++r) {
+    const int* ii = &m.rxi[(size_t)r * kRxInts];
+    uint32_t v = 0;
+    for (int u = 0; u < 4; ++u) v |= (uint32_t)(ii[u] < 0 ? 255 : ii[u] & 255) << (8 * u);
+    m.rx4[r] = v;
+    const double* d = &m.rxd[(size_t)r * kRxDoubles];
+    m.fxk[r] = to_fixed(d[0] * log2e, 52, ok);
+    m.rxd_t[r] = d[1];
+    m.rxd_t[R + r] = d[2];
+    m.fxk[R + r] = to_fixed(d[1], 57, ok);
+    m.fxk[2 * R + r] = to_fixed(d[2] * log2e, 46, ok);
+    if (r < nf) {
+      const double* q = &m.fo[(size_t)r * kFoDoubles];
+      m.fxo[r] = to_fixed(q[0] * log2e, 52, ok);
+      m.fxo[nf + r] = to_fixed(q[1], 57, ok);
+      m.fxo[2 * nf + r] = to_fixed(q[2] * log2e, 46, ok);
+      m.fod[r] = 1.0 - q[3];
+      m.fod[nf + r] = q[3];
+      m.fod[2 * nf + r] = (double)(q[8] * log2e);
+      m.fod[3 * nf + r] = (double)(q[9] * log2e);
+      m.fod[4 * nf + r] = (double)(q[6] * log2e);
+    }
+  }
+  m.spf.assign((size_t)kSpfRows * K, 0.0);
+  for (int k = 0; k < K; ++k) {
+    const double* sp = &m.sp[(size_t)k * kSpDoubles];
+    for (int i = 0; i < 3; ++i) m.spf[(size_t)i * K + k] = sp[i];
+    for (int range = 0; range < 2; ++range) {
+      const double* a = sp + 3 + 7 * range;
+      const long double v[kSpfRange] = {a[0], a[1], a[2], a[3], a[4],
+                                        a[1] / 2.0L, a[2] / 3.0L, a[3] / 4.0L, a[4] / 5.0L, a[5],
+                                        ((long double)a[0] - a[6]) * log2e, -(long double)a[0], a[5] * log2e,
+                                        -a[1] / 2.0L * log2e, -a[2] / 6.0L * log2e, -a[3] / 12.0L * log2e,
+                                        -a[4] / 20.0L * log2e, 2.0L * a[2], 3.0L * a[3], 4.0L * a[4]};
+      for (int i = 0; i < kSpfRange; ++i) {
+        const int bits = i == 10 ? 52 : i == 11 ? 57 : i == 12 ? 45 : 0;
+        double& o = m.spf[(size_t)(3 + kSpfRange * range + i) * K + k];
+        o = (double)v[i];
+        if (bits) {
+          const int64_t x = to_fixed(v[i], bits, ok);
+          std::memcpy(&o, &x, 8);
+        }
+      }
+    }
+  }
+  m.eff_t.assign((size_t)std::max(npd, 1) * K, 0.0);
+  for (int r = 0; r < npd; ++r)
+    for (int k = 0; k < K; ++k) m.eff_t[(size_t)k * npd + r] = m.eff[(size_t)r * K + k];
+  int longest = 0;
+  for (int k = 0; k < K; ++k) longest = std::max(longest, m.sr_ptr[k + 1] - m.sr_ptr[k]);
+  m.srx.assign((size_t)std::max(longest, 1) * K, 0);
+  for (int k = 0; k < K; ++k)
+    for (int e = m.sr_ptr[k]; e < m.sr_ptr[k + 1]; ++e) {
+      uint64_t b;
+      std::memcpy(&b, &m.sr_nu[e], 8);
+      m.srx[(size_t)(e - m.sr_ptr[k]) * K + k] = (uint32_t)(m.sr_idx[e] & 0xffff) | (uint32_t)(b >> 48) << 16;
+    }
+  // The temperature interval in which no exponent can leave its range.  Within an interval where
+  // every species stays in one of its two ranges, each term's magnitude is largest at an end, so
+  // bounds taken there hold inside: |log2 k| < 1000 for each rate constant and < 900 for the
+  // equilibrium exponent of a reaction (the sums of two rate exponents and of one with the
+  // equilibrium exponent stay below 2048), and |g/RT|/ln 2 < 1000 for each species (the range of the
+  // conversion).  lo > 128 keeps 1/T * 2^70 inside 63 bits, hi <= 8192 keeps log2 T below 13.
+  m.fx_T = {0.0, 0.0};
+  const double candidates[][2] = {{160.0, 8192.0}, {256.0, 8192.0}, {512.0, 8192.0}, {160.0, 4096.0}, {256.0, 4096.0},
+                                  {512.0, 4096.0}, {1024.0, 4096.0}};
+  for (const auto& cand : candidates) {
+    const double lo = cand[0], hi = cand[1];
+    bool fits = ok;
+    auto rate_fits = [&](double lnA, double b, double E) {
+      return (std::fabs(lnA) + std::fabs(E) / lo) * 1.4427 + std::fabs(b) * 13.0 < 1000.0;
+    };
+    // bound over [lo, hi] of |sum_k c_k (g_k/RT)| / ln 2
+    auto g_bound = [&](const std::vector<std::pair<int, double>>& terms) {
+      std::vector<double> ends = {lo, hi};
+      for (const auto& t : terms) {
+        const double mid = m.spf[(size_t)2 * K + t.first];
+        if (mid > lo && mid < hi) ends.push_back(mid);
+      }
+      std::sort(ends.begin(), ends.end());
+      double worst = 0.0;
+      for (size_t e = 0; e + 1 < ends.size(); ++e) {
+        const double t0 = ends[e], t1 = ends[e + 1], mid = 0.5 * (t0 + t1);
+        double c[7] = {0, 0, 0, 0, 0, 0, 0};
+        for (const auto& t : terms) {
+          const int first = 3 + (mid <= m.spf[(size_t)2 * K + t.first] ? 0 : kSpfRange) + 10;
+          for (int i = 0; i < 7; ++i) {
+            const double o = m.spf[(size_t)(first + i) * K + t.first];
+            int64_t x;
+            std::memcpy(&x, &o, 8);
+            c[i] += t.second * (i > 2 ? o : std::ldexp((double)x, i == 0 ? -52 : i == 1 ? -57 : -45));
+          }
+        }
+        const double v = std::fabs(c[0]) + 13.0 * std::fabs(c[1]) + std::fabs(c[2]) / t0 +
+                         t1 * (std::fabs(c[3]) + t1 * (std::fabs(c[4]) + t1 * (std::fabs(c[5]) + t1 * std::fabs(c[6]))));
+        worst = std::max(worst, v);
+      }
+      return worst;
+    };
+    for (int k = 0; k < K && fits; ++k) fits = g_bound({{k, 1.0}}) < 1000.0;
+    for (int r = 0; r < R && fits; ++r) {
+      const double* d = &m.rxd[(size_t)r * kRxDoubles];
+      fits = rate_fits(d[0], d[1], d[2]);
+      if (fits && r < nf) {
+        const double* q = &m.fo[(size_t)r * kFoDoubles];
+        fits = rate_fits(q[0], q[1], q[2]);
+      }
+      const int* ii = &m.rxi[(size_t)r * kRxInts];
+      std::vector<std::pair<int, double>> terms;
+      for (int u = 0; u < 4; ++u)
+        if (ii[u] >= 0) terms.push_back({ii[u], u < 2 ? -1.0 : 1.0});
+      fits = fits && g_bound(terms) < 900.0;
+    }
+    if (fits) {
+      m.fx_T = {lo, hi};
+      break;
+    }
+  }
+}
+
 namespace {
 
 constexpr double kRcal = 8.314462618 / 4.184;  // cal/(mol K)
@@ -78,10 +217,12 @@ void build_jacobian_plan(HostMech& m) {
   const int K = m.K, d = K - 1;
   struct Contrib { int dst, src, src2; double coef; };
   std::vector<Contrib> cs;
+  // (the columns are the four slots themselves: a species in two slots of a reaction receives the
+  // derivatives through both)
   for (int r = 0; r < m.R; ++r) {
     const int* ii = &m.rxi[(size_t)r * kRxInts];
     for (int u = 0; u < 4; ++u) {
-      const int col = ii[4 + u];
+      const int col = ii[u];
       if (col < 0) continue;
       for (int rs = 0; rs < 4; ++rs) {
         const int row = ii[8 + rs];
@@ -137,7 +278,7 @@ void build_jacobian_plan(HostMech& m) {
     return (m.pr_ptr[a + 1] - m.pr_ptr[a]) < (m.pr_ptr[b + 1] - m.pr_ptr[b]);
   });
   // column lists for products with J^T: for each species column j, the scratch entries
-  // dq/dC_j (u * R + r) of the reactions that have j among their distinct slot species
+  // dq/dC_j (u * R + r) of the slots u that hold j
   m.cl_ptr.assign(K + 1, 0);
   m.cl_src.clear(); m.cl_rx.clear();
   for (int j = 0; j < K; ++j) {
@@ -145,7 +286,7 @@ void build_jacobian_plan(HostMech& m) {
     for (int r = 0; r < m.R; ++r) {
       const int* ii = &m.rxi[(size_t)r * kRxInts];
       for (int u = 0; u < 4; ++u)
-        if (ii[4 + u] == j) { m.cl_src.push_back(u * m.R + r); m.cl_rx.push_back(r); }
+        if (ii[u] == j) { m.cl_src.push_back(u * m.R + r); m.cl_rx.push_back(r); }
     }
   }
   m.cl_ptr[K] = (int)m.cl_src.size();
@@ -321,6 +462,7 @@ bool build_tables(const char* path, HostMech& m, std::vector<FileReaction>& rx, 
   }
   m.sr_ptr[K] = (int)m.sr_idx.size();
   build_jacobian_plan(m);
+  build_fx_tables(m);
   return true;
 }
 

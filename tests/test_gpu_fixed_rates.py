@@ -1,0 +1,122 @@
+"""The fixed-point rate evaluation at the edges of its range, against the oracle: temperatures on both
+sides of the interval it takes and of Tmid, states with zero, tiny and slightly negative mass
+fractions, a species on both sides of a reaction, mechanisms it must leave to the general form, and a change of ln A that moves the
+interval under a captured launch.  Tolerances as in test_gpu_parity.py (1e-11 of the gross flux,
+1e-12 of the row)."""
+import copy
+import os
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O
+from paper_2105_12070_gb300 import chem, synth
+
+pytestmark = pytest.mark.gpu
+
+P = 5.0 * synth.P_ATM_PA
+EDGES = [100.0, 159.0, 160.0, 161.0, 256.0, 256.5, 512.0, 999.9, 1000.0, 1000.1, 2999.0, 4095.0, 4097.0, 6000.0,
+         8191.0, 8193.0]
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _states(K, n_per_T=3, seed=5):
+    rng = np.random.default_rng(seed)
+    T = np.repeat(EDGES, n_per_T)
+    Y = rng.dirichlet(np.ones(K), size=T.size)
+    Y[::3, : K // 2] = 0.0          # absent species
+    Y[1::3, 0] = 1e-30              # a trace
+    Y[2::3, 1] = -1e-12             # what a transport scheme may hand over
+    return T, np.ascontiguousarray(Y.T)
+
+
+def _check(mech, ora, T, Y, p=P):
+    f = torch.empty((mech.N, T.size), dtype=torch.float64, device="cuda")
+    J = torch.empty((T.size, mech.N, mech.N), dtype=torch.float64, device="cuda")
+    chem.chem_rates(mech, p, _dev(T), _dev(Y), f)
+    chem.chem_jacobian(mech, p, _dev(T), _dev(Y), J)
+    torch.cuda.synchronize()
+    f, J = f.cpu().numpy(), J.cpu().numpy()
+    fo, gross = ora.rates(p, T, Y, gross=True)
+    Jo = ora.jacobian(p, T, Y)
+    ok = np.isfinite(fo).all(axis=0) & np.isfinite(gross).all(axis=0) & np.isfinite(Jo).all(axis=(1, 2))
+    assert ok.sum() >= T.size // 2
+    assert np.all(np.abs(f - fo)[:, ok] <= 1e-11 * gross[:, ok] + 1e-300)
+    rel = np.abs(J - Jo)[ok] / np.maximum(np.abs(Jo[ok]).max(axis=2, keepdims=True), 1e-300)
+    assert rel.max() <= 1e-12, (rel.max(), T[ok][np.unravel_index(np.argmax(rel), rel.shape)[0]])
+
+
+@pytest.mark.parametrize("make", [synth.mechanism_small, synth.mechanism_53, synth.mechanism_100])
+def test_edges_of_the_range(make):
+    path = make().write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    T, Y = _states(mech.K)
+    _check(mech, ora, T, Y)
+
+
+def test_species_on_both_sides(tmp_path):
+    """A + B = 2 B (isomers): one species in three slots of a reaction."""
+    text = open(os.path.join(os.path.dirname(__file__), "golden", "isomer_AB.txt")).read()
+    text = text.replace("0 1 0 -1 1 1 -1 3000.0 0.5 10000.0", "0 2 0 1 2 1 1 3e12 0.5 10000.0")
+    text = text.replace("-1000.0 11.386294361119891", "-1500.0 11.386294361119891")  # a heat of reaction
+    assert "0 2 0 1 2 1 1" in text and text.count("-1500.0 11.38") == 2
+    path = tmp_path / "autocatalytic.txt"
+    path.write_text(text)
+    mech, ora = chem.Mechanism(str(path)), O.OracleMechanism(str(path))
+    _check(mech, ora, *_states(mech.K))
+
+
+@pytest.mark.parametrize("change", ["barrier", "exponent", "prefactor"])
+def test_mechanisms_outside_the_limits(change):
+    m = copy.deepcopy(synth.mechanism_small())
+    if change == "barrier":
+        m.Ea[3] = 400e3     # beyond the table's 2^17 K ln 2
+    elif change == "exponent":
+        m.b[5] = 70.0
+        m.A[5] = 1e-180
+    else:
+        m.A[7] = 1e290
+    path = m.write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    T, Y = _states(mech.K)
+    keep = (T > 200.0) & (T < 5000.0)
+    T, Y = T[keep], np.ascontiguousarray(Y[:, keep])
+    # one reaction may dwarf the others here: the source term against its gross flux stays meaningful
+    f = torch.empty((mech.N, T.size), dtype=torch.float64, device="cuda")
+    chem.chem_rates(mech, P, _dev(T), _dev(Y), f)
+    torch.cuda.synchronize()
+    fo, gross = ora.rates(P, T, Y, gross=True)
+    ok = np.isfinite(fo).all(axis=0) & np.isfinite(gross).all(axis=0)
+    assert np.all(np.abs(f.cpu().numpy() - fo)[:, ok] <= 1e-11 * gross[:, ok] + 1e-300)
+
+
+def test_ln_a_change_moves_the_interval_of_a_captured_launch():
+    w = synth.workload_small()
+    path = w["mech"].write_temp()
+    mech = chem.Mechanism(path)
+    lnA = chem.chem_get_lnA(mech)
+    opts = chem.default_opts(use_graph=1)
+    T0, Y0 = _dev(w["T"][:40]), _dev(w["Y"][:, :40])
+    T, Y = torch.empty_like(T0), torch.empty_like(Y0)
+
+    def step(o):
+        T.copy_(T0)
+        Y.copy_(Y0)
+        chem.chem_integrate(mech, w["p_Pa"], T, Y, 1e-7, opts=o)
+        torch.cuda.synchronize()
+        return T.clone(), Y.clone()
+
+    first = step(opts)
+    far = lnA.copy()
+    far[4] = -1500.0        # a reaction switched off by its pre-factor: outside the fixed-point range
+    chem.chem_set_lnA(mech, far)
+    replayed, direct = step(opts), step(chem.default_opts())
+    assert torch.equal(replayed[0], direct[0]) and torch.equal(replayed[1], direct[1])
+    chem.chem_set_lnA(mech, lnA)
+    again = step(opts)
+    assert torch.equal(first[0], again[0]) and torch.equal(first[1], again[1])
