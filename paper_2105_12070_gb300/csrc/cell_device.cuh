@@ -145,11 +145,10 @@ struct Grp {
     if (G == 1) {
       __syncwarp();
     } else {
-      // bar.sync is an aligned barrier: every lane of the warp has to execute it together.  After a
-      // divergent branch the compiler does not have to join the lanes before inline PTX, and a warp that
-      // arrives in two parts counts twice.
-      __syncwarp();
-      asm volatile("bar.sync %0, %1;" ::"r"(gid + 1), "r"(NT) : "memory");
+      // the unaligned form: the lanes of a warp may arrive apart.  bar.sync, the aligned one, counts a warp that
+      // arrives in two parts twice and lets the others through early, and after a divergent branch the
+      // compiler does not have to join the lanes before inline PTX.
+      __barrier_sync_count(gid + 1, NT);
     }
   }
   __device__ double sum(double v) const {

@@ -78,3 +78,24 @@ def test_uneven_field_mech100_parity_and_order_independence():
     Tall, Yall, st2 = _run(mech, w, chem.default_opts(), T=w["T"][perm], Y=w["Y"][:, perm])
     inv = np.argsort(perm)
     np.testing.assert_array_equal(Tall[inv][idx], Tg)
+
+
+@pytest.mark.parametrize("solver,dt,max_steps", [(chem.CHEM_SOLVER_ROSENBROCK, 1e-10, 3000),
+                                                 (chem.CHEM_SOLVER_SEULEX, 1e-6, 600)])
+def test_cells_beside_each_other_do_not_matter(solver, dt, max_steps):
+    """The warps of a cell meet only at their group's barrier: with one to five cells on an SM, whose
+    timing differs, every cell has the same bits."""
+    w = synth.workload_shear_layer(32)
+    mech = chem.Mechanism(w["mech"].write_temp())
+    idx = np.arange(0, 1024, 5)
+    ref = None
+    for cpc in (1, 2, 3, 4, 5):
+        T = torch.from_numpy(w["T"][idx].copy()).cuda()
+        Y = torch.from_numpy(np.ascontiguousarray(w["Y"][:, idx])).cuda()
+        opts = chem.default_opts(solver=solver, max_steps=max_steps, cells_per_cta=cpc, warps_per_cell=2)
+        st = chem.chem_integrate(mech, w["p_Pa"], T, Y, dt, w["rtol"], w["atol"], opts=opts, want_stats=True)
+        got = (st.steps, st.rejects, T, Y)
+        assert st.failed_cells == 0
+        if ref is None:
+            ref = got
+        assert got[:2] == ref[:2] and torch.equal(T, ref[2]) and torch.equal(Y, ref[3]), cpc
