@@ -240,17 +240,17 @@ struct Grp {
     parity++;
     if (lane() == 0) {
       r[3 * warp()] = __longlong_as_double(key);
-      r[3 * warp() + 1] = __int2double_rn(idx);
+      r[3 * warp() + 1] = __longlong_as_double(idx);  // as bits: a conversion is an FP64 instruction
       r[3 * warp() + 2] = val;
     }
     sync();
     key = __double_as_longlong(r[0]);
-    idx = (int)r[1];
+    idx = (int)__double_as_longlong(r[1]);
     val = r[2];
 #pragma unroll
     for (int i = 1; i < G; ++i) {
       const long long ok = __double_as_longlong(r[3 * i]);
-      const int oi = (int)r[3 * i + 1];
+      const int oi = (int)__double_as_longlong(r[3 * i + 1]);
       if (ok > key || (ok == key && oi < idx)) { key = ok; idx = oi; val = r[3 * i + 2]; }
     }
   }
@@ -357,42 +357,11 @@ struct CellScalarsT {
 };
 using CellScalars = CellScalarsT<double>;
 
-// 1/a by Newton's iteration for the reciprocal, r <- r + r (1 - m r), on the significand m of a
-// (normalised to +-[1, 2) by replacing the exponent field): the seed is the FP32 approximate
-// reciprocal (rcp.approx) of m's leading 24 bits, relative error below 2^-21; two steps in FP64
-// square the error twice (below 2^-84, under the final rounding), so the result is within one
-// unit in the last place of 1/a.  The exponent is then restored by an integer subtraction.  Four
-// FP64 operations instead of a full division; zero, subnormal, very large, infinite and NaN
-// arguments take the division.
-__device__ inline double rcp_newton(double a) {
-  const long long b = __double_as_longlong(a);
-  const int ef = (int)((b >> 52) & 0x7ff);
-  if (ef < 3 || ef > 2044) return 1.0 / a;
-  const long long mb = (b & (long long)0x800fffffffffffffULL) | (1023LL << 52);
-  const double m = __longlong_as_double(mb);
-  const unsigned hi = (unsigned)((unsigned long long)b >> 32);
-  // m as a float: sign, exponent 127, the top 23 significand bits (truncated)
-  const float mf = __uint_as_float((hi & 0x80000000u) | 0x3f800000u | (unsigned)((b >> 29) & 0x7fffff));
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(mf));
-  // rf in +-[0.5, 1]: the same value as a double, by moving its fields
-  const unsigned fb = __float_as_uint(rf);
-  const long long rb = ((long long)(fb >> 31) << 63) | ((long long)(((fb >> 23) & 0xff) - 127 + 1023) << 52) |
-                       ((long long)(fb & 0x7fffff) << 29);
-  double r = __longlong_as_double(rb);
-  double e = fma(-m, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-m, r, 1.0);
-  r = fma(r, e, r);
-  // 1/a = r 2^-(ef - 1023); r's exponent field is 1022 or 1023, the result's stays in [1, 2043]
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)(ef - 1023) << 52));
-}
-
-// 1/x for the scalar types of the rate code (the fall-off quotients): Newton's reciprocal, and for
-// a dual number (1/v, -d/v^2) from it.
-__device__ inline double recip(double x) { return rcp_newton(x); }
+// 1/x for the scalar types of the rate code (the fall-off quotients), and for a dual number
+// (1/v, -d/v^2) from it.
+__device__ inline double recip(double x) { return fx_rcp(x); }
 __device__ inline Dual recip(Dual x) {
-  const double r = rcp_newton(x.v);
+  const double r = fx_rcp(x.v);
   return Dual(r, -x.d * r * r);
 }
 
@@ -523,9 +492,9 @@ __device__ inline void troe_fx(const double* fd, int n, double T, double invT, d
   const double nn = fma(-1.27, L, 0.75);
   const double xc = log10_fx(Pr) + fma(-0.67, L, -0.4);
   const double den = fma(-0.14, xc, nn);
-  const double iden = rcp_newton(den);
+  const double iden = fx_rcp(den);
   const double f1 = xc * iden;
-  const double ig = rcp_newton(fma(f1, f1, 1.0));
+  const double ig = fx_rcp(fma(f1, f1, 1.0));
   const double Lg = L * ig;
   F = fx_exp2_of(Lg * 3.3219280948873623479);
   if (jac) {
@@ -534,7 +503,7 @@ __device__ inline void troe_fx(const double* fd, int n, double T, double invT, d
     dlF = -2.0 * t * (nn * iden2);
     // d Fcent / dT; the table's exponents carry log2(e): times ln 2
     const double dFc = 0.69314718055994530942 * (T2 * (invT * invT) * e2 - (oma * iT3 * e3 + a * iT1 * e1));
-    const double dL = dFc * rcp_newton(Fcent);  // ln(10) dL/dT
+    const double dL = dFc * fx_rcp(Fcent);  // ln(10) dL/dT
     const double df1_dL = fma(-0.67, den, xc * (1.27 - 0.14 * 0.67)) * iden2;
     dlnF_dT = fma(-2.0 * t, df1_dL, ig) * dL;
   }
@@ -811,7 +780,7 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
   if (jac) g.sum2(cp, dcp);
   else cp = g.sum(cp);
   s.cp = cp * kRu;
-  s.inv_cp = rcp_newton(s.cp);
+  s.inv_cp = fx_rcp(s.cp);
   s.dcp_dT = dcp * kRu;
   if (G == 1) g.sync();  // (with several warps the reduction's barrier has published C and the thermo)
   for (int r = g.t; r < npd; r += NT) {
@@ -858,7 +827,7 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
       const double ratio = fx_exp2(X0 - Xf);  // k0 / k_inf
       Pr = ratio * Mr;
       if (m.fo[(size_t)r * kFoDoubles + 7] != 0.0) troe_fx(m.fod + r, nfo, s.T, s.invT, Pr, F, dlF, dlnF_dT, jac);
-      inv1p = rcp_newton(1.0 + Pr);
+      inv1p = fx_rcp(1.0 + Pr);
       const double kF = kf * (F * inv1p);
       if (jac) dk_dM = ratio * kF * (inv1p + dlF);
       kf = kF * Pr;
@@ -1381,11 +1350,7 @@ __device__ inline S lu_recip(double c);
 
 template <>
 __device__ inline double lu_recip<double>(double c) {
-#ifdef CHEM_LU_RCP_DIVISION
-  return 1.0 / c;
-#else
-  return rcp_newton(c);
-#endif
+  return fx_rcp(c);
 }
 template <>
 __device__ inline float lu_recip<float>(double c) { return 1.0f / f32_of(c); }
@@ -1539,7 +1504,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
     }
     if (g.lane() == 0) {
       cand[3 * g.warp()] = __longlong_as_double(best);
-      cand[3 * g.warp() + 1] = __int2double_rn(bi);
+      cand[3 * g.warp() + 1] = __longlong_as_double(bi);
       cand[3 * g.warp() + 2] = bv;
     }
   }
@@ -1547,12 +1512,12 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
   for (int k = 0; k < N; ++k) {
     const double* cr = cand + (k & 1) * 3 * G;
     long long best = __double_as_longlong(cr[0]);
-    int bi = (int)cr[1];
+    int bi = (int)__double_as_longlong(cr[1]);
     double bv = cr[2];
 #pragma unroll
     for (int w = 1; w < G; ++w) {
       const long long ob = __double_as_longlong(cr[3 * w]);
-      const int oi = (int)cr[3 * w + 1];
+      const int oi = (int)__double_as_longlong(cr[3 * w + 1]);
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; bv = cr[3 * w + 2]; }
     }
     if (best <= 0) ok = false;  // zero column: singular
@@ -1609,27 +1574,32 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
       const int mc = mm - 1;  // columns k+2 .. N-1
       const int tot = mm * mc;
       if (tot > 0) {
-        const float inv_m = 1.0f / (float)mc;
+        // entry e = i mc + j of the trailing block; the thread's entries are NT apart, so the row and
+        // column advance by (NT / mc, NT mod mc) with at most one wrap
+        const int di = (int)(((float)NT + 0.5f) / (float)mc), dj = NT - di * mc;
+        int i = (int)(((float)g.t + 0.5f) / (float)mc), j = g.t - i * mc + 1;
         int e = g.t;
         for (; e + 3 * NT < tot; e += 4 * NT) {
-          int ii[4], jj[4];
+          int at[4];
           S l[4], u[4], a[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const int x = e + q * NT;
-            ii[q] = (int)(((float)x + 0.5f) * inv_m);
-            jj[q] = x - ii[q] * mc + 1;
-            l[q] = Ak[ii[q] * N];
-            u[q] = U[jj[q]];
-            a[q] = T0[ii[q] * N + jj[q]];
+            at[q] = i * N + j;
+            l[q] = Ak[i * N];
+            u[q] = U[j];
+            a[q] = T0[at[q]];
+            i += di;
+            j += dj;
+            if (j > mc) { j -= mc; ++i; }
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) T0[ii[q] * N + jj[q]] = fma(-l[q], u[q], a[q]);
+          for (int q = 0; q < 4; ++q) T0[at[q]] = fma(-l[q], u[q], a[q]);
         }
         for (; e < tot; e += NT) {
-          const int i = (int)(((float)e + 0.5f) * inv_m);
-          const int j = e - i * mc + 1;
           T0[i * N + j] = fma(-Ak[i * N], U[j], T0[i * N + j]);
+          i += di;
+          j += dj;
+          if (j > mc) { j -= mc; ++i; }
         }
       }
     }
@@ -1644,7 +1614,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
       if (g.lane() == 0) {
         double* cw = cand + ((k + 1) & 1) * 3 * G;
         cw[3 * g.warp()] = __longlong_as_double(nb);
-        cw[3 * g.warp() + 1] = __int2double_rn(ni);
+        cw[3 * g.warp() + 1] = __longlong_as_double(ni);
         cw[3 * g.warp() + 2] = nv;
       }
     }

@@ -57,6 +57,13 @@ __device__ void cell_fd_jacobian(const DevMech& m, const Grp<G>& g, double p, co
   }
 }
 
+// x^(-q), 0 < q <= 1, of an error norm: exp2(-q log2 x) in fixed point (every thread by itself, no
+// FP64 transcendental); zero, subnormal, infinite and NaN arguments take pow.
+__device__ __noinline__ double inv_root_wide(double x, double q) { return pow(x, -q); }
+__device__ inline double inv_root(double x, double q) {
+  return fx_log2_takes(x) ? fx_exp2_of(-q * fx_value(fx_log2(x))) : inv_root_wide(x, q);
+}
+
 // ------------------------------------------------------------------------------------------
 // Mixed precision (FP32 LU + FP64-residual iterative refinement).
 
@@ -270,8 +277,8 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
       // iteration matrix W = I/(gamma h) - J and its factors.  Mixed precision first tries the
       // FP32 factors of the equilibrated matrix with FP64-residual refinement; if a stage solve
       // does not converge the attempt is redone with FP64 factors.
-      const double gh = 1.0 / (gam * h);
-      const double invh = 1.0 / h;
+      const double gh = fx_rcp(gam * h);
+      const double invh = fx_rcp(h);
       double err = INFINITY;
       // after a fallback the next attempts go straight to FP64 factors for a while
       for (int pass = (a.mixed && attempt >= f64_until) ? 0 : 1; pass < 2; ++pass) {
@@ -280,7 +287,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
         if (lowp) {
           // reciprocal error-control scales of the refinement's stopping test (the error vector is
           // free until the stages are combined)
-          for (int i = g.t; i < N; i += NT) w.err[i] = 1.0 / (a.atol + a.rtol * fabs(w.y[i]));
+          for (int i = g.t; i < N; i += NT) w.err[i] = fx_rcp(a.atol + a.rtol * fabs(w.y[i]));
         }
         if (lowp == 1) {
           ok = form_and_factor_low<G, float>(g, w, N, gh, w.invd32);
@@ -357,20 +364,12 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
         double e = 0.0;
         for (int i = g.t; i < N; i += NT) {
           const double sc = a.atol + a.rtol * fmax(fabs(w.y[i]), fabs(w.ynew[i]));
-          e = Grp<G>::nanmax(e, fabs(w.err[i] * gh) / sc);
+          e = Grp<G>::nanmax(e, fabs(w.err[i] * gh) * fx_rcp(sc));
         }
         err = g.max_nan(e);
         break;
       }
-      // err^(-1/4) of the step-size factor, by one thread for the group (see cell_rates)
-      double p25;
-      if (G > 1) {
-        if (g.t == 0) w.bc[5] = pow(err, -0.25);
-        g.sync();
-        p25 = w.bc[5];
-      } else {
-        p25 = pow(err, -0.25);
-      }
+      const double p25 = inv_root(err, 0.25);  // err^(-1/4) of the step-size factor
       double fac;
       if (err <= 1.0) {
         if (a.rec) {
@@ -435,6 +434,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
 // give-up keeps J and shrinks H by min(fac, 1/2); a singular matrix or a non-finite error by 1/5.
 // The tableau row lives in eight of the cell's vectors and is updated element by element.
 constexpr int kSeulexKmax = 8;
+__constant__ double c_inv_int[9] = {0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8};
 
 __device__ inline double seulex_work(int j) {
   // A_1 = 2.5 + 2 + (0.2 + 1); A_j = A_{j-1} + 2 + 0.2 j + (j - 1)
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(Dev
       bool badstep = false;
       for (int j = 1; j <= k + 1; ++j) {
         last = j;
-        const double gh = (double)j / H;  // 1/h
+        const double gh = (double)j * fx_rcp(H);  // 1/h
         for (int e = g.t; e < N * N; e += NT) w.B[e] = w.A[e];
         g.sync();
         for (int i = g.t; i < N; i += NT) w.B[i * N + i] += gh;
@@ -522,16 +522,16 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(Dev
         for (int i = g.t; i < N; i += NT) {
           double q = yi[i];
           for (int l = 2; l <= j; ++l) {
-            const double r = (double)j / (double)(j - l + 1);
+            // 1 / (n_j / n_{j-l+1} - 1) = (j - l + 1) / (l - 1)
             double* tl = tab(l - 1);
-            const double qn = q + (q - tl[i]) / (r - 1.0);
+            const double qn = fma(q - tl[i], (double)(j - l + 1) * c_inv_int[l - 1], q);
             tl[i] = q;
             q = qn;
           }
           tab(j)[i] = q;
           if (j >= 2) {
             const double sc = a.atol + a.rtol * fmax(fabs(w.y[i]), fabs(q));
-            e = Grp<G>::nanmax(e, fabs(q - tab(j - 1)[i]) / sc);
+            e = Grp<G>::nanmax(e, fabs(q - tab(j - 1)[i]) * fx_rcp(sc));
           }
         }
         g.sync();
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(Dev
         e = g.max_nan(e);
         if (!(e < INFINITY)) { badstep = true; break; }  // NaN or infinite
         fac_prv = fac_cur;
-        fac_cur = (e > 0.0) ? fmin(4.0, fmax(0.02, 0.94 * pow(e, -1.0 / j))) : 4.0;
+        fac_cur = (e > 0.0) ? fmin(4.0, fmax(0.02, 0.94 * inv_root(e, c_inv_int[j]))) : 4.0;
         if (j == k - 1) {
           if (e <= 1.0) { accepted = j; break; }
         } else if (j == k) {
