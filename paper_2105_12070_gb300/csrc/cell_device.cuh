@@ -275,7 +275,7 @@ __host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G) {
   p.off_B = p.SA;
   p.off_vec = 2 * p.SA;
   // vectors: y, ynew, f0, fs, u0..u3, err, invdiag, rhs, res, (er, ec as ints), (FP32 inverse
-  // pivots)  (14 x N); the Jacobian's temporaries zc, dwT, rowA, rowB, ccol reuse u0..u3, err
+  // pivots)  (14 x N); the Jacobian's temporaries zc, dwT, rowA, rowB, ccol reuse ynew, fs, u2, u3, err
   p.off_sp = p.off_vec + 14 * round2(K);
   // species: C, hRT, cpR, gRT, omega, dcpR  (6 x K)
   p.off_q = p.off_sp + 6 * round2(K);
@@ -308,7 +308,7 @@ __device__ inline CellMem carve(double* base, const Plan& p) {
   w.y = v; w.ynew = v + n; w.f0 = v + 2 * n; w.fs = v + 3 * n;
   for (int i = 0; i < 4; ++i) w.u[i] = v + (4 + i) * n;
   w.err = v + 8 * n; w.invdiag = v + 9 * n;
-  w.zc = w.u[0]; w.dwT = w.u[1]; w.rowA = w.u[2]; w.rowB = w.u[3]; w.ccol = w.err;
+  w.zc = w.ynew; w.dwT = w.fs; w.rowA = w.u[2]; w.rowB = w.u[3]; w.ccol = w.err;
   w.rhs = v + 10 * n; w.res = v + 11 * n;
   w.er = reinterpret_cast<int*>(v + 12 * n);
   w.ec = w.er + n;
@@ -337,7 +337,8 @@ struct EvalMem {
 };
 
 // The solve's evaluation arrays: the Jacobian temporaries reuse the stage vectors, which are
-// free while the Jacobian is built (pv spans u0 .. res, n_pairs <= 8 round2(K)).
+// free while the Jacobian is built (pv spans u0 .. res, n_pairs <= 8 round2(K); zc and dwT, which the
+// rate evaluation writes before pv is used, lie outside it).
 __device__ inline EvalMem<double> eval_mem(const CellMem& w) {
   EvalMem<double> e;
   e.C = w.C; e.hRT = w.hRT; e.cpR = w.cpR; e.gRT = w.gRT; e.omega = w.omega; e.dcpR = w.dcpR;
@@ -513,7 +514,8 @@ __device__ inline void troe_fx(const double* fd, int n, double T, double invT, d
 // scr[u * R + r], u = 0..6: {dq/dC through each of the 4 slots (an empty slot's entry is not read),
 // phi (coefficient of the efficiencies; pressure-dependent reactions only), sum_j dq/dC_j C_j,
 // dq/dT at fixed C} (rows of R, so that the threads of consecutive reactions store to consecutive
-// words), and the species production rates in w.omega.
+// words), the species production rates in w.omega and the species' sums of the last two rows in w.zc
+// and w.dwT.
 // With kP (adjoint use, requires jac) it also writes P[r] = v . d f / d ln A_r for the weight
 // vector v = vP (N): with q'_r = d q_r / d ln A_r (q_r for elementary and third-body
 // reactions; q_r (Pr/(1+Pr) - d ln F/d ln Pr) for fall-off reactions, whose A is that of
@@ -707,6 +709,18 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
     w.omega[k] = om;
     Qp = fma(w.hRT[k], om, Qp);
     if (k < d) f[1 + k] = m.sp[k * kSpDoubles] * om * s.inv_rho;
+    if (jac) {
+      // the species' sums of sum_j dq/dC_j C_j and dq/dT
+      S zc = cst<S>(0.0), dw = cst<S>(0.0);
+      for (e = eb; e < ee; ++e) {
+        const double nu = m.sr_nu[e];
+        const int r = m.sr_idx[e];
+        zc = fma(nu, scr[5 * m.R + r], zc);
+        dw = fma(nu, scr[6 * m.R + r], dw);
+      }
+      w.zc[k] = zc;
+      w.dwT[k] = dw;
+    }
   }
   const S Q = g.sum(Qp) * kRu * s.T;
   s.fT = -Q * s.inv_rho * s.inv_cp;
@@ -899,9 +913,24 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
     double om = 0.0;
     const int len = m.sr_ptr[k + 1] - m.sr_ptr[k];
     const uint32_t* e = m.srx + k;
-    for (int i = 0; i < len; ++i) {
-      const uint32_t v = e[(size_t)i * K];
-      om = fma(__hiloint2double((int)(v & 0xffff0000u), 0), w.q[v & 0xffffu], om);
+    if (jac) {
+      // with the species' sums of sum_j dq/dC_j C_j and dq/dT
+      double zc = 0.0, dw = 0.0;
+      for (int i = 0; i < len; ++i) {
+        const uint32_t v = e[(size_t)i * K];
+        const double nu = __hiloint2double((int)(v & 0xffff0000u), 0);
+        const double* o = scr + (v & 0xffffu);
+        om = fma(nu, w.q[v & 0xffffu], om);
+        zc = fma(nu, o[5 * R], zc);
+        dw = fma(nu, o[6 * R], dw);
+      }
+      w.zc[k] = zc;
+      w.dwT[k] = dw;
+    } else {
+      for (int i = 0; i < len; ++i) {
+        const uint32_t v = e[(size_t)i * K];
+        om = fma(__hiloint2double((int)(v & 0xffff0000u), 0), w.q[v & 0xffffu], om);
+      }
     }
     w.omega[k] = om;
     Qp = fma(w.hRT[k], om, Qp);
@@ -939,57 +968,58 @@ __device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Gr
 
 // Assemble the analytical Jacobian (Sec. 2.3) at the state of the preceding cell_rates(jac)
 // call.  J (overwritten) holds the per-reaction data on entry, Z is N*N scratch, J receives
-// -d f / d phi (stored negated, so that W = I/(gamma h) - J is a copy plus the diagonal).  Chain rule through C_j = rho Y_j / W_j, rho = p Wbar/(Ru T), Y_K = 1 - sum Y_i;
+// -d f / d phi (stored negated, so that W = I/(gamma h) - J is a copy plus the diagonal).  Chain rule
+// through C_j = rho Y_j / W_j, rho = p Wbar/(Ru T), Y_K = 1 - sum Y_i;
 // Z rows k < K-1 hold d omega_k / dC, row K-1 holds d Q / dC (Q = sum_k H_k omega_k).
-template <int G, class S>
-__device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScalarsT<S>& s, const S* f,
-                              const EvalMem<S>& w, S* J, S* Z) {
+// Bound by FP64 issue; the plans are read as packed 4-byte words in the threads' order (8 KB of the
+// SM's L1 is left beside the cells' shared memory for 53 species, so their volume counts).
+template <int G>
+__device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScalars& s, const double* f,
+                              const EvalMem<double>& w, double* J, double* Z) {
   constexpr int NT = Grp<G>::NT;
   const int K = m.K, N = K, d = K - 1;
-  const S* scr = J;
-  for (int e = g.t; e < N * N; e += NT) Z[e] = cst<S>(0.0);
-  g.sync();
-  // mass-action part: one thread per receiving Z entry sums its contributions (a fixed plan
-  // built with the mechanism; no two threads write the same entry, no atomics).  Each thread
-  // takes four entries at once, NT apart, so that four independent FMA chains hide each other's
-  // FP64 latency; every entry still sums its contributions in plan order.
-  for (int e0 = g.t; e0 < m.zg_entries; e0 += 4 * NT) {
-    int cb[4], len[4];
-    S acc[4];
-    int lmax = 0;
+  const double* scr = J;
+  // mass-action part: one thread per entry of the species rows sums its contributions (a fixed plan
+  // built with the mechanism; no two threads write the same entry, no atomics).  The entries are in
+  // order of decreasing list length and the plan is stored contribution by contribution: the c-th one of
+  // entry e, for the entries that have it, at zgb[c] + e.  Each thread takes four entries at once, NT
+  // apart (independent FMA chains); every entry sums its contributions in plan order, and the
+  // entries without any, at the end, become zero.
+  const int entries = d * K;
+  for (int e0 = g.t; e0 < entries; e0 += 4 * NT) {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    int b = m.zgb[0];
+    for (int c = 0;; ++c) {
+      const int nb = m.zgb[c + 1], have = nb - b;
+      if (e0 >= have) break;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = e0 + q * NT;
-      const bool ok = e < m.zg_entries;
-      cb[q] = ok ? m.zg_ptr[e] : 0;
-      len[q] = ok ? m.zg_ptr[e + 1] - cb[q] : 0;
-      lmax = max(lmax, len[q]);
-      acc[q] = cst<S>(0.0);
-    }
-    for (int c = 0; c < lmax; ++c) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (c < len[q]) acc[q] = fma(m.zg_coef[cb[q] + c], scr[m.zg_src[cb[q] + c]], acc[q]);
+      for (int q = 0; q < 4; ++q) {
+        const int e = e0 + q * NT;
+        if (e < have) {
+          const uint32_t v = m.zgx[b + e];
+          acc[q] = fma(__hiloint2double((int)(v & 0xffff0000u), 0), scr[v & 0xffffu], acc[q]);
+        }
+      }
+      b = nb;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (e0 + q * NT < m.zg_entries) Z[m.zg_dst[e0 + q * NT]] = acc[q];
+      if (e0 + q * NT < entries) Z[m.zg_dst[e0 + q * NT]] = acc[q];
   }
-  g.sync();
   // efficiency part of the pressure-dependent reactions: Z[k][j] += sum_r v_kr eff_rj over the
   // (row k, reaction r) pairs, v_kr = nu_kr phi_r.  The coefficients go to the stage-vector area
   // first (free while the Jacobian is built).
-  S* v = w.pv;
+  double* v = w.pv;
   for (int c = g.t; c < m.n_pairs; c += NT) v[c] = m.pr_nu[c] * scr[4 * m.R + m.pr_pd[c]];
   g.sync();
   {
     // four (row, column) items per thread at once, NT apart (independent FMA chains); each item
-    // sums its row's pairs in plan order
+    // continues its entry's sum with its row's pairs in plan order
     const float invK = 1.0f / (float)K;
     const int items = m.n_prows * K;
     for (int x0 = g.t; x0 < items; x0 += 4 * NT) {
       int zi[4], jj[4], cb[4], len[4];
-      S acc[4];
+      double acc[4];
       int lmax = 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -1002,7 +1032,7 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
         cb[q] = m.pr_ptr[row];
         len[q] = ok ? m.pr_ptr[row + 1] - cb[q] : 0;
         lmax = max(lmax, len[q]);
-        acc[q] = cst<S>(0.0);
+        acc[q] = Z[zi[q]];
       }
       for (int c = 0; c < lmax; ++c) {
 #pragma unroll
@@ -1011,106 +1041,90 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (x0 + q * NT < items) Z[zi[q]] += acc[q];
+        if (x0 + q * NT < items) Z[zi[q]] = acc[q];
     }
   }
   g.sync();
-  // per-species gathers of sum_j dq/dC_j C_j and dq/dT; enthalpy weights of the species rows
-  const double invWd = m.sp[d * kSpDoubles + 1];
-  const S RuT = kRu * s.T;
-  S* wq = w.wq;
-  for (int k = g.t; k < d; k += NT) {
-    // two partial sums each (four independent FMA chains)
-    S zc0 = cst<S>(0.0), dw0 = cst<S>(0.0), zc1 = cst<S>(0.0), dw1 = cst<S>(0.0);
-    const int eb = m.sr_ptr[k], ee = m.sr_ptr[k + 1];
-    int e = eb;
-    for (; e + 1 < ee; e += 2) {
-      const double nu0 = m.sr_nu[e], nu1 = m.sr_nu[e + 1];
-      const int r0 = m.sr_idx[e], r1 = m.sr_idx[e + 1];
-      zc0 = fma(nu0, scr[5 * m.R + r0], zc0);
-      dw0 = fma(nu0, scr[6 * m.R + r0], dw0);
-      zc1 = fma(nu1, scr[5 * m.R + r1], zc1);
-      dw1 = fma(nu1, scr[6 * m.R + r1], dw1);
+  // enthalpy weights of the species rows and per-row and per-column factors: mass conservation
+  // (sum_k W_k omega_k = 0) gives omega_K = -sum_{k<K} (W_k/W_K) omega_k, so
+  // Q = sum_k H_k omega_k = sum_{k<K} (H_k - H_K W_k/W_K) omega_k: the enthalpy row is a weighted sum of
+  // the species rows
+  const double* sp = m.spf;  // W at [k], 1/W at [K + k]
+  const double invWd = sp[K + d];
+  const double RuT = kRu * s.T;
+  double* wq = w.wq;
+  {
+    const double hd = w.hRT[d] * invWd;
+    for (int k = g.t; k < d; k += NT) {
+      const double Wk = sp[k];
+      wq[k] = RuT * fma(-hd, Wk, w.hRT[k]);
+      w.rowA[k] = Wk * invWd * Z[k * N + d];
+      w.rowB[k] = Wk * s.inv_rho * (w.zc[k] - w.omega[k]);
+      w.ccol[k] = -s.Wbar * (sp[K + k] - invWd);
     }
-    if (e < ee) {
-      const double nu = m.sr_nu[e];
-      const int r = m.sr_idx[e];
-      zc0 = fma(nu, scr[5 * m.R + r], zc0);
-      dw0 = fma(nu, scr[6 * m.R + r], dw0);
-    }
-    w.zc[k] = zc0 + zc1;
-    w.dwT[k] = dw0 + dw1;
-    // mass conservation (sum_k W_k omega_k = 0) gives omega_K = -sum_{k<K} (W_k/W_K) omega_k, so
-    // Q = sum_k H_k omega_k = sum_{k<K} (H_k - H_K W_k/W_K) omega_k: the enthalpy row is a
-    // weighted sum of the species rows
-    wq[k] = RuT * (w.hRT[k] - w.hRT[d] * m.sp[k * kSpDoubles] * invWd);
   }
   g.sync();
-  // enthalpy row Z_Q[j] = sum_k wq_k Z[k][j] (stored in row K-1), with sum_j Z_Q[j] C_j and
-  // dQ/dT|_C = sum_k wq_k dw_k/dT|_C
-  S zqc = cst<S>(0.0), dqt = cst<S>(0.0), cpw = cst<S>(0.0);
+  // enthalpy row Z_Q[j] = sum_k wq_k Z[k][j] (stored in row K-1), with sum_j Z_Q[j] C_j and the part
+  // of dQ/dT that is not in it: sum_k wq_k dw_k/dT|_C + Ru sum_j cp_j omega_j
+  double zqc = 0.0, dqt = 0.0;
   for (int j = g.t; j < K; j += NT) {
-    S a0 = cst<S>(0.0), a1 = cst<S>(0.0), a2 = cst<S>(0.0), a3 = cst<S>(0.0);
+    double a0 = 0.0, a1 = 0.0;
     int k = 0;
-    for (; k + 3 < d; k += 4) {
+    for (; k + 1 < d; k += 2) {
       a0 = fma(wq[k], Z[k * N + j], a0);
       a1 = fma(wq[k + 1], Z[(k + 1) * N + j], a1);
-      a2 = fma(wq[k + 2], Z[(k + 2) * N + j], a2);
-      a3 = fma(wq[k + 3], Z[(k + 3) * N + j], a3);
     }
-    for (; k < d; ++k) a0 = fma(wq[k], Z[k * N + j], a0);
-    const S zq = (a0 + a1) + (a2 + a3);
+    if (k < d) a0 = fma(wq[k], Z[k * N + j], a0);
+    const double zq = a0 + a1;
     Z[d * N + j] = zq;
     zqc = fma(zq, w.C[j], zqc);
-    cpw = fma(w.cpR[j], w.omega[j], cpw);
+    dqt = fma(kRu * w.cpR[j], w.omega[j], dqt);
+    if (j < d) dqt = fma(wq[j], w.dwT[j], dqt);
   }
-  for (int k = g.t; k < d; k += NT) dqt = fma(wq[k], w.dwT[k], dqt);
   g.sum2(zqc, dqt);
-  cpw = g.sum(cpw) * kRu;
-  g.sync();
-  // per-row and per-column factors
-  for (int k = g.t; k < d; k += NT) {
-    const double Wk = m.sp[k * kSpDoubles];
-    w.rowA[k] = Wk * invWd * Z[k * N + d];
-    w.rowB[k] = Wk * s.inv_rho * (w.zc[k] - w.omega[k]);
-    w.ccol[k] = -s.Wbar * (m.sp[k * kSpDoubles + 1] - invWd);
-  }
-  g.sync();
-  const S inv_cp = s.inv_cp;
-  const S inv_rhocp = s.inv_rho * inv_cp;
-  const S fT = s.fT;
+  if (G == 1) g.sync();  // (with several warps the reduction's barrier has published the row)
+  const double inv_cp = s.inv_cp;
+  const double inv_rhocp = s.inv_rho * inv_cp;
+  const double fT = s.fT;
   // temperature row and column, then the species block (J now overwrites the scratch)
-  const S ZQd = Z[d * N + d];
-  const S cpd = w.cpR[d] * invWd;
+  const double ZQd = Z[d * N + d] * invWd;
+  const double cpd = w.cpR[d] * invWd;
+  const double RuCp = kRu * inv_cp;
   for (int i = g.t; i < d; i += NT) {
-    const S ci = w.ccol[i];
-    const double invWi = m.sp[i * kSpDoubles + 1];
-    const S dQdY = s.rho * (invWi * Z[d * N + i] - invWd * ZQd) + zqc * ci;
-    const S dcpdY = (w.cpR[i] * invWi - cpd) * kRu;
-    J[1 + i] = fma(dQdY, inv_rhocp, fT * (ci + dcpdY * inv_cp));
-    const double Wk = m.sp[i * kSpDoubles];
-    J[(1 + i) * N] = -(Wk * s.inv_rho * (w.dwT[i] - w.zc[i] * s.invT) + f[1 + i] * s.invT);
+    const double ci = w.ccol[i];
+    const double invWi = sp[K + i];
+    const double dQdY = fma(s.rho, fma(invWi, Z[d * N + i], -ZQd), zqc * ci);
+    const double dcpdY = fma(w.cpR[i], invWi, -cpd);
+    J[1 + i] = fma(dQdY, inv_rhocp, fT * fma(dcpdY, RuCp, ci));
+    const double Wr = sp[i] * s.inv_rho;
+    J[(1 + i) * N] = -fma(Wr, fma(-w.zc[i], s.invT, w.dwT[i]), f[1 + i] * s.invT);
   }
-  if (g.t == 0) J[0] = (cpw + dqt - zqc * s.invT) * inv_rhocp + fT * (-s.invT + s.dcp_dT * inv_cp);
+  if (g.t == 0) J[0] = (dqt - zqc * s.invT) * inv_rhocp + fT * (-s.invT + s.dcp_dT * inv_cp);
+  // species block: two FMAs per entry (mwr[k][i] = -W_k / W_i); the threads' entries are NT apart, so
+  // the row and column advance by (NT / d, NT mod d) with at most one wrap
   const int nb = d * d;
-  const float inv_d = 1.0f / (float)d;
-  // two entries per thread and iteration (independent chains), the same operations per entry
+  const int dk = (int)(((float)NT + 0.5f) / (float)d), di = NT - dk * d;
+  int k = (int)(((float)g.t + 0.5f) / (float)d), i = g.t - k * d;
   int e = g.t;
-  for (; e + NT < nb; e += 2 * NT) {
-    const int k0 = (int)(((float)e + 0.5f) * inv_d), i0 = e - k0 * d;
-    const int k1 = (int)(((float)(e + NT) + 0.5f) * inv_d), i1 = e + NT - k1 * d;
-    const double W0 = m.sp[k0 * kSpDoubles], iW0 = m.sp[i0 * kSpDoubles + 1];
-    const double W1 = m.sp[k1 * kSpDoubles], iW1 = m.sp[i1 * kSpDoubles + 1];
-    const S j0 = fma(-w.rowB[k0], w.ccol[i0], fma(-W0 * iW0, Z[k0 * N + i0], w.rowA[k0]));
-    const S j1 = fma(-w.rowB[k1], w.ccol[i1], fma(-W1 * iW1, Z[k1 * N + i1], w.rowA[k1]));
-    J[(1 + k0) * N + 1 + i0] = j0;
-    J[(1 + k1) * N + 1 + i1] = j1;
+  for (; e + 3 * NT < nb; e += 4 * NT) {
+    int at[4];
+    double j[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      at[q] = (1 + k) * N + 1 + i;
+      j[q] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e + q * NT], Z[k * N + i], w.rowA[k]));
+      k += dk;
+      i += di;
+      if (i >= d) { i -= d; ++k; }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) J[at[q]] = j[q];
   }
-  if (e < nb) {
-    const int k = (int)(((float)e + 0.5f) * inv_d), i = e - k * d;
-    const double Wk = m.sp[k * kSpDoubles];
-    const double invWi = m.sp[i * kSpDoubles + 1];
-    J[(1 + k) * N + 1 + i] = fma(-w.rowB[k], w.ccol[i], fma(-Wk * invWi, Z[k * N + i], w.rowA[k]));
+  for (; e < nb; e += NT) {
+    J[(1 + k) * N + 1 + i] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e], Z[k * N + i], w.rowA[k]));
+    k += dk;
+    i += di;
+    if (i >= d) { i -= d; ++k; }
   }
   g.sync();
 }
@@ -1137,19 +1151,8 @@ __device__ void cell_jacobian_vjp(const DevMech& m, const Grp<G>& g, const CellS
   S* fB = fA + npd;
   S* t = tz;
   S* zq = tz + K;
-  // species: enthalpy weights and the gathers of sum_j dq/dC_j C_j and dq/dT
-  for (int k = g.t; k < d; k += NT) {
-    S zc = cst<S>(0.0), dw = cst<S>(0.0);
-    for (int e = m.sr_ptr[k]; e < m.sr_ptr[k + 1]; ++e) {
-      const double nu = m.sr_nu[e];
-      const int r = m.sr_idx[e];
-      zc = fma(nu, scr[5 * R + r], zc);
-      dw = fma(nu, scr[6 * R + r], dw);
-    }
-    w.zc[k] = zc;
-    w.dwT[k] = dw;
-    w.wq[k] = RuT * (w.hRT[k] - w.hRT[d] * m.sp[k * kSpDoubles] * invWd);
-  }
+  // enthalpy weights
+  for (int k = g.t; k < d; k += NT) w.wq[k] = RuT * (w.hRT[k] - w.hRT[d] * m.sp[k * kSpDoubles] * invWd);
   g.sync();
   // per-reaction row weights
   for (int r = g.t; r < R; r += NT) {

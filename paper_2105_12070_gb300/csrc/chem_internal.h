@@ -66,14 +66,15 @@ struct HostMech {
   // species production lists, entry e of species k at [e * K + k]: reaction index in the low half,
   // the top 16 bits of the net coefficient as a double in the high half (small integers have no others)
   std::vector<uint32_t> srx;
-  // Jacobian gather plan (mass-action part).  Z entries (species row k < K-1, column j) that
-  // receive contributions, each a list of (per-reaction scratch index src, coefficient):
-  // Z[dst] = sum coef * s[src].  (src2 is kept for the layout and is always -1.)
-  std::vector<int> zg_ptr;             // [n_entries + 1]
-  std::vector<int> zg_dst;             // [n_entries] row * K + col
-  std::vector<int> zg_src;             // [n_contrib]
-  std::vector<int> zg_src2;            // [n_contrib]
-  std::vector<double> zg_coef;         // [n_contrib]
+  // Jacobian gather plan (mass-action part).  Every Z entry of the species rows (k < K-1, all columns)
+  // sums coef * s[src] over its contributions (src an index into the per-reaction scratch).  Entries in
+  // order of decreasing list length; the c-th contribution of entry e, where it has one, is at
+  // zgx[zgb[c] + e]: src in the low half, the top 16 bits of the coefficient (a small integer) as a
+  // double in the high half.
+  std::vector<int> zg_dst;             // [(K-1) K] row * K + col
+  std::vector<int> zgb;                // [longest list + 2], the last two equal
+  std::vector<uint32_t> zgx;           // [contributions]
+  std::vector<double> mwr;             // [K-1][K-1] -W_k / W_i
   // Efficiency part: for each species row k < K-1, the pressure-dependent reactions in it:
   // (pd index, net coefficient)
   std::vector<int> pr_ptr;             // [K + 1]
@@ -107,12 +108,10 @@ struct DevMech {
   const int* sr_ptr;
   const int* sr_idx;
   const double* sr_nu;
-  int zg_entries;
-  const int* zg_ptr;
   const int* zg_dst;
-  const int* zg_src;
-  const int* zg_src2;
-  const double* zg_coef;
+  const int* zgb;
+  const uint32_t* zgx;
+  const double* mwr;
   const int* pr_ptr;
   const int* pr_pd;
   const double* pr_nu;

@@ -592,11 +592,10 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   const size_t o_srp = place(h.sr_ptr.size() * sizeof(int));
   const size_t o_sri = place(std::max<size_t>(1, h.sr_idx.size()) * sizeof(int));
   const size_t o_srn = place(std::max<size_t>(1, h.sr_nu.size()) * sizeof(double));
-  const size_t o_zgp = place(h.zg_ptr.size() * sizeof(int));
   const size_t o_zgd = place(std::max<size_t>(1, h.zg_dst.size()) * sizeof(int));
-  const size_t o_zgs = place(std::max<size_t>(1, h.zg_src.size()) * sizeof(int));
-  const size_t o_zgs2 = place(std::max<size_t>(1, h.zg_src2.size()) * sizeof(int));
-  const size_t o_zgc = place(std::max<size_t>(1, h.zg_coef.size()) * sizeof(double));
+  const size_t o_zgb = place(h.zgb.size() * sizeof(int));
+  const size_t o_zgx = place(std::max<size_t>(1, h.zgx.size()) * sizeof(uint32_t));
+  const size_t o_mwr = place(std::max<size_t>(1, h.mwr.size()) * sizeof(double));
   const size_t o_prp = place(h.pr_ptr.size() * sizeof(int));
   const size_t o_prd = place(std::max<size_t>(1, h.pr_pd.size()) * sizeof(int));
   const size_t o_prn = place(std::max<size_t>(1, h.pr_nu.size()) * sizeof(double));
@@ -627,11 +626,10 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   put(o_srp, h.sr_ptr.data(), h.sr_ptr.size() * sizeof(int));
   put(o_sri, h.sr_idx.data(), h.sr_idx.size() * sizeof(int));
   put(o_srn, h.sr_nu.data(), h.sr_nu.size() * sizeof(double));
-  put(o_zgp, h.zg_ptr.data(), h.zg_ptr.size() * sizeof(int));
   put(o_zgd, h.zg_dst.data(), h.zg_dst.size() * sizeof(int));
-  put(o_zgs, h.zg_src.data(), h.zg_src.size() * sizeof(int));
-  put(o_zgs2, h.zg_src2.data(), h.zg_src2.size() * sizeof(int));
-  put(o_zgc, h.zg_coef.data(), h.zg_coef.size() * sizeof(double));
+  put(o_zgb, h.zgb.data(), h.zgb.size() * sizeof(int));
+  put(o_zgx, h.zgx.data(), h.zgx.size() * sizeof(uint32_t));
+  put(o_mwr, h.mwr.data(), h.mwr.size() * sizeof(double));
   put(o_prp, h.pr_ptr.data(), h.pr_ptr.size() * sizeof(int));
   put(o_prd, h.pr_pd.data(), h.pr_pd.size() * sizeof(int));
   put(o_prn, h.pr_nu.data(), h.pr_nu.size() * sizeof(double));
@@ -671,12 +669,10 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   d.sr_ptr = reinterpret_cast<const int*>(b + o_srp);
   d.sr_idx = reinterpret_cast<const int*>(b + o_sri);
   d.sr_nu = reinterpret_cast<const double*>(b + o_srn);
-  d.zg_entries = (int)h.zg_dst.size();
-  d.zg_ptr = reinterpret_cast<const int*>(b + o_zgp);
   d.zg_dst = reinterpret_cast<const int*>(b + o_zgd);
-  d.zg_src = reinterpret_cast<const int*>(b + o_zgs);
-  d.zg_src2 = reinterpret_cast<const int*>(b + o_zgs2);
-  d.zg_coef = reinterpret_cast<const double*>(b + o_zgc);
+  d.zgb = reinterpret_cast<const int*>(b + o_zgb);
+  d.zgx = reinterpret_cast<const uint32_t*>(b + o_zgx);
+  d.mwr = reinterpret_cast<const double*>(b + o_mwr);
   d.pr_ptr = reinterpret_cast<const int*>(b + o_prp);
   d.pr_pd = reinterpret_cast<const int*>(b + o_prd);
   d.pr_nu = reinterpret_cast<const double*>(b + o_prn);

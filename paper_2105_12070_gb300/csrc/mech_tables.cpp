@@ -215,7 +215,7 @@ struct FileReaction {
 // enthalpy (rows, so that the threads of consecutive reactions touch consecutive words).
 void build_jacobian_plan(HostMech& m) {
   const int K = m.K, d = K - 1;
-  struct Contrib { int dst, src, src2; double coef; };
+  struct Contrib { int dst, src; double coef; };
   std::vector<Contrib> cs;
   // (the columns are the four slots themselves: a species in two slots of a reaction receives the
   // derivatives through both)
@@ -227,34 +227,34 @@ void build_jacobian_plan(HostMech& m) {
       for (int rs = 0; rs < 4; ++rs) {
         const int row = ii[8 + rs];
         if (row < 0) continue;
-        cs.push_back({row * K + col, u * m.R + r, -1, (double)ii[12 + rs]});
+        cs.push_back({row * K + col, u * m.R + r, (double)ii[12 + rs]});
       }
     }
   }
-  std::stable_sort(cs.begin(), cs.end(), [](const Contrib& a, const Contrib& b) { return a.dst < b.dst; });
-  // entries, then ordered by decreasing list length so that threads of a pass get similar work
-  std::vector<std::pair<int, int>> ent;  // (begin, end) into cs
-  for (size_t i = 0; i < cs.size();) {
-    size_t j = i;
-    while (j < cs.size() && cs[j].dst == cs[i].dst) ++j;
-    ent.push_back({(int)i, (int)j});
-    i = j;
-  }
-  std::stable_sort(ent.begin(), ent.end(),
-                   [](const std::pair<int, int>& a, const std::pair<int, int>& b) {
-                     return (a.second - a.first) > (b.second - b.first);
-                   });
-  m.zg_ptr.assign(1, 0);
-  m.zg_dst.clear(); m.zg_src.clear(); m.zg_src2.clear(); m.zg_coef.clear();
-  for (const auto& e : ent) {
-    m.zg_dst.push_back(cs[e.first].dst);
-    for (int i = e.first; i < e.second; ++i) {
-      m.zg_src.push_back(cs[i].src);
-      m.zg_src2.push_back(cs[i].src2);
-      m.zg_coef.push_back(cs[i].coef);
+  std::vector<std::vector<Contrib>> ent((size_t)d * K);  // one list per entry of the species rows
+  for (const Contrib& c : cs) ent[c.dst].push_back(c);
+  std::vector<int> ord(ent.size());
+  for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int)i;
+  // decreasing list length, so that the threads of a pass get similar work
+  std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return ent[a].size() > ent[b].size(); });
+  m.zg_dst = ord;
+  m.zgb.assign(1, 0);
+  m.zgx.clear();
+  const size_t longest = ent.empty() ? 0 : ent[ord[0]].size();
+  for (size_t c = 0; c < longest; ++c) {
+    for (size_t i = 0; i < ord.size() && ent[ord[i]].size() > c; ++i) {
+      const Contrib& x = ent[ord[i]][c];
+      uint64_t b;
+      std::memcpy(&b, &x.coef, 8);
+      m.zgx.push_back((uint32_t)x.src | (uint32_t)(b >> 48) << 16);
     }
-    m.zg_ptr.push_back((int)m.zg_src.size());
+    m.zgb.push_back((int)m.zgx.size());
   }
+  m.zgb.push_back((int)m.zgx.size());
+  m.mwr.assign((size_t)d * d, 0.0);
+  for (int k = 0; k < d; ++k)
+    for (int i = 0; i < d; ++i)
+      m.mwr[(size_t)k * d + i] = -m.sp[(size_t)k * kSpDoubles] / m.sp[(size_t)i * kSpDoubles];
   // efficiency rows
   m.pr_ptr.assign(K + 1, 0);
   m.pr_pd.clear(); m.pr_nu.clear();
