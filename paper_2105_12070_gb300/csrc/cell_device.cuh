@@ -1471,6 +1471,28 @@ __device__ bool cell_lu(const Grp<G>& g, S* A, int N, int* piv, int* perm, S* in
   return ok;
 }
 
+// The warp's pivot candidate: the lane with the largest key (0: no entry), ties to the lowest row, writes
+// (key, row, carried value) to out, integers as bits.  Two or three warp reductions (redux.sync) in
+// place of five rounds of five shuffles.
+template <typename S>
+__device__ inline void warp_candidate(long long key, int row, double carried, int none, int lane, double* out) {
+  bool mine = true;
+  if (std::is_same<S, double>::value) {
+    const unsigned hi = (unsigned)((unsigned long long)key >> 32);
+    const unsigned top = __reduce_max_sync(kFull, hi);
+    mine = hi == top;
+  }
+  const unsigned lo = mine ? (unsigned)key : 0u;
+  const unsigned top = __reduce_max_sync(kFull, lo);  // by every lane, before the test below
+  mine = mine && lo == top;
+  const int first = __reduce_min_sync(kFull, mine ? row : 0x7fffffff);
+  if (first == none ? lane == 0 : mine && row == first) {
+    out[0] = __longlong_as_double(key);
+    out[1] = __longlong_as_double(row);
+    out[2] = carried;
+  }
+}
+
 // The same factorisation with two group barriers per pivot column instead of four (the same
 // pivots and the same operations on every entry in the same order, so the factors are bitwise
 // those of cell_lu):
@@ -1490,26 +1512,15 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
   bool ok = true;
   // pivot candidates of column 0
   {
-    long long best = -1;
+    long long best = 0;
     int bi = N;
     double bv = 0.0;
     for (int i = g.t; i < N; i += NT) {
       const S a = A[i * N];
-      const long long v = abs_key(a);
+      const long long v = abs_key(a) + 1;
       if (v > best) { best = v; bi = i; bv = lu_carry(a); }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ob = __shfl_xor_sync(kFull, best, o);
-      const int oi = __shfl_xor_sync(kFull, bi, o);
-      const double ov = __shfl_xor_sync(kFull, bv, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; bv = ov; }
-    }
-    if (g.lane() == 0) {
-      cand[3 * g.warp()] = __longlong_as_double(best);
-      cand[3 * g.warp() + 1] = __longlong_as_double(bi);
-      cand[3 * g.warp() + 2] = bv;
-    }
+    warp_candidate<S>(best, bi, bv, N, g.lane(), cand + 3 * g.warp());
   }
   g.sync();
   for (int k = 0; k < N; ++k) {
@@ -1523,7 +1534,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
       const int oi = (int)__double_as_longlong(cr[3 * w + 1]);
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; bv = cr[3 * w + 2]; }
     }
-    if (best <= 0) ok = false;  // zero column: singular
+    if (best <= 1) ok = false;  // zero column: singular
     // interchange rows k and bi in every other column; scaled multipliers of column k (the pivot
     // row's multiplier is the old row k's entry, and the pivot moves to the diagonal)
     if (bi != k)
@@ -1560,7 +1571,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
     // trailing update: column k+1 first (its entries are the next pivot's candidates, each thread
     // keeping the largest it produced), then the other columns
     const int mm = N - k - 1;
-    long long nb = -1;
+    long long nb = 0;
     int ni = N;
     double nv = 0.0;
     if (mm > 0) {
@@ -1571,7 +1582,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
       for (int i = g.t; i < mm; i += NT) {
         const S r = fma(-Ak[i * N], u0, T0[i * N]);
         T0[i * N] = r;
-        const long long v = abs_key(r);
+        const long long v = abs_key(r) + 1;
         if (v > nb) { nb = v; ni = k + 1 + i; nv = lu_carry(r); }
       }
       const int mc = mm - 1;  // columns k+2 .. N-1
@@ -1606,21 +1617,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
         }
       }
     }
-    if (k + 1 < N) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ob = __shfl_xor_sync(kFull, nb, o);
-        const int oi = __shfl_xor_sync(kFull, ni, o);
-        const double ov = __shfl_xor_sync(kFull, nv, o);
-        if (ob > nb || (ob == nb && oi < ni)) { nb = ob; ni = oi; nv = ov; }
-      }
-      if (g.lane() == 0) {
-        double* cw = cand + ((k + 1) & 1) * 3 * G;
-        cw[3 * g.warp()] = __longlong_as_double(nb);
-        cw[3 * g.warp() + 1] = __longlong_as_double(ni);
-        cw[3 * g.warp() + 2] = nv;
-      }
-    }
+    if (k + 1 < N) warp_candidate<S>(nb, ni, nv, N, g.lane(), cand + ((k + 1) & 1) * 3 * G + 3 * g.warp());
     g.sync();
   }
   // compose the row interchanges: row i of the factors is row perm[i] of the original matrix
