@@ -118,8 +118,7 @@ __device__ inline EvalMem<S> adj_eval_mem(double* base, const AdjPlan& p) {
 
 template <int G>
 __device__ inline void solve_t(const Grp<G>& g, const AdjMem& w, int N, double* x) {
-  if (g.warp() == g.lead) warp_lu_solve_t(w.M, N, w.perm, w.invdiag, x, x);
-  g.sync();
+  group_lu_solve<G, true>(g, w.M, N, w.perm, w.invdiag, x);
 }
 
 // One accepted step backwards: w.y = y_n, h = h_n, w.lam = dL/dy_{n+1} on entry; dL/dy_n in
@@ -139,7 +138,7 @@ __device__ bool adjoint_step(const DevMech& m, const Grp<G>& g, const AdjPlan& p
   cell_jacobian(m, g, s0, w.f, ed, LU, w.M + plan.SA);
   for (int i = g.t; i < N; i += NT) LU[i * N + i] += gh;
   g.sync();
-  if (!cell_lu<G, double>(g, LU, N, w.piv, w.perm, w.invdiag)) return false;
+  if (!cell_lu_default<G, double>(g, LU, N, w.piv, w.perm, w.invdiag)) return false;
   // the four stage increments
   for (int i = g.t; i < N; i += NT) w.u[0][i] = w.f[i];
   g.sync();

@@ -1961,12 +1961,98 @@ __device__ void warp_lu_solve_t(const double* A, int N, const int* perm, const d
   else warp_lu_solve_t_s<4>(A, N, perm, invdiag, b, x);
 }
 
-template <int G>
-__device__ inline void cell_solve(const Grp<G>& g, const double* A, int N, const int* perm, const double* invdiag,
-                                  double* x) {
-  if (g.warp() == g.lead) warp_lu_solve(A, N, perm, invdiag, x);
+// The same substitutions by the first S warps of the group (from its lead warp on): warp s holds rows
+// 32 s .. 32 s + 31, one per lane.  The warp that owns a block of 32 columns solves its triangle by
+// shuffles and publishes the solved values in x, 8 at a time; the warps with rows still to update
+// apply those 8 columns while it solves the next 8.  A row's columns are applied in the same order as
+// in the single-warp form (the same bits), which issues S FMAs per column from one warp; here the
+// chain is N columns of one FMA and a shuffle plus one lag of 8 columns per block.  x in and out;
+// kT: with the transposed factors, x <- W^-T x.
+template <int G, int S, bool kT>
+__device__ void group_lu_solve_s(const Grp<G>& g, const double* A, int N, const int* perm, const double* invdiag,
+                                 double* x) {
+  const int s = (g.warp() - g.lead + G) % G;
+  const int lane = g.lane(), i = lane + 32 * s;
+  const bool row = s < S && i < N;
+  // entry (i, j) of the factor that the sweep uses: L then U', or U'^T then L^T
+  const double* Ai = A + (size_t)(row ? i : 0) * (kT ? 1 : N);
+  const int cs = kT ? N : 1;
+  double xr = row ? x[kT ? i : perm[i]] : 0.0;
+  g.sync();
+#pragma unroll
+  for (int jb = 0; jb < S; ++jb) {
+    for (int j0 = 32 * jb; j0 < min(32 * jb + 32, N); j0 += 8) {
+      if (s == jb) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + c;
+          const double xj = __shfl_sync(kFull, xr, j & 31);
+          if (i > j && row) xr = fma(-Ai[j * cs], xj, xr);
+        }
+        if (jb < S - 1 && lane >= (j0 & 31) && lane < (j0 & 31) + 8) x[i] = xr;
+      }
+      if (jb < S - 1) {
+        g.sync();
+        if (s > jb && row) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) xr = fma(-Ai[(j0 + c) * cs], x[j0 + c], xr);
+        }
+      }
+    }
+  }
+  if (row) xr *= invdiag[i];
+#pragma unroll
+  for (int jb = S - 1; jb >= 0; --jb) {
+    const int last = min(32 * jb + 31, N - 1);
+    for (int j0 = last & ~7; j0 >= 32 * jb; j0 -= 8) {
+      if (s == jb) {
+#pragma unroll
+        for (int c = 7; c >= 0; --c) {
+          const int j = j0 + c;
+          const double xj = __shfl_sync(kFull, xr, j & 31);
+          if (i < j && j < N) xr = fma(-Ai[j * cs], xj, xr);
+        }
+        if (jb > 0 && row && lane >= (j0 & 31) && lane < (j0 & 31) + 8) x[i] = xr;
+      }
+      if (jb > 0) {
+        g.sync();
+        if (s < jb) {
+#pragma unroll
+          for (int c = 7; c >= 0; --c)
+            if (j0 + c < N) xr = fma(-Ai[(j0 + c) * cs], x[j0 + c], xr);
+        }
+      }
+    }
+  }
+  if (kT) g.sync();  // x is written in another order than it was published in
+  if (row) x[kT ? perm[i] : i] = xr;
   g.sync();
 }
 
+// x <- W^-1 x (kT: W^-T x) by the group: split over its warps where it has one per 32 rows, else by its
+// lead warp.
+template <int G, bool kT>
+__device__ __noinline__ void group_lu_solve(Grp<G> g, const double* A, int N, const int* perm, const double* invdiag,
+                                            double* x) {
+  if (G >= 2 && N > 32 && N <= 64) {
+    group_lu_solve_s<G, 2, kT>(g, A, N, perm, invdiag, x);
+  } else if (G >= 4 && N > 64 && N <= 96) {
+    group_lu_solve_s<G, 3, kT>(g, A, N, perm, invdiag, x);
+  } else if (G >= 4 && N > 96) {
+    group_lu_solve_s<G, 4, kT>(g, A, N, perm, invdiag, x);
+  } else {
+    if (g.warp() == g.lead) {
+      if (kT) warp_lu_solve_t(A, N, perm, invdiag, x, x);
+      else warp_lu_solve(A, N, perm, invdiag, x);
+    }
+    g.sync();
+  }
+}
+
+template <int G>
+__device__ inline void cell_solve(const Grp<G>& g, const double* A, int N, const int* perm, const double* invdiag,
+                                  double* x) {
+  group_lu_solve<G, false>(g, A, N, perm, invdiag, x);
+}
 
 }  // namespace
