@@ -72,6 +72,8 @@ struct is_dual<Dual> : std::true_type {};
 
 __device__ inline double val(double a) { return a; }
 __device__ inline double val(const Dual& a) { return a.v; }
+__device__ inline double der(double) { return 0.0; }
+__device__ inline double der(const Dual& a) { return a.d; }
 
 __device__ inline Dual operator+(Dual a, Dual b) { return Dual(a.v + b.v, a.d + b.d); }
 __device__ inline Dual operator+(Dual a, double b) { return Dual(a.v + b, a.d); }
@@ -109,9 +111,14 @@ __device__ inline Dual fma(double a, double b, Dual c) { return Dual(fma(a, b, c
 __device__ inline Dual log(Dual a) { return Dual(log(a.v), a.d / a.v); }
 __device__ inline Dual log10(Dual a) { return Dual(log10(a.v), a.d / (a.v * 2.302585092994045684)); }
 
-// the S-typed constant x
+// the S-typed constant x, and the S-typed value v whose derivative is d (dropped for double)
 template <class S>
 __device__ inline S cst(double x) { return S(x); }
+template <class S>
+__device__ inline S with_der(double v, double d) {
+  if constexpr (is_dual<S>::value) return Dual(v, d);
+  else return v;
+}
 
 // ------------------------------------------------------------------------------------------
 // Cell groups.  G warps (32 G threads) cooperate on one cell; several groups share a CTA and
@@ -477,35 +484,48 @@ __device__ inline void troe(const double* fo, S T, S invT, S Pr, S& F, S& dlF, S
   }
 }
 
-// The same in FP64 with the exponentials and logarithms in fixed point: fd[i * n] = 1 - alpha, alpha,
+// The same with the exponentials and logarithms of the values in fixed point: fd[i * n] = 1 - alpha, alpha,
 // log2(e)/T3, log2(e)/T1, T2 log2(e).  A centre or reduced pressure that is not a positive normal
 // number takes the library logarithm (minus infinity or NaN, as there).
 static __device__ __noinline__ double log10_wide(double x) { return log10(x); }
 __device__ inline double log10_fx(double x) {
   return fx_log2_takes(x) ? fx_value(fx_log2(x)) * 0.30102999566398119521 : log10_wide(x);
 }
-__device__ inline void troe_fx(const double* fd, int n, double T, double invT, double Pr, double& F, double& dlF,
-                               double& dlnF_dT, bool jac) {
+__device__ inline Dual log10_fx(Dual x) { return Dual(log10_fx(x.v), x.d * (fx_rcp(x.v) * 0.43429448190325182765)); }
+__device__ inline double exp2_fx(double x) { return fx_exp2_of(x); }
+__device__ inline Dual exp2_fx(Dual x) {
+  const double e = fx_exp2_of(x.v);
+  return Dual(e, e * (x.d * 0.69314718055994530942));
+}
+// 2^X with the derivative dlnX (along the dual direction) of its natural logarithm
+template <class S>
+__device__ inline S exp2_of_fx(fx_t X, double dlnX) {
+  const double e = fx_exp2(X);
+  if constexpr (is_dual<S>::value) return Dual(e, e * dlnX);
+  else return e;
+}
+template <class S>
+__device__ inline void troe_fx(const double* fd, int n, S T, S invT, S Pr, S& F, S& dlF, S& dlnF_dT, bool jac) {
   const double oma = fd[0], a = fd[n], iT3 = fd[2 * n], iT1 = fd[3 * n], T2 = fd[4 * n];
-  const double e3 = fx_exp2_of(-T * iT3), e1 = fx_exp2_of(-T * iT1), e2 = fx_exp2_of(-T2 * invT);
-  const double Fcent = fma(oma, e3, fma(a, e1, e2));
-  const double L = log10_fx(Fcent);
-  const double nn = fma(-1.27, L, 0.75);
-  const double xc = log10_fx(Pr) + fma(-0.67, L, -0.4);
-  const double den = fma(-0.14, xc, nn);
-  const double iden = fx_rcp(den);
-  const double f1 = xc * iden;
-  const double ig = fx_rcp(fma(f1, f1, 1.0));
-  const double Lg = L * ig;
-  F = fx_exp2_of(Lg * 3.3219280948873623479);
+  const S e3 = exp2_fx(-T * iT3), e1 = exp2_fx(-T * iT1), e2 = exp2_fx(-T2 * invT);
+  const S Fcent = fma(oma, e3, fma(a, e1, e2));
+  const S L = log10_fx(Fcent);
+  const S nn = fma(-1.27, L, 0.75);
+  const S xc = log10_fx(Pr) + fma(-0.67, L, -0.4);
+  const S den = fma(-0.14, xc, nn);
+  const S iden = recip(den);
+  const S f1 = xc * iden;
+  const S ig = recip(fma(f1, f1, 1.0));
+  const S Lg = L * ig;
+  F = exp2_fx(Lg * 3.3219280948873623479);
   if (jac) {
-    const double t = f1 * ig * Lg;  // L f1 / g^2
-    const double iden2 = iden * iden;
+    const S t = f1 * ig * Lg;  // L f1 / g^2
+    const S iden2 = iden * iden;
     dlF = -2.0 * t * (nn * iden2);
     // d Fcent / dT; the table's exponents carry log2(e): times ln 2
-    const double dFc = 0.69314718055994530942 * (T2 * (invT * invT) * e2 - (oma * iT3 * e3 + a * iT1 * e1));
-    const double dL = dFc * fx_rcp(Fcent);  // ln(10) dL/dT
-    const double df1_dL = fma(-0.67, den, xc * (1.27 - 0.14 * 0.67)) * iden2;
+    const S dFc = 0.69314718055994530942 * (T2 * (invT * invT) * e2 - (oma * iT3 * e3 + a * iT1 * e1));
+    const S dL = dFc * recip(Fcent);  // ln(10) dL/dT
+    const S df1_dL = fma(-0.67, den, xc * (1.27 - 0.14 * 0.67)) * iden2;
     dlnF_dT = fma(-2.0 * t, df1_dL, ig) * dL;
   }
 }
@@ -729,77 +749,88 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
   return s;
 }
 
-// The same evaluation for FP64 states whose temperature lies in the mechanism's fixed-point range:
-// the logarithms of the rate and equilibrium constants are summed in 64-bit fixed point and the
+// The same evaluation for states whose temperature lies in the mechanism's fixed-point range: the
+// logarithms of the rate and equilibrium constants are summed in 64-bit fixed point and the
 // exponentials and logarithms evaluated there (fixed_math.cuh), from tables with the constant
 // factors multiplied in.  Bound by FP64 issue (64 clocks per warp instruction and sub-partition):
 // a plain reaction takes 5 FP64 instructions here against 39 in the general form, a species' thermo
 // 17 against about 45.
 // The tables are laid out so that consecutive threads read consecutive words: at this pace the
 // strided records of the general form would be bound by L1 wavefronts.
-template <int G, bool kP>
-__device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p, const double* y, double* f,
-                                     const EvalMem<double>& w, double* scr, bool jac, const double* vP, double* P) {
+// For dual numbers only the values go through fixed point; every exponent is a function of T alone, so
+// its derivative along the direction is the logarithmic derivative that the Jacobian data needs anyway
+// times T's.
+template <int G, class S, bool kP>
+__device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
+                                         const EvalMem<S>& w, S* scr, bool jac, const double* vP, S* P) {
   constexpr int NT = Grp<G>::NT;
+  constexpr bool kDual = is_dual<S>::value;
   const int K = m.K, R = m.R, d = K - 1, npd = m.n_pd, nfo = m.n_fo;
   const double* sp = m.spf;
-  CellScalars s;
+  CellScalarsT<S> s;
   s.T = y[0];
-  double ysum = 0.0, yw = 0.0;
+  const double T = val(s.T), Td = der(s.T);
+  S ysum = cst<S>(0.0), yw = cst<S>(0.0);
   for (int k = g.t; k < d; k += NT) {
-    const double Yk = y[1 + k];
+    const S Yk = y[1 + k];
     ysum += Yk;
     yw = fma(Yk, sp[K + k], yw);
   }
   g.sum2(ysum, yw);
-  const double Yd = 1.0 - ysum;
+  const S Yd = 1.0 - ysum;
   yw = fma(Yd, sp[K + d], yw);
   // the reciprocals of T, yw and p on three lanes of each warp: one Newton iteration for all three
   const int third = g.lane() & 3;
-  const double a3 = third == 0 ? s.T : third == 1 ? yw : p;
+  const double a3 = third == 0 ? T : third == 1 ? val(yw) : p;
   uint64_t rT;
   const double rcp = fx_rcp(a3, rT);
-  s.invT = __shfl_sync(kFull, rcp, 0);
-  s.Wbar = __shfl_sync(kFull, rcp, 1);
+  const double invT = __shfl_sync(kFull, rcp, 0), Wbar = __shfl_sync(kFull, rcp, 1);
   const double invp = __shfl_sync(kFull, rcp, 2);
+  s.invT = with_der<S>(invT, -Td * (invT * invT));
+  s.Wbar = with_der<S>(Wbar, -der(yw) * (Wbar * Wbar));
   s.rho = (p * s.Wbar) * (s.invT * (1.0 / kRu));
   s.inv_rho = (yw * s.T) * (kRu * invp);
-  const fx_t L2 = fx_log2(s.T);
+  const fx_t L2 = fx_log2(T);
   // 1/T in units of 2^-70, with the reciprocal's 62 bits (T in (128, 8192): exponent 7 to 12)
   const int64_t iT = (int64_t)(__shfl_sync(kFull, (unsigned long long)rT, 0) >>
-                               ((int)(__double_as_longlong(s.T) >> 52) - 1029));
+                               ((int)(__double_as_longlong(T) >> 52) - 1029));
   const int64_t L2s = L2 << 7;
-  double cp = 0.0, dcp = 0.0;
+  S cp = cst<S>(0.0), dcp = cst<S>(0.0);
   int64_t* g2 = reinterpret_cast<int64_t*>(w.gRT);  // (g/RT) / ln 2 as fx
   for (int k = g.t; k < K; k += NT) {
-    const double Yk = (k < d) ? y[1 + k] : Yd;
-    const double yiw = Yk * sp[K + k];
-    const double* a = sp + (size_t)(3 + (s.T <= sp[2 * K + k] ? 0 : kSpfRange)) * K + k;
+    const S Yk = (k < d) ? y[1 + k] : Yd;
+    const S yiw = Yk * sp[K + k];
+    const double* a = sp + (size_t)(3 + (T <= sp[2 * K + k] ? 0 : kSpfRange)) * K + k;
     auto c = [&](int i) { return a[(size_t)i * K]; };
-    const double T = s.T;
-    const double cpR = fma(T, fma(T, fma(T, fma(T, c(4), c(3)), c(2)), c(1)), c(0));
-    const double hRT = fma(T, fma(T, fma(T, fma(T, c(8), c(7)), c(6)), c(5)), fma(c(9), s.invT, c(0)));
+    const double cpv = fma(T, fma(T, fma(T, fma(T, c(4), c(3)), c(2)), c(1)), c(0));
+    const double hv = fma(T, fma(T, fma(T, fma(T, c(8), c(7)), c(6)), c(5)), fma(c(9), invT, c(0)));
     auto cx = [&](int i) { return __double_as_longlong(c(i)); };
     const double gT = T * fma(T, fma(T, fma(T, c(16), c(15)), c(14)), c(13));
-    w.C[k] = s.rho * yiw;
-    w.cpR[k] = cpR;
-    w.hRT[k] = hRT;
     g2[k] = cx(10) + fx_mulhi(cx(11), L2s) + 2 * fx_mulhi(cx(12), iT) + fx_of(gT);
-    cp = fma(yiw, cpR, cp);
-    if (jac) {
-      const double dcpR = fma(T, fma(T, fma(T, c(19), c(18)), c(17)), c(1));
+    w.C[k] = s.rho * yiw;
+    if (kDual || jac) {
+      const double dcpv = fma(T, fma(T, fma(T, c(19), c(18)), c(17)), c(1));
+      const S dcpR = with_der<S>(dcpv, kDual ? fma(T, fma(3.0 * T, c(19), 2.0 * c(18)), c(17)) * Td : 0.0);
+      const S cpR = with_der<S>(cpv, dcpv * Td);
       dcp = fma(yiw, dcpR, dcp);
+      cp = fma(yiw, cpR, cp);
+      w.cpR[k] = cpR;
+      w.hRT[k] = with_der<S>(hv, (cpv - hv) * invT * Td);
+    } else {
+      cp = fma(yiw, cst<S>(cpv), cp);
+      w.cpR[k] = cst<S>(cpv);
+      w.hRT[k] = cst<S>(hv);
     }
   }
   if (jac) g.sum2(cp, dcp);
   else cp = g.sum(cp);
   s.cp = cp * kRu;
-  s.inv_cp = fx_rcp(s.cp);
+  s.inv_cp = recip(s.cp);
   s.dcp_dT = dcp * kRu;
   if (G == 1) g.sync();  // (with several warps the reduction's barrier has published C and the thermo)
   for (int r = g.t; r < npd; r += NT) {
     const double* e = m.eff_t + r;
-    double a0 = 0.0, a1 = 0.0;
+    S a0 = cst<S>(0.0), a1 = cst<S>(0.0);
     int k = 0;
     for (; k + 1 < K; k += 2) {
       a0 = fma(e[(size_t)k * npd], w.C[k], a0);
@@ -818,9 +849,9 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
     const uint32_t slots = m.rx4[r];
     const int a0 = slots & 255, a1 = (slots >> 8) & 255, p0 = (slots >> 16) & 255, p1 = slots >> 24;
     const bool two_r = a1 != 255, two_p = p1 != 255;
-    const double Ca0 = w.C[a0], Ca1 = two_r ? w.C[a1] : 1.0;
-    const double Cp0 = w.C[p0], Cp1 = two_p ? w.C[p1] : 1.0;
-    const double pf = Ca0 * Ca1, pr = Cp0 * Cp1;
+    const S Ca0 = w.C[a0], Ca1 = two_r ? w.C[a1] : cst<S>(1.0);
+    const S Cp0 = w.C[p0], Cp1 = two_p ? w.C[p1] : cst<S>(1.0);
+    const S pf = Ca0 * Ca1, pr = Cp0 * Cp1;
     // log2 of the forward constant, and of 1/Kc = exp(sum nu g/RT - dnu ln(Patm/(Ru T))); sums that
     // wrap on the way are right modulo 2^64
     const int64_t Xf = m.fxk[r] + fx_mulhi(m.fxk[R + r], L2s) - fx_mulhi(m.fxk[2 * R + r], iT);
@@ -830,19 +861,31 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
     if (two_r) Xc -= (uint64_t)g2[a1];
     if (dnu != 0) Xc = dnu > 0 ? Xc - (uint64_t)P2 : Xc + (uint64_t)P2;
     const bool pd = r < npd, fo = r < nfo;
-    double kf = fx_exp2(Xf), kr;
+    // d ln k_inf / dT, the reaction enthalpy over RT and d ln Kc / dT
+    S dlnk = cst<S>(0.0), dH = cst<S>(0.0), dlnKc_dT = cst<S>(0.0), dlnk0 = cst<S>(0.0);
+    if (kDual || jac) {
+      dlnk = fma(m.rxd_t[R + r], s.invT, m.rxd_t[r]) * s.invT;
+      dH = w.hRT[p0] - w.hRT[a0];
+      if (two_p) dH += w.hRT[p1];
+      if (two_r) dH -= w.hRT[a1];
+      dlnKc_dT = (dnu == 0 ? dH : dH - (dnu > 0 ? 1.0 : -1.0)) * s.invT;
+      if (fo) dlnk0 = fma(m.fo[(size_t)r * kFoDoubles + 2], s.invT, m.fo[(size_t)r * kFoDoubles + 1]) * s.invT;
+    }
+    S kf = exp2_of_fx<S>(Xf, val(dlnk) * Td), kr;
     // reverse constant: directly from the summed logarithm, except for fall-off reactions
-    const double er = fx_exp2((fx_t)(fo ? Xc : Xc + (uint64_t)Xf));
-    double Mr = 1.0, mfac = 1.0;
-    double F = 1.0, dlF = 0.0, dlnF_dT = 0.0, dk_dM = 0.0, inv1p = 1.0, Pr = 0.0;
+    const S er = exp2_of_fx<S>((fx_t)(fo ? Xc : Xc + (uint64_t)Xf),
+                               ((fo ? 0.0 : val(dlnk)) - val(dlnKc_dT)) * Td);
+    S Mr = cst<S>(1.0), mfac = cst<S>(1.0);
+    S F = cst<S>(1.0), dlF = cst<S>(0.0), dlnF_dT = cst<S>(0.0), dk_dM = cst<S>(0.0), inv1p = cst<S>(1.0),
+      Pr = cst<S>(0.0);
     if (pd) Mr = w.M[r];
     if (fo) {
       const int64_t X0 = m.fxo[r] + fx_mulhi(m.fxo[nfo + r], L2s) - fx_mulhi(m.fxo[2 * nfo + r], iT);
-      const double ratio = fx_exp2(X0 - Xf);  // k0 / k_inf
+      const S ratio = exp2_of_fx<S>(X0 - Xf, (val(dlnk0) - val(dlnk)) * Td);  // k0 / k_inf
       Pr = ratio * Mr;
-      if (m.fo[(size_t)r * kFoDoubles + 7] != 0.0) troe_fx(m.fod + r, nfo, s.T, s.invT, Pr, F, dlF, dlnF_dT, jac);
-      inv1p = fx_rcp(1.0 + Pr);
-      const double kF = kf * (F * inv1p);
+      if (m.fo[(size_t)r * kFoDoubles + 7] != 0.0) troe_fx<S>(m.fod + r, nfo, s.T, s.invT, Pr, F, dlF, dlnF_dT, jac);
+      inv1p = recip(1.0 + Pr);
+      const S kF = kf * (F * inv1p);
       if (jac) dk_dM = ratio * kF * (inv1p + dlF);
       kf = kF * Pr;
       kr = kf * er;
@@ -850,18 +893,18 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
       kr = er;
       if (pd) mfac = Mr;
     }
-    double Rr = kr * pr;
+    S Rr = kr * pr;
     if (!jac) {
-      double q = fma(kf, pf, -Rr);
+      S q = fma(kf, pf, -Rr);
       if (pd) q *= mfac;
       w.q[r] = q;
     } else {
-      double Rf = kf * pf;
-      double q = Rf - Rr;
-      double* o = scr + r;  // o[u * R]
-      double DC = 0.0;
+      S Rf = kf * pf;
+      S q = Rf - Rr;
+      S* o = scr + r;  // o[u * R]
+      S DC = cst<S>(0.0);
       if (pd) {
-        double phi = q;  // plain third body: q / [M]
+        S phi = q;  // plain third body: q / [M]
         if (fo) {
           phi = dk_dM * fma(-er, pr, pf);
         } else {
@@ -875,16 +918,7 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
         DC = phi * Mr;
       }
       w.q[r] = q;
-      double dH = w.hRT[p0] - w.hRT[a0];
-      if (two_p) dH += w.hRT[p1];
-      if (two_r) dH -= w.hRT[a1];
-      const double dHn = dnu == 0 ? dH : dH - (dnu > 0 ? 1.0 : -1.0);
-      const double dlnKc_dT = dHn * s.invT;
-      double dlnk = fma(m.rxd_t[R + r], s.invT, m.rxd_t[r]) * s.invT;  // d ln k_inf / dT
-      if (fo) {
-        const double dlnk0 = fma(m.fo[(size_t)r * kFoDoubles + 2], s.invT, m.fo[(size_t)r * kFoDoubles + 1]) * s.invT;
-        dlnk = fma(inv1p + dlF, dlnk0 - dlnk, dlnk) + dlnF_dT;
-      }
+      if (fo) dlnk = fma(inv1p + dlF, dlnk0 - dlnk, dlnk) + dlnF_dT;
       o[0] = kf * Ca1;
       o[R] = kf * Ca0;
       o[2 * R] = -(kr * Cp1);
@@ -901,25 +935,25 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
           const int k = ii[8 + u];
           if (k >= 0) gw = fma(rd[3 + u] * sp[k], vP[1 + k], gw);
         }
-        const double dq = fo ? q * (Pr * inv1p - dlF) : q;
+        const S dq = fo ? q * (Pr * inv1p - dlF) : q;
         P[r] = dq * s.inv_rho * (gw - vP[0] * (dH * kRu * s.T * s.inv_cp));
       }
     }
   }
   g.sync();
   // species production rates and the source term
-  double Qp = 0.0;
+  S Qp = cst<S>(0.0);
   for (int k = g.t; k < K; k += NT) {
-    double om = 0.0;
+    S om = cst<S>(0.0);
     const int len = m.sr_ptr[k + 1] - m.sr_ptr[k];
     const uint32_t* e = m.srx + k;
     if (jac) {
       // with the species' sums of sum_j dq/dC_j C_j and dq/dT
-      double zc = 0.0, dw = 0.0;
+      S zc = cst<S>(0.0), dw = cst<S>(0.0);
       for (int i = 0; i < len; ++i) {
         const uint32_t v = e[(size_t)i * K];
         const double nu = __hiloint2double((int)(v & 0xffff0000u), 0);
-        const double* o = scr + (v & 0xffffu);
+        const S* o = scr + (v & 0xffffu);
         om = fma(nu, w.q[v & 0xffffu], om);
         zc = fma(nu, o[5 * R], zc);
         dw = fma(nu, o[6 * R], dw);
@@ -936,7 +970,7 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
     Qp = fma(w.hRT[k], om, Qp);
     if (k < d) f[1 + k] = sp[k] * om * s.inv_rho;
   }
-  const double Q = g.sum(Qp) * (kRu * s.T);
+  const S Q = g.sum(Qp) * (kRu * s.T);
   s.fT = -Q * s.inv_rho * s.inv_cp;
   if (g.t == 0) f[0] = s.fT;
   g.sync();
@@ -945,11 +979,10 @@ __device__ CellScalars cell_rates_fx(const DevMech& m, const Grp<G>& g, double p
 
 // The general form as a call (states outside the fixed-point range, rare in the solve): its code is
 // kept out of the kernels' loop, and its arguments are passed by value so that the caller's stay in registers.
-template <int G, bool kP>
-__device__ __noinline__ CellScalars cell_rates_wide(const DevMech& m, Grp<G> g, double p, const double* y, double* f,
-                                                    EvalMem<double> w, double* scr, bool jac, const double* vP,
-                                                    double* P) {
-  return cell_rates_any<G, double, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+template <int G, class S, bool kP>
+__device__ __noinline__ CellScalarsT<S> cell_rates_wide(const DevMech& m, Grp<G> g, double p, const S* y, S* f,
+                                                        EvalMem<S> w, S* scr, bool jac, const double* vP, S* P) {
+  return cell_rates_any<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
 }
 
 // f(y) and, with jac, the per-reaction derivative data (see cell_rates_any).
@@ -957,13 +990,9 @@ template <int G, class S, bool kP = false>
 __device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
                                                       const EvalMem<S>& w, S* scr, bool jac, const double* vP = nullptr,
                                                       S* P = nullptr) {
-  if constexpr (std::is_same<S, double>::value) {
-    const double T = y[0];
-    if (T > m.fx_T[0] && T < m.fx_T[1]) return cell_rates_fx<G, kP>(m, g, p, y, f, w, scr, jac, vP, P);
-    return cell_rates_wide<G, kP>(m, g, p, y, f, w, scr, jac, vP, P);
-  } else {
-    return cell_rates_any<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
-  }
+  const double T = val(y[0]);
+  if (T > m.fx_T[0] && T < m.fx_T[1]) return cell_rates_fx<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+  return cell_rates_wide<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
 }
 
 // Assemble the analytical Jacobian (Sec. 2.3) at the state of the preceding cell_rates(jac)
