@@ -201,37 +201,39 @@ struct Grp {
     sum2(a.v, a.d);
     sum2(b.v, b.d);
   }
-  // max that propagates NaN (a NaN error norm must reject the step)
-  __device__ static double nanmax(double a, double b) { return (a > b || a != a) ? a : b; }
+  // The larger magnitude, NaN if either is (a NaN error norm must reject the step): the bit patterns
+  // with the sign masked are ordered like the values, NaN above infinity, so no FP64 comparison (which
+  // takes the FP64 pipe for as long as an addition) is issued.
+  __device__ static unsigned long long mag(double a) {
+    return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffULL;
+  }
+  __device__ static double max_mag(double a, double b) { return __longlong_as_double((long long)max(mag(a), mag(b))); }
+  // the largest magnitude in the group
   __device__ double max_nan(double v) const {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = nanmax(v, __shfl_xor_sync(kFull, v, o));
-    if (G == 1) return v;
-    double* r = red + (parity & 1) * 3 * G;
-    parity++;
-    if (lane() == 0) r[warp()] = v;
-    sync();
-    double s = r[0];
-#pragma unroll
-    for (int i = 1; i < G; ++i) s = nanmax(s, r[i]);
-    return s;
+    bool none = false;
+    return max_nan_any(v, none);
   }
   // max_nan of v, and whether any thread of the group has flag set (one exchange)
   __device__ double max_nan_any(double v, bool& flag) const {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = nanmax(v, __shfl_xor_sync(kFull, v, o));
+    unsigned long long k = mag(v);
+    const unsigned hi = __reduce_max_sync(kFull, (unsigned)(k >> 32));
+    const unsigned lo = __reduce_max_sync(kFull, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+    k = (unsigned long long)hi << 32 | lo;
     flag = __any_sync(kFull, flag);
-    if (G == 1) return v;
+    if (G == 1) return __longlong_as_double((long long)k);
     double* r = red + (parity & 1) * 3 * G;
     parity++;
-    if (lane() == 0) { r[2 * warp()] = v; r[2 * warp() + 1] = flag ? 1.0 : 0.0; }
+    if (lane() == 0) { r[2 * warp()] = __longlong_as_double((long long)k); r[2 * warp() + 1] = flag ? 1.0 : 0.0; }
     sync();
-    double s = r[0];
-    bool f = r[1] != 0.0;
+    k = 0;
+    bool f = false;
 #pragma unroll
-    for (int i = 1; i < G; ++i) { s = nanmax(s, r[2 * i]); f = f || r[2 * i + 1] != 0.0; }
+    for (int i = 0; i < G; ++i) {
+      k = max(k, mag(r[2 * i]));
+      f = f || __double_as_longlong(r[2 * i + 1]) != 0;
+    }
     flag = f;
-    return s;
+    return __longlong_as_double((long long)k);
   }
   // argmax of key (ties to the lowest index) over the group, carrying a value along
   __device__ void argmax(long long& key, int& idx, double& val) const {
@@ -268,16 +270,17 @@ struct Grp {
 
 struct Plan {
   int N, K, R, n_pd, G;
-  int SA;  // size of each of the two matrix buffers: max(N*N, 8*R)
+  int SA;  // size of each of the two matrix buffers: max(N*N, 8*R), or 0
   int off_A, off_B, off_vec, off_sp, off_q, off_M, off_piv, off_red, off_bc, total;
 };
 
 __host__ __device__ inline int round2(int x) { return (x + 1) & ~1; }
 
-__host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G) {
+// matrices false: without the two matrix buffers (source terms only)
+__host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G, bool matrices = true) {
   Plan p;
   p.N = K; p.K = K; p.R = R; p.n_pd = n_pd; p.G = G;
-  p.SA = round2(max(K * K, 8 * R));
+  p.SA = matrices ? round2(max(K * K, 8 * R)) : 0;
   p.off_A = 0;
   p.off_B = p.SA;
   p.off_vec = 2 * p.SA;
@@ -800,7 +803,7 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   for (int k = g.t; k < K; k += NT) {
     const S Yk = (k < d) ? y[1 + k] : Yd;
     const S yiw = Yk * sp[K + k];
-    const double* a = sp + (size_t)(3 + (T <= sp[2 * K + k] ? 0 : kSpfRange)) * K + k;
+    const double* a = sp + (size_t)(3 + (__double_as_longlong(T) <= __double_as_longlong(sp[2 * K + k]) ? 0 : kSpfRange)) * K + k;
     auto c = [&](int i) { return a[(size_t)i * K]; };
     const double cpv = fma(T, fma(T, fma(T, fma(T, c(4), c(3)), c(2)), c(1)), c(0));
     const double hv = fma(T, fma(T, fma(T, fma(T, c(8), c(7)), c(6)), c(5)), fma(c(9), invT, c(0)));
@@ -990,8 +993,9 @@ template <int G, class S, bool kP = false>
 __device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Grp<G>& g, double p, const S* y, S* f,
                                                       const EvalMem<S>& w, S* scr, bool jac, const double* vP = nullptr,
                                                       S* P = nullptr) {
-  const double T = val(y[0]);
-  if (T > m.fx_T[0] && T < m.fx_T[1]) return cell_rates_fx<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
+  // (as bits: the limits are positive, and negative, zero and NaN patterns fall outside)
+  const long long T = __double_as_longlong(val(y[0]));
+  if (T > __double_as_longlong(m.fx_T[0]) && T < __double_as_longlong(m.fx_T[1])) return cell_rates_fx<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
   return cell_rates_wide<G, S, kP>(m, g, p, y, f, w, scr, jac, vP, P);
 }
 

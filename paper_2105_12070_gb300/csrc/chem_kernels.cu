@@ -30,10 +30,11 @@
 #include "integrate.h"
 
 namespace {
-// One-shot source term / Jacobian for chem_rates and chem_jacobian.
-template <int G>
-__global__ void __launch_bounds__(256, 1) rates_kernel(DevMech m, Plan plan, double p, const double* T, const double* Y,
-                                                    int64_t ncells, double* out_f, double* out_J) {
+// One-shot source term (kJac false) or Jacobian for chem_rates and chem_jacobian.  The source term needs
+// no matrix buffers: a 53-species cell takes 12 KB instead of 57, so two CTAs of 8 warps share an SM.
+template <int G, bool kJac>
+__global__ void __launch_bounds__(256, kJac ? 1 : 2) rates_kernel(DevMech m, Plan plan, double p, const double* T,
+                                                               const double* Y, int64_t ncells, double* out) {
   extern __shared__ double smem[];
   Grp<G> g;
   g.init(threadIdx.x % Grp<G>::NT, threadIdx.x / Grp<G>::NT);
@@ -46,15 +47,14 @@ __global__ void __launch_bounds__(256, 1) rates_kernel(DevMech m, Plan plan, dou
   for (int64_t cell = (int64_t)blockIdx.x * groups_per_cta + g.gid; cell < ncells; cell += ngroups) {
     for (int i = g.t; i < N; i += NT) w.y[i] = (i == 0) ? T[cell] : Y[(size_t)(i - 1) * ncells + cell];
     g.sync();
-    const bool jac = out_J != nullptr;
-    CellScalars s = cell_rates(m, g, p, w.y, w.f0, eval_mem(w), w.A, jac);
-    if (jac) {
+    CellScalars s = cell_rates(m, g, p, w.y, w.f0, eval_mem(w), kJac ? w.A : nullptr, kJac);
+    if (kJac) {
       cell_jacobian(m, g, s, w.f0, eval_mem(w), w.A, w.B);
-      double* o = out_J + (size_t)cell * N * N;
+      double* o = out + (size_t)cell * N * N;
       for (int e = g.t; e < N * N; e += NT) o[e] = -w.A[e];
+    } else {
+      for (int i = g.t; i < N; i += NT) out[(size_t)i * ncells + cell] = w.f0[i];
     }
-    if (out_f)
-      for (int i = g.t; i < N; i += NT) out_f[(size_t)i * ncells + cell] = w.f0[i];
     g.sync();
   }
 }
@@ -211,23 +211,23 @@ __global__ void exp_probe_kernel(const double* x, double* y, int64_t n) {
 
 namespace chemgpu {
 
-const void* integrate_kernel_fn(int G, int solver) {
+const void* integrate_kernel_fn(int G, int variant) {
   switch (G) {
-    case 1: return integrate_kernel_fn_g1(solver);
-    case 2: return integrate_kernel_fn_g2(solver);
-    case 4: return integrate_kernel_fn_g4(solver);
-    case 8: return integrate_kernel_fn_g8(solver);
+    case 1: return integrate_kernel_fn_g1(variant);
+    case 2: return integrate_kernel_fn_g2(variant);
+    case 4: return integrate_kernel_fn_g4(variant);
+    case 8: return integrate_kernel_fn_g8(variant);
     default: return nullptr;
   }
 }
 
-void integrate_launch(int G, int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+void integrate_launch(int G, int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                       const IntegrateArgs& a) {
   switch (G) {
-    case 1: integrate_launch_g1(solver, grid, threads, smem, st, d, a); break;
-    case 2: integrate_launch_g2(solver, grid, threads, smem, st, d, a); break;
-    case 4: integrate_launch_g4(solver, grid, threads, smem, st, d, a); break;
-    default: integrate_launch_g8(solver, grid, threads, smem, st, d, a); break;
+    case 1: integrate_launch_g1(variant, grid, threads, smem, st, d, a); break;
+    case 2: integrate_launch_g2(variant, grid, threads, smem, st, d, a); break;
+    case 4: integrate_launch_g4(variant, grid, threads, smem, st, d, a); break;
+    default: integrate_launch_g8(variant, grid, threads, smem, st, d, a); break;
   }
 }
 
@@ -355,8 +355,13 @@ int ensure_stage(chem_mech* m, size_t bytes) {
   return 0;
 }
 
+// Most warps a cell of an automatic launch shape gets when the call has few cells per SM
+#ifndef CHEM_FEW_CELLS_MAX_G
+#define CHEM_FEW_CELLS_MAX_G 8
+#endif
+
 struct Launch {
-  int G, cells_per_cta, grid, threads;
+  int G, variant, cells_per_cta, grid, threads;
   size_t smem;
   Plan plan;
 };
@@ -372,26 +377,43 @@ unsigned long long* phase_counters() {
 }
 #endif
 
-const void* integrate_fn(int G, int solver) { return integrate_kernel_fn(G, solver); }
-
+template <bool kJac>
 const void* rates_fn(int G) {
-  return G == 1 ? (const void*)rates_kernel<1>
-         : G == 2 ? (const void*)rates_kernel<2>
-         : G == 4 ? (const void*)rates_kernel<4>
-                  : (const void*)rates_kernel<8>;
+  return G == 1 ? (const void*)rates_kernel<1, kJac>
+         : G == 2 ? (const void*)rates_kernel<2, kJac>
+         : G == 4 ? (const void*)rates_kernel<4, kJac>
+                  : (const void*)rates_kernel<8, kJac>;
+}
+
+template <bool kJac>
+void launch_rates(const Launch& L, cudaStream_t st, const DevMech& d, double p, const double* T, const double* Y,
+                  int64_t ncells, double* out) {
+  switch (L.G) {
+    case 1: rates_kernel<1, kJac><<<L.grid, L.threads, L.smem, st>>>(d, L.plan, p, T, Y, ncells, out); break;
+    case 2: rates_kernel<2, kJac><<<L.grid, L.threads, L.smem, st>>>(d, L.plan, p, T, Y, ncells, out); break;
+    case 4: rates_kernel<4, kJac><<<L.grid, L.threads, L.smem, st>>>(d, L.plan, p, T, Y, ncells, out); break;
+    default: rates_kernel<8, kJac><<<L.grid, L.threads, L.smem, st>>>(d, L.plan, p, T, Y, ncells, out); break;
+  }
 }
 
 void launch_integrate(const Launch& L, cudaStream_t st, const DevMech& d, IntegrateArgs a) {
 #ifdef CHEM_PHASE_TIMERS
   a.phase = phase_counters();
 #endif
-  integrate_launch(L.G, a.solver, L.grid, L.threads, L.smem, st, d, a);
+  integrate_launch(L.G, L.variant, L.grid, L.threads, L.smem, st, d, a);
 }
+
+// The kernels of pick_launch: one of the integrate variants (integrate.h), or the one-shot ones.
+enum : int { kLaunchRates = 100, kLaunchJacobian = 101 };
 
 // Launch shape: G warps per cell, as many cells per CTA as the shared memory allows (at most 8
 // warps per CTA, 15 named barriers), one persistent CTA wave.
-int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, int want_ctas_per_sm, bool integ,
-                Launch& L, int solver = CHEM_SOLVER_ROSENBROCK) {
+int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, int want_ctas_per_sm, int variant,
+                Launch& L) {
+  const bool matrices = variant != kLaunchRates;
+  auto plan_for = [&](int G) { return make_plan(m->host.K, m->host.R, m->dev.n_pd, G, matrices); };
+  // cells per SM of a call that does not fill the device
+  const int64_t per_sm = (ncells + m->num_sms - 1) / m->num_sms;
   int G = want_G;
   if (G <= 0) {
     // automatic: about 8 warps per SM -- G = 8 / (cells that fit), a power of two in 1..8, and
@@ -402,21 +424,30 @@ int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, in
     while (G < 8 && G * fit < 8) G *= 2;
     if (m->host.K >= 32 && G < 2) G = 2;
     if (m->host.K < 32 && fit >= 8) G = 1;
+    // A call with few cells per SM gives each of them the warps that would stand idle.  Only where
+    // every thread of the group holds at most one species either way: the reductions then add the
+    // same numbers in the same order, so that a cell's result does not depend on its company.
+    if (32 * G >= m->host.K && m->host.R >= 64)
+      while (G < CHEM_FEW_CELLS_MAX_G && 2 * G * per_sm <= 8) G *= 2;
   }
   if (G != 1 && G != 2 && G != 4 && G != 8) return set_err(CHEM_EINVAL, "warps_per_cell must be 1, 2, 4 or 8");
   L.G = G;
-  L.plan = make_plan(m->host.K, m->host.R, m->dev.n_pd, G);
+  L.variant = variant;
+  L.plan = plan_for(G);
   const size_t per_cell = (size_t)L.plan.total * sizeof(double);
   int max_cpc = (int)std::min<size_t>(std::max(1, std::min(CHEM_MAX_THREADS_PER_CTA / 32 / G, 15)),
                                       m->max_smem / per_cell);
   if (max_cpc < 1)
     return set_err(CHEM_ESIZE, "mechanism working set (" + std::to_string(per_cell) +
                                    " B per cell) exceeds the shared memory of one CTA");
-  const int cpc = want_cpc > 0 ? std::min(want_cpc, max_cpc) : max_cpc;
+  // (automatic: no more cells per CTA than spread the call over all SMs)
+  const int cpc = want_cpc > 0 ? std::min(want_cpc, max_cpc) : (int)std::min<int64_t>(max_cpc, std::max<int64_t>(1, per_sm));
   L.cells_per_cta = cpc;
   L.threads = 32 * G * cpc;
   L.smem = per_cell * cpc;
-  const void* kernel = integ ? integrate_fn(G, solver) : rates_fn(G);
+  const void* kernel = variant == kLaunchRates      ? rates_fn<false>(G)
+                       : variant == kLaunchJacobian ? rates_fn<true>(G)
+                                                    : integrate_kernel_fn(G, variant);
   int occ = 0;
   CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, L.threads, L.smem));
@@ -437,7 +468,8 @@ int enqueue_integrate(chem_mech* m, const chem_opts& o, IntegrateArgs a, cudaStr
     a.first = first;
     a.count = std::min(batch, total - first);
     Launch L;
-    int rc = pick_launch(m, a.count, o.warps_per_cell, o.cells_per_cta, o.ctas_per_sm, true, L, a.solver);
+    int rc = pick_launch(m, a.count, o.warps_per_cell, o.cells_per_cta, o.ctas_per_sm,
+                         integrate_variant(a.solver, a.mixed != 0, a.fdjac != 0), L);
     if (rc) return rc;
     CK(cudaMemsetAsync(a.queue, 0, sizeof(int), st));
     launch_integrate(L, st, m->dev, a);
@@ -773,14 +805,10 @@ static int rates_or_jacobian(const chem_mech* mc, double p_Pa, const double* T, 
     dJ = J ? sJ : nullptr;
   }
   Launch L;
-  int rc = pick_launch(m, ncells, 0, 0, 0, false, L);
+  int rc = pick_launch(m, ncells, 0, 0, 0, dJ ? kLaunchJacobian : kLaunchRates, L);
   if (rc) return rc;
-  switch (L.G) {
-    case 1: rates_kernel<1><<<L.grid, L.threads, L.smem, st>>>(m->dev, L.plan, p_Pa * 10.0, dT, dY, ncells, df, dJ); break;
-    case 2: rates_kernel<2><<<L.grid, L.threads, L.smem, st>>>(m->dev, L.plan, p_Pa * 10.0, dT, dY, ncells, df, dJ); break;
-    case 4: rates_kernel<4><<<L.grid, L.threads, L.smem, st>>>(m->dev, L.plan, p_Pa * 10.0, dT, dY, ncells, df, dJ); break;
-    default: rates_kernel<8><<<L.grid, L.threads, L.smem, st>>>(m->dev, L.plan, p_Pa * 10.0, dT, dY, ncells, df, dJ); break;
-  }
+  if (dJ) launch_rates<true>(L, st, m->dev, p_Pa * 10.0, dT, dY, ncells, dJ);
+  else launch_rates<false>(L, st, m->dev, p_Pa * 10.0, dT, dY, ncells, df);
   CK(cudaGetLastError());
   if (!dev) {
     if (f) CK(cudaMemcpyAsync(f, df, sizeof(double) * N * ncells, cudaMemcpyDeviceToHost, st));
@@ -1160,7 +1188,8 @@ int chem_integrate_noalloc(const chem_mech* mc, double p_Pa, double* T, double* 
   unsigned char* s = static_cast<unsigned char*>(scratch);
   CK(cudaMemsetAsync(s, 0, kNoAllocCounters, st));  // queue counter and totals start at zero
   Launch L;
-  rc = pick_launch(m, ncells, o.warps_per_cell, o.cells_per_cta, o.ctas_per_sm, true, L, o.solver);
+  rc = pick_launch(m, ncells, o.warps_per_cell, o.cells_per_cta, o.ctas_per_sm,
+                   integrate_variant(o.solver, o.precision != CHEM_PREC_FP64, o.jacobian == CHEM_JAC_FD), L);
   if (rc) return rc;
   int32_t* d_steps = reinterpret_cast<int32_t*>(s + kNoAllocCounters);
   int32_t* d_rej = d_steps + kNoAllocMaxCells;

@@ -16,6 +16,11 @@
 
 namespace chemgpu {
 
+// Resident CTAs per SM the kernels are compiled for.  Groups of one warp serve small mechanisms, whose
+// cells take a few KB of shared memory: there the registers limit the warps per SM, and two CTAs of
+// 128 registers a thread hide more latency than one of 255.
+constexpr int integrate_min_ctas(int G) { return G == 1 ? 2 : 1; }
+
 // Arguments of one integrate launch (all pointers device memory).
 struct IntegrateArgs {
   double p, dt, rtol, atol;
@@ -40,27 +45,35 @@ struct IntegrateArgs {
   const double* p_cells;  // per-cell pressure in Pa (NULL: p for every cell)
   unsigned long long* phase;  // per-phase cycle counters (builds with CHEM_PHASE_TIMERS; else NULL)
 };
-// The integrate kernel of one group width (G = 1, 2, 4 or 8 warps per cell) and solver
-// (CHEM_SOLVER_*), for occupancy queries and attributes; NULL for another G.
-const void* integrate_kernel_fn(int G, int solver);
+// The kernels of one group width: the Rosenbrock solve with the analytical Jacobian and FP64 factors (the
+// default, and the only one that records), Seulex, and the Rosenbrock solve with every option
+// (low-precision factors, forward-difference Jacobian), whose code would cost the default registers.
+enum : int { kIntegrateFp64 = 0, kIntegrateSeulex = 1, kIntegrateOptions = 2 };
+inline int integrate_variant(int solver, bool mixed, bool fdjac) {
+  return solver != 0 ? kIntegrateSeulex : (mixed || fdjac) ? kIntegrateOptions : kIntegrateFp64;
+}
+
+// The integrate kernel of one group width (G = 1, 2, 4 or 8 warps per cell) and variant, for occupancy
+// queries and attributes; NULL for another G.
+const void* integrate_kernel_fn(int G, int variant);
 
 // Launches it: grid CTAs of `threads` threads with `smem` bytes of dynamic shared memory each,
 // the per-cell plan of make_plan(K, R, n_pd, G).
-void integrate_launch(int G, int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+void integrate_launch(int G, int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                       const IntegrateArgs& a);
 
 // One translation unit per G defines these.
-const void* integrate_kernel_fn_g1(int solver);
-const void* integrate_kernel_fn_g2(int solver);
-const void* integrate_kernel_fn_g4(int solver);
-const void* integrate_kernel_fn_g8(int solver);
-void integrate_launch_g1(int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+const void* integrate_kernel_fn_g1(int variant);
+const void* integrate_kernel_fn_g2(int variant);
+const void* integrate_kernel_fn_g4(int variant);
+const void* integrate_kernel_fn_g8(int variant);
+void integrate_launch_g1(int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                          const IntegrateArgs& a);
-void integrate_launch_g2(int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+void integrate_launch_g2(int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                          const IntegrateArgs& a);
-void integrate_launch_g4(int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+void integrate_launch_g4(int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                          const IntegrateArgs& a);
-void integrate_launch_g8(int solver, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
+void integrate_launch_g8(int variant, int grid, int threads, size_t smem, cudaStream_t st, const DevMech& d,
                          const IntegrateArgs& a);
 
 }  // namespace chemgpu

@@ -184,7 +184,7 @@ __device__ __forceinline__ bool stage_solve_low(const Grp<G>& g, const CellMem& 
     for (int i = g.t; i < N; i += NT) {
       const double d = w.res[i];
       u[i] += d;
-      c = Grp<G>::nanmax(c, fabs(d) * w.err[i]);  // w.err: 1 / (atol + rtol |y|), set per attempt
+      c = Grp<G>::max_mag(c, d * w.err[i]);  // w.err: 1 / (atol + rtol |y|), set per attempt
     }
     conv = g.max_nan_any(c, above);
     if (!above && conv == conv) conv = 0.0;  // residual at the FP64 rounding level
@@ -194,12 +194,14 @@ __device__ __forceinline__ bool stage_solve_low(const Grp<G>& g, const CellMem& 
 }
 
 // u <- W^-1 rhs: FP64 factors (lowp 0: one solve), FP32 factors (1) or FP32 pairs (2).
-template <int G>
+template <bool kAll, int G>
 __device__ __forceinline__ bool stage_solve(const Grp<G>& g, const CellMem& w, const IntegrateArgs& a, int N, double gh, int lowp,
                             double* u) {
   constexpr int NT = Grp<G>::NT;
-  if (lowp == 1) return stage_solve_low<G, float>(g, w, a, N, gh, u);
-  if (lowp == 2) return stage_solve_low<G, FF>(g, w, a, N, gh, u);
+  if constexpr (kAll) {
+    if (lowp == 1) return stage_solve_low<G, float>(g, w, a, N, gh, u);
+    if (lowp == 2) return stage_solve_low<G, FF>(g, w, a, N, gh, u);
+  }
   for (int i = g.t; i < N; i += NT) u[i] = w.rhs[i];
   g.sync();
   cell_solve(g, w.B, N, w.perm, w.invdiag, u);
@@ -223,8 +225,10 @@ __device__ inline int64_t next_cell(const IntegrateArgs& a, const Grp<G>& g, con
   return c < a.count ? a.first + c : -1;
 }
 
-template <int G>
-__global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(DevMech m, Plan plan, IntegrateArgs a) {
+// kAll: with the low-precision factors and the forward-difference Jacobian; without them the default's
+// code and registers are not shared with theirs.
+template <int G, bool kAll>
+__global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G)) integrate_kernel(DevMech m, Plan plan, IntegrateArgs a) {
   extern __shared__ double smem[];
   Grp<G> g;
   g.init(threadIdx.x % Grp<G>::NT, threadIdx.x / Grp<G>::NT);
@@ -264,7 +268,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
       if (h_next < 1e-14 * a.dt) { status = CHEM_CELL_H_UNDERFLOW; break; }
       PHASE_BEGIN
       if (need_jac) {
-        if (a.fdjac) {
+        if (kAll && a.fdjac) {
           cell_fd_jacobian(m, g, pc, w);
         } else {
           const CellScalars s0 = cell_rates(m, g, pc, w.y, w.f0, eval_mem(w), w.A, true);
@@ -281,8 +285,8 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
       const double invh = fx_rcp(h);
       double err = INFINITY;
       // after a fallback the next attempts go straight to FP64 factors for a while
-      for (int pass = (a.mixed && attempt >= f64_until) ? 0 : 1; pass < 2; ++pass) {
-        const int lowp = pass == 0 ? a.mixed : 0;
+      for (int pass = (kAll && a.mixed && attempt >= f64_until) ? 0 : 1; pass < 2; ++pass) {
+        const int lowp = (kAll && pass == 0) ? a.mixed : 0;
         bool ok;
         if (lowp) {
           // reciprocal error-control scales of the refinement's stopping test (the error vector is
@@ -306,7 +310,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
         // stage 1
         for (int i = g.t; i < N; i += NT) w.rhs[i] = w.f0[i];
         g.sync();
-        conv = stage_solve(g, w, a, N, gh, lowp, w.u[0]);
+        conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[0]);
         PHASE_END(3);
         // stage 2
         if (conv) {
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
           PHASE_END(4);
           for (int i = g.t; i < N; i += NT) w.rhs[i] = fma(c_c21 * invh, w.u[0][i], w.fs[i]);
           g.sync();
-          conv = stage_solve(g, w, a, N, gh, lowp, w.u[1]);
+          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[1]);
           PHASE_END(3);
         }
         // stage 3
@@ -328,14 +332,14 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
           for (int i = g.t; i < N; i += NT)
             w.rhs[i] = w.fs[i] + invh * (c_c31 * w.u[0][i] + c_c32 * w.u[1][i]);
           g.sync();
-          conv = stage_solve(g, w, a, N, gh, lowp, w.u[2]);
+          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[2]);
         }
         // stage 4 (same argument as stage 3)
         if (conv) {
           for (int i = g.t; i < N; i += NT)
             w.rhs[i] = w.fs[i] + invh * (c_c41 * w.u[0][i] + c_c42 * w.u[1][i] + c_c43 * w.u[2][i]);
           g.sync();
-          conv = stage_solve(g, w, a, N, gh, lowp, w.u[3]);
+          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[3]);
         }
         if (!conv) {
           if (g.t == 0) atomicAdd(&a.totals[3], 1ull);
@@ -363,8 +367,8 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) integrate_kernel(
         PHASE_END(3);
         double e = 0.0;
         for (int i = g.t; i < N; i += NT) {
-          const double sc = a.atol + a.rtol * fmax(fabs(w.y[i]), fabs(w.ynew[i]));
-          e = Grp<G>::nanmax(e, fabs(w.err[i] * gh) * fx_rcp(sc));
+          const double sc = fma(a.rtol, Grp<G>::max_mag(w.y[i], w.ynew[i]), a.atol);
+          e = Grp<G>::max_mag(e, w.err[i] * gh * fx_rcp(sc));
         }
         err = g.max_nan(e);
         break;
@@ -444,7 +448,7 @@ __device__ inline double seulex_work(int j) {
 }
 
 template <int G>
-__global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(DevMech m, Plan plan, IntegrateArgs a) {
+__global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G)) seulex_kernel(DevMech m, Plan plan, IntegrateArgs a) {
   extern __shared__ double smem[];
   Grp<G> g;
   g.init(threadIdx.x % Grp<G>::NT, threadIdx.x / Grp<G>::NT);
@@ -530,8 +534,8 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(Dev
           }
           tab(j)[i] = q;
           if (j >= 2) {
-            const double sc = a.atol + a.rtol * fmax(fabs(w.y[i]), fabs(q));
-            e = Grp<G>::nanmax(e, fabs(q - tab(j - 1)[i]) * fx_rcp(sc));
+            const double sc = fma(a.rtol, Grp<G>::max_mag(w.y[i], q), a.atol);
+            e = Grp<G>::max_mag(e, (q - tab(j - 1)[i]) * fx_rcp(sc));
           }
         }
         g.sync();
@@ -622,15 +626,19 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, 1) seulex_kernel(Dev
 // The launchers of integrate.h for one G (used once per integrate_g*.cu).
 #define CHEM_DEFINE_INTEGRATE_LAUNCHERS(G)                                                          \
   namespace chemgpu {                                                                              \
-  const void* integrate_kernel_fn_g##G(int solver) {                                               \
-    return solver == CHEM_SOLVER_SEULEX ? (const void*)seulex_kernel<G> : (const void*)integrate_kernel<G>; \
+  const void* integrate_kernel_fn_g##G(int variant) {                                              \
+    return variant == kIntegrateSeulex  ? (const void*)seulex_kernel<G>                             \
+           : variant == kIntegrateFp64 ? (const void*)integrate_kernel<G, false>                    \
+                                       : (const void*)integrate_kernel<G, true>;                    \
   }                                                                                                \
-  void integrate_launch_g##G(int solver, int grid, int threads, size_t smem, cudaStream_t st,      \
+  void integrate_launch_g##G(int variant, int grid, int threads, size_t smem, cudaStream_t st,     \
                              const DevMech& d, const IntegrateArgs& a) {                           \
     const Plan plan = make_plan(d.K, d.R, d.n_pd, G);                                              \
-    if (solver == CHEM_SOLVER_SEULEX)                                                              \
+    if (variant == kIntegrateSeulex)                                                               \
       seulex_kernel<G><<<grid, threads, smem, st>>>(d, plan, a);                                   \
+    else if (variant == kIntegrateFp64)                                                            \
+      integrate_kernel<G, false><<<grid, threads, smem, st>>>(d, plan, a);                         \
     else                                                                                           \
-      integrate_kernel<G><<<grid, threads, smem, st>>>(d, plan, a);                                \
+      integrate_kernel<G, true><<<grid, threads, smem, st>>>(d, plan, a);                          \
   }                                                                                                \
   }
