@@ -1504,11 +1504,22 @@ __device__ bool cell_lu(const Grp<G>& g, S* A, int N, int* piv, int* perm, S* in
   return ok;
 }
 
+// A pivot's reciprocal as it travels in the candidate record (as bits for FP32 and pairs).
+__device__ inline double lu_pack_recip(double a) { return fx_rcp(a); }
+__device__ inline double lu_pack_recip(float a) { return __hiloint2double(0, __float_as_int(1.0f / a)); }
+__device__ inline double lu_pack_recip(FF a) { return lu_carry(ff_recip(a)); }
+template <typename S>
+__device__ inline S lu_unpack(double c) {
+  if constexpr (std::is_same<S, double>::value) return c;
+  else if constexpr (std::is_same<S, float>::value) return __int_as_float(__double2loint(c));
+  else return FF(__int_as_float(__double2hiint(c)), __int_as_float(__double2loint(c)));
+}
+
 // The warp's pivot candidate: the lane with the largest key (0: no entry), ties to the lowest row, writes
-// (key, row, carried value) to out, integers as bits.  Two or three warp reductions (redux.sync) in
+// (key, row, reciprocal) to out, integers as bits.  Two or three warp reductions (redux.sync) in
 // place of five rounds of five shuffles.
 template <typename S>
-__device__ inline void warp_candidate(long long key, int row, double carried, int none, int lane, double* out) {
+__device__ inline void warp_candidate(long long key, int row, double inv, int none, int lane, double* out) {
   bool mine = true;
   if (std::is_same<S, double>::value) {
     const unsigned hi = (unsigned)((unsigned long long)key >> 32);
@@ -1522,7 +1533,7 @@ __device__ inline void warp_candidate(long long key, int row, double carried, in
   if (first == none ? lane == 0 : mine && row == first) {
     out[0] = __longlong_as_double(key);
     out[1] = __longlong_as_double(row);
-    out[2] = carried;
+    out[2] = inv;
   }
 }
 
@@ -1533,27 +1544,28 @@ __device__ inline void warp_candidate(long long key, int row, double carried, in
 //     an entry of column k+1 keeps the largest |a| it produced, the warps reduce by shuffles and
 //     leave one (key, row) each in the reduction scratch, and the barrier that ends the update
 //     also publishes them;
-//   * every thread then combines the G candidates itself (ties to the lowest row) and takes the
-//     pivot's reciprocal, so no thread waits for another to compute it;
+//   * the candidates' reciprocals are taken there too (integer and FP32 work beside the update's FP64),
+//     so that a column's pivot is known with its reciprocal when the update ends;
+//   * every thread then combines the G candidates itself (ties to the lowest row);
 //   * the row interchange (threads over columns) and the scaled multipliers of column k (threads
 //     over rows, reading the interchanged value for the pivot row) form one phase;
 //   * row k-1 of the unit upper factor is scaled during step k's update (no pass at the end).
 template <int G, typename S>
 __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm, S* invdiag) {
   constexpr int NT = Grp<G>::NT;
-  double* cand = g.red;  // [2 halves][G][3]: key bits, row and carried value of each warp's best entry
+  double* cand = g.red;  // [2 halves][G][3]: key bits, row and reciprocal of each warp's best entry
   bool ok = true;
   // pivot candidates of column 0
   {
     long long best = 0;
     int bi = N;
-    double bv = 0.0;
+    S bv = S(1.0f);
     for (int i = g.t; i < N; i += NT) {
       const S a = A[i * N];
       const long long v = abs_key(a) + 1;
-      if (v > best) { best = v; bi = i; bv = lu_carry(a); }
+      if (v > best) { best = v; bi = i; bv = a; }
     }
-    warp_candidate<S>(best, bi, bv, N, g.lane(), cand + 3 * g.warp());
+    warp_candidate<S>(best, bi, lu_pack_recip(bv), N, g.lane(), cand + 3 * g.warp());
   }
   g.sync();
   for (int k = 0; k < N; ++k) {
@@ -1578,7 +1590,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
         A[bi * N + j] = t;
       }
     if (k + 1 + 32 * g.warp() < N || g.t == 0) {  // this warp scales a row, or records the pivot
-      const S inv = lu_recip<S>(bv);
+      const S inv = lu_unpack<S>(bv);
       if (g.t == 0) {
         piv[k] = bi;
         invdiag[k] = inv;
@@ -1606,7 +1618,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
     const int mm = N - k - 1;
     long long nb = 0;
     int ni = N;
-    double nv = 0.0;
+    S nv = S(1.0f);
     if (mm > 0) {
       const S* Ak = A + (size_t)(k + 1) * N + k;  // multipliers of the trailing rows
       const S* U = A + (size_t)k * N + k + 1;     // pivot row right of the diagonal
@@ -1616,8 +1628,9 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
         const S r = fma(-Ak[i * N], u0, T0[i * N]);
         T0[i * N] = r;
         const long long v = abs_key(r) + 1;
-        if (v > nb) { nb = v; ni = k + 1 + i; nv = lu_carry(r); }
+        if (v > nb) { nb = v; ni = k + 1 + i; nv = r; }
       }
+      warp_candidate<S>(nb, ni, lu_pack_recip(nv), N, g.lane(), cand + ((k + 1) & 1) * 3 * G + 3 * g.warp());
       const int mc = mm - 1;  // columns k+2 .. N-1
       const int tot = mm * mc;
       if (tot > 0) {
@@ -1650,7 +1663,6 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
         }
       }
     }
-    if (k + 1 < N) warp_candidate<S>(nb, ni, nv, N, g.lane(), cand + ((k + 1) & 1) * 3 * G + 3 * g.warp());
     g.sync();
   }
   // compose the row interchanges: row i of the factors is row perm[i] of the original matrix
