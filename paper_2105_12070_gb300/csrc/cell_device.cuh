@@ -818,7 +818,9 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
       dcp = fma(yiw, dcpR, dcp);
       cp = fma(yiw, cpR, cp);
       w.cpR[k] = cpR;
-      w.hRT[k] = with_der<S>(hv, (cpv - hv) * invT * Td);
+      const S h = with_der<S>(hv, (cpv - hv) * invT * Td);
+      w.hRT[k] = h;
+      w.dcpR[k] = (h - 1.0) * s.invT;  // the species' term of d ln Kc / dT
     } else {
       cp = fma(yiw, cst<S>(cpv), cp);
       w.cpR[k] = cst<S>(cpv);
@@ -864,14 +866,13 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
     if (two_r) Xc -= (uint64_t)g2[a1];
     if (dnu != 0) Xc = dnu > 0 ? Xc - (uint64_t)P2 : Xc + (uint64_t)P2;
     const bool pd = r < npd, fo = r < nfo;
-    // d ln k_inf / dT, the reaction enthalpy over RT and d ln Kc / dT
-    S dlnk = cst<S>(0.0), dH = cst<S>(0.0), dlnKc_dT = cst<S>(0.0), dlnk0 = cst<S>(0.0);
+    // d ln k_inf / dT and d ln Kc / dT = sum nu (h/RT - 1) / T
+    S dlnk = cst<S>(0.0), dlnKc_dT = cst<S>(0.0), dlnk0 = cst<S>(0.0);
     if (kDual || jac) {
       dlnk = fma(m.rxd_t[R + r], s.invT, m.rxd_t[r]) * s.invT;
-      dH = w.hRT[p0] - w.hRT[a0];
-      if (two_p) dH += w.hRT[p1];
-      if (two_r) dH -= w.hRT[a1];
-      dlnKc_dT = (dnu == 0 ? dH : dH - (dnu > 0 ? 1.0 : -1.0)) * s.invT;
+      dlnKc_dT = w.dcpR[p0] - w.dcpR[a0];
+      if (two_p) dlnKc_dT += w.dcpR[p1];
+      if (two_r) dlnKc_dT -= w.dcpR[a1];
       if (fo) dlnk0 = fma(m.fo[(size_t)r * kFoDoubles + 2], s.invT, m.fo[(size_t)r * kFoDoubles + 1]) * s.invT;
     }
     S kf = exp2_of_fx<S>(Xf, val(dlnk) * Td), kr;
@@ -927,9 +928,10 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
       o[2 * R] = -(kr * Cp1);
       o[3 * R] = -(kr * Cp0);
       // R_f and R_r are homogeneous in the concentrations of their side's slots
-      o[5 * R] = DC + ((two_r ? Rf + Rf : Rf) - (two_p ? Rr + Rr : Rr));
+      o[5 * R] = fma(two_p ? -2.0 : -1.0, Rr, fma(two_r ? 2.0 : 1.0, Rf, DC));
       o[6 * R] = fma(q, dlnk, Rr * dlnKc_dT);
       if (kP) {
+        const S dH = fma(dlnKc_dT, s.T, (double)dnu);  // reaction enthalpy / RT
         const int* ii = m.rxi + r * kRxInts;
         const double* rd = m.rxd + r * kRxDoubles;
         double gw = 0.0;  // sum over the species rows of nu_kr W_k v_Yk
@@ -1018,22 +1020,31 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
   // entry e, for the entries that have it, at zgb[c] + e.  Each thread takes four entries at once, NT
   // apart (independent FMA chains); every entry sums its contributions in plan order, and the
   // entries without any, at the end, become zero.
+  // Four contributions of each are read at once (zgb ends in four equal values), the next four's list
+  // starts beside them: the loads of a long list would otherwise follow one another at L2 latency.
   const int entries = d * K;
   for (int e0 = g.t; e0 < entries; e0 += 4 * NT) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    int b = m.zgb[0];
-    for (int c = 0;; ++c) {
-      const int nb = m.zgb[c + 1], have = nb - b;
-      if (e0 >= have) break;
+    int b[5];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int e = e0 + q * NT;
-        if (e < have) {
-          const uint32_t v = m.zgx[b + e];
-          acc[q] = fma(__hiloint2double((int)(v & 0xffff0000u), 0), scr[v & 0xffffu], acc[q]);
-        }
-      }
-      b = nb;
+    for (int i = 0; i < 5; ++i) b[i] = m.zgb[i];
+    for (int c = 0; e0 < b[1] - b[0]; c += 4) {
+      int nx[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) nx[i] = m.zgb[c + 5 + i];
+      uint32_t v[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[i][q] = e0 + q * NT < b[i + 1] - b[i] ? m.zgx[b[i] + e0 + q * NT] : 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (v[i][q]) acc[q] = fma(__hiloint2double((int)(v[i][q] & 0xffff0000u), 0), scr[v[i][q] & 0xffffu], acc[q]);
+      b[0] = b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) b[i + 1] = nx[i];
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)

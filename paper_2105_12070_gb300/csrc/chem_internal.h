@@ -72,7 +72,7 @@ struct HostMech {
   // zgx[zgb[c] + e]: src in the low half, the top 16 bits of the coefficient (a small integer) as a
   // double in the high half.
   std::vector<int> zg_dst;             // [(K-1) K] row * K + col
-  std::vector<int> zgb;                // [longest list + 2], the last two equal
+  std::vector<int> zgb;                // [longest list + 12], the last twelve equal
   std::vector<uint32_t> zgx;           // [contributions]
   std::vector<double> mwr;             // [K-1][K-1] -W_k / W_i
   // Efficiency part: for each species row k < K-1, the pressure-dependent reactions in it:

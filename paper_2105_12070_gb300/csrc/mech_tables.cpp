@@ -250,7 +250,7 @@ void build_jacobian_plan(HostMech& m) {
     }
     m.zgb.push_back((int)m.zgx.size());
   }
-  m.zgb.push_back((int)m.zgx.size());
+  for (int i = 0; i < 11; ++i) m.zgb.push_back((int)m.zgx.size());  // (the kernel reads them ahead)
   m.mwr.assign((size_t)d * d, 0.0);
   for (int k = 0; k < d; ++k)
     for (int i = 0; i < d; ++i)
