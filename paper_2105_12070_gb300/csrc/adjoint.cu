@@ -47,9 +47,9 @@ AdjPlan make_adj_plan(int K, int R, int n_pd, int n_pairs, int G) {
   p.nM2 = round2(std::max(n_pd, 1));
   p.nP2 = round2(std::max(n_pairs, 1));
   p.nAB2 = round2(2 * R + 2 * n_pd);
-  // matrix region, reused by the phases of a step: the Jacobian at y_n (scratch, then -J, then
-  // W and its LU in place) with its Z scratch behind it; the LU with the per-reaction scratch of
-  // the stage-state evaluations behind it; the dual-number per-reaction scratch
+  // matrix region, reused by the phases of a step: the Jacobian at y_n (-J, then W and its LU in
+  // place) with the per-reaction scratch of the evaluations behind it; the dual-number per-reaction
+  // scratch
   p.off_M = 0;
   const int msize = round2(std::max({p.SA + K * K, K * K + 8 * R, 16 * R}));
   // 18 vectors: y f ys rhs u0..u3 ub0..ub3 (v_i overwrite ub_i) ybar lam invdiag wv (+2 spare)
@@ -112,8 +112,17 @@ __device__ inline EvalMem<S> adj_eval_mem(double* base, const AdjPlan& p) {
   m.zc = e + 6 * n; m.dwT = e + 7 * n; m.rowA = e + 8 * n; m.rowB = e + 9 * n; m.ccol = e + 10 * n; m.wq = e + 11 * n;
   m.q = e + 12 * n;
   m.M = m.q + p.nR2;
+  m.DC = m.dqdT = nullptr;  // set with the scratch (with_scratch)
   m.pv = m.M + p.nM2;
   return m;
+}
+
+// The evaluation arrays with the last two per-reaction rows behind the five of the scratch.
+template <class S>
+__device__ inline EvalMem<S> with_scratch(EvalMem<S> e, S* scr, int R) {
+  e.DC = scr + 5 * R;
+  e.dqdT = scr + 6 * R;
+  return e;
 }
 
 template <int G>
@@ -125,17 +134,18 @@ __device__ inline void solve_t(const Grp<G>& g, const AdjMem& w, int N, double* 
 // w.lam and the step's ln A terms added to w.gA on exit.  False if W is exactly singular.
 template <int G>
 __device__ bool adjoint_step(const DevMech& m, const Grp<G>& g, const AdjPlan& plan, double p, double h,
-                             const AdjMem& w, const EvalMem<double>& ed, const EvalMem<Dual>& eD, double* abd,
+                             const AdjMem& w, const EvalMem<double>& ed0, const EvalMem<Dual>& eD0, double* abd,
                              Dual* abD, double* tzd, Dual* tzD, double* Pd, Dual* PD) {
   constexpr int NT = Grp<G>::NT;
   const int N = m.N, R = m.R;
   const double gh = 1.0 / (c_gamma * h);
   const double invh = 1.0 / h;
   double* LU = w.M;            // -J(y_n), then W, then its factors
-  double* scr = w.M + N * N;   // per-reaction scratch of the stage-state evaluations
+  double* scr = w.M + N * N;   // per-reaction scratch of the evaluations beside it
+  const EvalMem<double> ed = with_scratch(ed0, scr, R);
   // J(y) and the factors of W (as in the solve)
-  const CellScalars s0 = cell_rates(m, g, p, w.y, w.f, ed, LU, true);
-  cell_jacobian(m, g, s0, w.f, ed, LU, w.M + plan.SA);
+  const CellScalars s0 = cell_rates(m, g, p, w.y, w.f, ed, scr, true);
+  cell_jacobian(m, g, s0, w.f, ed, LU, scr);
   for (int i = g.t; i < N; i += NT) LU[i * N + i] += gh;
   g.sync();
   if (!cell_lu_default<G, double>(g, LU, N, w.piv, w.perm, w.invdiag)) return false;
@@ -213,6 +223,7 @@ __device__ bool adjoint_step(const DevMech& m, const Grp<G>& g, const AdjPlan& p
   // parts are the terms of W's dependence on y; the value part of the first pass is
   // J(y)^T v_1 and v_1 . df/dlnA(y), the stage-1 terms
   Dual* scrD = reinterpret_cast<Dual*>(w.M);
+  const EvalMem<Dual> eD = with_scratch(eD0, scrD, R);
   for (int k = 0; k < 4; ++k) {
     const double* uk = w.u[0] + k * w.n2;
     const double* vk = w.v[0] + k * w.n2;

@@ -270,26 +270,39 @@ struct Grp {
 
 struct Plan {
   int N, K, R, n_pd, G;
-  int SA;  // size of each of the two matrix buffers: max(N*N, 8*R), or 0
-  int off_A, off_B, off_vec, off_sp, off_q, off_M, off_piv, off_red, off_bc, total;
+  int SA;  // size of a matrix buffer
+  int off_A, off_B, off_scr, off_vec, off_sp, off_q, off_M, off_piv, off_red, off_bc, total;
 };
 
 __host__ __device__ inline int round2(int x) { return (x + 1) & ~1; }
 
-// matrices false: without the two matrix buffers (source terms only)
-__host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G, bool matrices = true) {
+// What a cell's plan holds beside its vectors:
+//   kPlanFull     two matrix buffers: the Jacobian stays beside the iteration matrix (several factorisations
+//                 or refinement residuals per Jacobian); the second is the per-reaction scratch of the
+//                 assembly first;
+//   kPlanCompact  one, which the Jacobian, the iteration matrix and its factors use in turn, and the
+//                 scratch apart: 43 KB per cell of 53 species in place of 57, so that five share an SM
+//                 instead of four;
+//   kPlanRates    none (source terms only).
+enum : int { kPlanFull = 0, kPlanCompact = 1, kPlanRates = 2 };
+
+__host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G, int kind = kPlanFull) {
   Plan p;
   p.N = K; p.K = K; p.R = R; p.n_pd = n_pd; p.G = G;
-  p.SA = matrices ? round2(max(K * K, 8 * R)) : 0;
+  // (the assembly keeps three rows of per-reaction data in the Jacobian's buffer and four in the scratch)
+  p.SA = kind == kPlanFull ? round2(max(K * K, 8 * R)) : kind == kPlanCompact ? round2(max(K * K, 3 * R)) : 0;
   p.off_A = 0;
-  p.off_B = p.SA;
-  p.off_vec = 2 * p.SA;
-  // vectors: y, ynew, f0, fs, u0..u3, err, invdiag, rhs, res, (er, ec as ints), (FP32 inverse
-  // pivots)  (14 x N); the Jacobian's temporaries zc, dwT, rowA, rowB, ccol reuse ynew, fs, u2, u3, err
-  p.off_sp = p.off_vec + 14 * round2(K);
+  p.off_B = kind == kPlanFull ? p.SA : 0;
+  p.off_scr = p.SA;
+  p.off_vec = kind == kPlanFull ? 2 * p.SA : kind == kPlanCompact ? p.SA + round2(4 * R + max(n_pd, 1)) : 0;
+  // vectors: y, ynew, f0, fs, u0..u3, err, invdiag, rhs, res, and with low-precision factors and Seulex (er, ec as
+  // ints), (FP32 inverse pivots): 12 or 14 x N; the Jacobian's temporaries zc, dwT, rowA, rowB, ccol
+  // reuse ynew, fs, u2, u3, err
+  p.off_sp = p.off_vec + (kind == kPlanCompact ? 12 : 14) * round2(K);
   // species: C, hRT, cpR, gRT, omega, dcpR  (6 x K)
-  p.off_q = p.off_sp + 6 * round2(K);
-  p.off_M = p.off_q + round2(R);
+  // net rates of progress: the compact plan keeps a stage evaluation's in the scratch
+  p.off_q = kind == kPlanCompact ? p.off_scr : p.off_sp + 6 * round2(K);
+  p.off_M = p.off_sp + 6 * round2(K) + (kind == kPlanCompact ? 0 : round2(R));
   p.off_piv = p.off_M + round2(max(n_pd, 1));
   p.off_red = p.off_piv + round2(K + 2);  // pivots and the composed permutation (ints)
   p.off_bc = p.off_red + 6 * G + 2;  // reduction scratch + queue slot
@@ -298,7 +311,7 @@ __host__ __device__ inline Plan make_plan(int K, int R, int n_pd, int G, bool ma
 }
 
 struct CellMem {
-  double *A, *B;
+  double *A, *B, *scr;
   double *y, *ynew, *f0, *fs, *u[4], *err, *invdiag, *zc, *dwT, *rowA, *rowB, *ccol, *rhs, *res;
   int *er, *ec;
   float* invd32;
@@ -313,6 +326,7 @@ __device__ inline CellMem carve(double* base, const Plan& p) {
   CellMem w;
   w.A = base + p.off_A;
   w.B = base + p.off_B;
+  w.scr = base + p.off_scr;
   const int n = round2(p.K);
   double* v = base + p.off_vec;
   w.y = v; w.ynew = v + n; w.f0 = v + 2 * n; w.fs = v + 3 * n;
@@ -341,6 +355,7 @@ template <class S>
 struct EvalMem {
   S *C, *hRT, *cpR, *gRT, *omega, *dcpR;  // species [K]
   S *q, *M;                               // net rates [R]; [M] of the pressure-dependent [n_pd]
+  S *DC, *dqdT;                           // with derivatives: sum_j dq/dC_j C_j and dq/dT [R]
   S *zc, *dwT, *rowA, *rowB, *ccol, *wq;  // Jacobian temporaries [K]
   S* pv;                                  // efficiency-pair coefficients [n_pairs]
   S* bc = nullptr;                        // broadcast slot of the cell scalars [5] (or none)
@@ -349,10 +364,14 @@ struct EvalMem {
 // The solve's evaluation arrays: the Jacobian temporaries reuse the stage vectors, which are
 // free while the Jacobian is built (pv spans u0 .. res, n_pairs <= 8 round2(K); zc and dwT, which the
 // rate evaluation writes before pv is used, lie outside it).
-__device__ inline EvalMem<double> eval_mem(const CellMem& w) {
+// With derivatives the per-reaction rows that the rate evaluation itself consumes lie in the
+// Jacobian's buffer, which is free until the assembly.
+__device__ inline EvalMem<double> eval_mem(const CellMem& w, int R = 0, bool jac = false) {
   EvalMem<double> e;
   e.C = w.C; e.hRT = w.hRT; e.cpR = w.cpR; e.gRT = w.gRT; e.omega = w.omega; e.dcpR = w.dcpR;
-  e.q = w.q; e.M = w.M;
+  e.q = jac ? w.A : w.q; e.M = w.M;
+  e.DC = w.A + R;
+  e.dqdT = w.A + 2 * R;
   e.zc = w.zc; e.dwT = w.dwT; e.rowA = w.rowA; e.rowB = w.rowB; e.ccol = w.ccol; e.wq = w.res;
   e.pv = w.u[0];
   e.bc = w.bc;
@@ -534,11 +553,10 @@ __device__ inline void troe_fx(const double* fd, int n, S T, S invT, S Pr, S& F,
 }
 
 // Evaluates f(y) into f[0..N).  With jac, also leaves per-reaction derivative data in
-// scr[u * R + r], u = 0..6: {dq/dC through each of the 4 slots (an empty slot's entry is not read),
-// phi (coefficient of the efficiencies; pressure-dependent reactions only), sum_j dq/dC_j C_j,
-// dq/dT at fixed C} (rows of R, so that the threads of consecutive reactions store to consecutive
-// words), the species production rates in w.omega and the species' sums of the last two rows in w.zc
-// and w.dwT.
+// scr[u * R + r], u = 0..4: {dq/dC through each of the 4 slots (an empty slot's entry is not read),
+// phi (coefficient of the efficiencies; pressure-dependent reactions only)} (rows of R, so that the
+// threads of consecutive reactions store to consecutive words), the species production rates in
+// w.omega and the species' sums of sum_j dq/dC_j C_j and of dq/dT at fixed C in w.zc and w.dwT.
 // With kP (adjoint use, requires jac) it also writes P[r] = v . d f / d ln A_r for the weight
 // vector v = vP (N): with q'_r = d q_r / d ln A_r (q_r for elementary and third-body
 // reactions; q_r (Pr/(1+Pr) - d ln F/d ln Pr) for fall-off reactions, whose A is that of
@@ -701,8 +719,8 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
       o[2 * R] = -krm * Cp1;
       o[3 * R] = -krm * Cp0;
       o[4 * R] = phi;
-      o[5 * R] = fma(phi, Mr, ((a1 >= 0) ? Rf + Rf : Rf) - ((p1 >= 0) ? Rr + Rr : Rr));
-      o[6 * R] = dqdT;
+      w.DC[r] = fma(phi, Mr, ((a1 >= 0) ? Rf + Rf : Rf) - ((p1 >= 0) ? Rr + Rr : Rr));
+      w.dqdT[r] = dqdT;
       if (kP) {
         double gw = 0.0;  // sum over the species rows of nu_kr W_k v_Yk
 #pragma unroll
@@ -738,8 +756,8 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
       for (e = eb; e < ee; ++e) {
         const double nu = m.sr_nu[e];
         const int r = m.sr_idx[e];
-        zc = fma(nu, scr[5 * m.R + r], zc);
-        dw = fma(nu, scr[6 * m.R + r], dw);
+        zc = fma(nu, w.DC[r], zc);
+        dw = fma(nu, w.dqdT[r], dw);
       }
       w.zc[k] = zc;
       w.dwT[k] = dw;
@@ -928,8 +946,8 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
       o[2 * R] = -(kr * Cp1);
       o[3 * R] = -(kr * Cp0);
       // R_f and R_r are homogeneous in the concentrations of their side's slots
-      o[5 * R] = fma(two_p ? -2.0 : -1.0, Rr, fma(two_r ? 2.0 : 1.0, Rf, DC));
-      o[6 * R] = fma(q, dlnk, Rr * dlnKc_dT);
+      w.DC[r] = fma(two_p ? -2.0 : -1.0, Rr, fma(two_r ? 2.0 : 1.0, Rf, DC));
+      w.dqdT[r] = fma(q, dlnk, Rr * dlnKc_dT);
       if (kP) {
         const S dH = fma(dlnKc_dT, s.T, (double)dnu);  // reaction enthalpy / RT
         const int* ii = m.rxi + r * kRxInts;
@@ -958,10 +976,10 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
       for (int i = 0; i < len; ++i) {
         const uint32_t v = e[(size_t)i * K];
         const double nu = __hiloint2double((int)(v & 0xffff0000u), 0);
-        const S* o = scr + (v & 0xffffu);
-        om = fma(nu, w.q[v & 0xffffu], om);
-        zc = fma(nu, o[5 * R], zc);
-        dw = fma(nu, o[6 * R], dw);
+        const int r = v & 0xffffu;
+        om = fma(nu, w.q[r], om);
+        zc = fma(nu, w.DC[r], zc);
+        dw = fma(nu, w.dqdT[r], dw);
       }
       w.zc[k] = zc;
       w.dwT[k] = dw;
@@ -1002,18 +1020,18 @@ __device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Gr
 }
 
 // Assemble the analytical Jacobian (Sec. 2.3) at the state of the preceding cell_rates(jac)
-// call.  J (overwritten) holds the per-reaction data on entry, Z is N*N scratch, J receives
-// -d f / d phi (stored negated, so that W = I/(gamma h) - J is a copy plus the diagonal).  Chain rule
-// through C_j = rho Y_j / W_j, rho = p Wbar/(Ru T), Y_K = 1 - sum Y_i;
-// Z rows k < K-1 hold d omega_k / dC, row K-1 holds d Q / dC (Q = sum_k H_k omega_k).
+// call, from its per-reaction data in scr.  J receives -d f / d phi (stored negated, so that
+// W = I/(gamma h) - J is its copy plus the diagonal).  Chain rule through C_j = rho Y_j / W_j,
+// rho = p Wbar/(Ru T), Y_K = 1 - sum Y_i, in place on Z: rows k < K-1 hold d omega_k / dC, row K-1
+// d Q / dC (Q = sum_k H_k omega_k).  Z's entry (k, j) is kept at row k + 1 and column j + 1, both modulo K,
+// where the entry of J made from it belongs; Z's last row and column become J's temperature row and column.
 // Bound by FP64 issue; the plans are read as packed 4-byte words in the threads' order (8 KB of the
 // SM's L1 is left beside the cells' shared memory for 53 species, so their volume counts).
 template <int G>
 __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScalars& s, const double* f,
-                              const EvalMem<double>& w, double* J, double* Z) {
+                              const EvalMem<double>& w, double* J, const double* scr) {
   constexpr int NT = Grp<G>::NT;
   const int K = m.K, N = K, d = K - 1;
-  const double* scr = J;
   // mass-action part: one thread per entry of the species rows sums its contributions (a fixed plan
   // built with the mechanism; no two threads write the same entry, no atomics).  The entries are in
   // order of decreasing list length and the plan is stored contribution by contribution: the c-th one of
@@ -1048,7 +1066,7 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (e0 + q * NT < entries) Z[m.zg_dst[e0 + q * NT]] = acc[q];
+      if (e0 + q * NT < entries) J[m.zg_dst[e0 + q * NT]] = acc[q];
   }
   // efficiency part of the pressure-dependent reactions: Z[k][j] += sum_r v_kr eff_rj over the
   // (row k, reaction r) pairs, v_kr = nu_kr phi_r.  The coefficients go to the stage-vector area
@@ -1072,11 +1090,11 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
         const int ri = ok ? (int)(((float)x + 0.5f) * invK) : 0;
         jj[q] = ok ? x - ri * K : 0;
         const int row = m.pr_rows[ri];
-        zi[q] = row * N + jj[q];
+        zi[q] = (row + 1) * N + (jj[q] < d ? jj[q] + 1 : 0);
         cb[q] = m.pr_ptr[row];
         len[q] = ok ? m.pr_ptr[row + 1] - cb[q] : 0;
         lmax = max(lmax, len[q]);
-        acc[q] = Z[zi[q]];
+        acc[q] = J[zi[q]];
       }
       for (int c = 0; c < lmax; ++c) {
 #pragma unroll
@@ -1085,7 +1103,7 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (x0 + q * NT < items) Z[zi[q]] = acc[q];
+        if (x0 + q * NT < items) J[zi[q]] = acc[q];
     }
   }
   g.sync();
@@ -1102,25 +1120,27 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
     for (int k = g.t; k < d; k += NT) {
       const double Wk = sp[k];
       wq[k] = RuT * fma(-hd, Wk, w.hRT[k]);
-      w.rowA[k] = Wk * invWd * Z[k * N + d];
+      w.rowA[k] = Wk * invWd * J[(k + 1) * N];
       w.rowB[k] = Wk * s.inv_rho * (w.zc[k] - w.omega[k]);
       w.ccol[k] = -s.Wbar * (sp[K + k] - invWd);
     }
   }
   g.sync();
-  // enthalpy row Z_Q[j] = sum_k wq_k Z[k][j] (stored in row K-1), with sum_j Z_Q[j] C_j and the part
+  // enthalpy row Z_Q[j] = sum_k wq_k Z[k][j] (its last entry also in zc[K-1]), with sum_j Z_Q[j] C_j and the part
   // of dQ/dT that is not in it: sum_k wq_k dw_k/dT|_C + Ru sum_j cp_j omega_j
   double zqc = 0.0, dqt = 0.0;
   for (int j = g.t; j < K; j += NT) {
+    const double* Zj = J + (j < d ? j + 1 : 0);
     double a0 = 0.0, a1 = 0.0;
     int k = 0;
     for (; k + 1 < d; k += 2) {
-      a0 = fma(wq[k], Z[k * N + j], a0);
-      a1 = fma(wq[k + 1], Z[(k + 1) * N + j], a1);
+      a0 = fma(wq[k], Zj[(k + 1) * N], a0);
+      a1 = fma(wq[k + 1], Zj[(k + 2) * N], a1);
     }
-    if (k < d) a0 = fma(wq[k], Z[k * N + j], a0);
+    if (k < d) a0 = fma(wq[k], Zj[(k + 1) * N], a0);
     const double zq = a0 + a1;
-    Z[d * N + j] = zq;
+    if (j < d) J[j + 1] = zq;
+    else w.zc[d] = zq;
     zqc = fma(zq, w.C[j], zqc);
     dqt = fma(kRu * w.cpR[j], w.omega[j], dqt);
     if (j < d) dqt = fma(wq[j], w.dwT[j], dqt);
@@ -1130,14 +1150,14 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
   const double inv_cp = s.inv_cp;
   const double inv_rhocp = s.inv_rho * inv_cp;
   const double fT = s.fT;
-  // temperature row and column, then the species block (J now overwrites the scratch)
-  const double ZQd = Z[d * N + d] * invWd;
+  // temperature row and column, then the species block
+  const double ZQd = w.zc[d] * invWd;
   const double cpd = w.cpR[d] * invWd;
   const double RuCp = kRu * inv_cp;
   for (int i = g.t; i < d; i += NT) {
     const double ci = w.ccol[i];
     const double invWi = sp[K + i];
-    const double dQdY = fma(s.rho, fma(invWi, Z[d * N + i], -ZQd), zqc * ci);
+    const double dQdY = fma(s.rho, fma(invWi, J[1 + i], -ZQd), zqc * ci);
     const double dcpdY = fma(w.cpR[i], invWi, -cpd);
     J[1 + i] = fma(dQdY, inv_rhocp, fT * fma(dcpdY, RuCp, ci));
     const double Wr = sp[i] * s.inv_rho;
@@ -1156,7 +1176,7 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       at[q] = (1 + k) * N + 1 + i;
-      j[q] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e + q * NT], Z[k * N + i], w.rowA[k]));
+      j[q] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e + q * NT], J[at[q]], w.rowA[k]));
       k += dk;
       i += di;
       if (i >= d) { i -= d; ++k; }
@@ -1165,7 +1185,8 @@ __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScala
     for (int q = 0; q < 4; ++q) J[at[q]] = j[q];
   }
   for (; e < nb; e += NT) {
-    J[(1 + k) * N + 1 + i] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e], Z[k * N + i], w.rowA[k]));
+    const int at = (1 + k) * N + 1 + i;
+    J[at] = fma(-w.rowB[k], w.ccol[i], fma(m.mwr[e], J[at], w.rowA[k]));
     k += dk;
     i += di;
     if (i >= d) { i -= d; ++k; }

@@ -71,7 +71,7 @@ struct HostMech {
   // order of decreasing list length; the c-th contribution of entry e, where it has one, is at
   // zgx[zgb[c] + e]: src in the low half, the top 16 bits of the coefficient (a small integer) as a
   // double in the high half.
-  std::vector<int> zg_dst;             // [(K-1) K] row * K + col
+  std::vector<int> zg_dst;             // [(K-1) K] ((row + 1) mod K) * K + (col + 1) mod K
   std::vector<int> zgb;                // [longest list + 12], the last twelve equal
   std::vector<uint32_t> zgx;           // [contributions]
   std::vector<double> mwr;             // [K-1][K-1] -W_k / W_i

@@ -33,7 +33,7 @@ namespace {
 // One-shot source term (kJac false) or Jacobian for chem_rates and chem_jacobian.  The source term needs
 // no matrix buffers: a 53-species cell takes 12 KB instead of 57, so two CTAs of 8 warps share an SM.
 template <int G, bool kJac>
-__global__ void __launch_bounds__(256, kJac ? 1 : 2) rates_kernel(DevMech m, Plan plan, double p, const double* T,
+__global__ void __launch_bounds__(kJac && G == 2 ? 320 : 256, kJac ? 1 : 2) rates_kernel(DevMech m, Plan plan, double p, const double* T,
                                                                const double* Y, int64_t ncells, double* out) {
   extern __shared__ double smem[];
   Grp<G> g;
@@ -47,9 +47,9 @@ __global__ void __launch_bounds__(256, kJac ? 1 : 2) rates_kernel(DevMech m, Pla
   for (int64_t cell = (int64_t)blockIdx.x * groups_per_cta + g.gid; cell < ncells; cell += ngroups) {
     for (int i = g.t; i < N; i += NT) w.y[i] = (i == 0) ? T[cell] : Y[(size_t)(i - 1) * ncells + cell];
     g.sync();
-    CellScalars s = cell_rates(m, g, p, w.y, w.f0, eval_mem(w), kJac ? w.A : nullptr, kJac);
+    CellScalars s = cell_rates(m, g, p, w.y, w.f0, eval_mem(w, m.R, kJac), kJac ? w.scr : nullptr, kJac);
     if (kJac) {
-      cell_jacobian(m, g, s, w.f0, eval_mem(w), w.A, w.B);
+      cell_jacobian(m, g, s, w.f0, eval_mem(w, m.R, true), w.A, w.scr);
       double* o = out + (size_t)cell * N * N;
       for (int e = g.t; e < N * N; e += NT) o[e] = -w.A[e];
     } else {
@@ -410,8 +410,7 @@ enum : int { kLaunchRates = 100, kLaunchJacobian = 101 };
 // warps per CTA, 15 named barriers), one persistent CTA wave.
 int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, int want_ctas_per_sm, int variant,
                 Launch& L) {
-  const bool matrices = variant != kLaunchRates;
-  auto plan_for = [&](int G) { return make_plan(m->host.K, m->host.R, m->dev.n_pd, G, matrices); };
+  const int kind = variant == kLaunchRates ? kPlanRates : variant == kLaunchJacobian ? kPlanCompact : integrate_plan(variant);
   // cells per SM of a call that does not fill the device
   const int64_t per_sm = (ncells + m->num_sms - 1) / m->num_sms;
   int G = want_G;
@@ -433,15 +432,21 @@ int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, in
   if (G != 1 && G != 2 && G != 4 && G != 8) return set_err(CHEM_EINVAL, "warps_per_cell must be 1, 2, 4 or 8");
   L.G = G;
   L.variant = variant;
-  L.plan = plan_for(G);
+  L.plan = make_plan(m->host.K, m->host.R, m->dev.n_pd, G, kind);
+  const int most = variant == kLaunchRates ? 256 : integrate_max_threads(G, variant == kLaunchJacobian ? kIntegrateFp64 : variant);
   const size_t per_cell = (size_t)L.plan.total * sizeof(double);
-  int max_cpc = (int)std::min<size_t>(std::max(1, std::min(CHEM_MAX_THREADS_PER_CTA / 32 / G, 15)),
+  int max_cpc = (int)std::min<size_t>(std::max(1, std::min(most / 32 / G, 15)),
                                       m->max_smem / per_cell);
   if (max_cpc < 1)
     return set_err(CHEM_ESIZE, "mechanism working set (" + std::to_string(per_cell) +
                                    " B per cell) exceeds the shared memory of one CTA");
-  // (automatic: no more cells per CTA than spread the call over all SMs)
-  const int cpc = want_cpc > 0 ? std::min(want_cpc, max_cpc) : (int)std::min<int64_t>(max_cpc, std::max<int64_t>(1, per_sm));
+  // (automatic: a call of one round takes no more cells per CTA than spread it over all SMs, one of two
+  // rounds as many as make them even -- 4 and 3 for 1000 cells instead of 5 and 2: a cell takes longer
+  // beside more others, 882 against 944 ms; a few cells over a full round do not count as another)
+  const int64_t round = (int64_t)m->num_sms * max_cpc;
+  const int64_t rounds = ncells <= round + round / 8 ? 1 : ncells <= 2 * round + round / 8 ? 2 : 0;
+  const int even = rounds ? (int)std::min<int64_t>(max_cpc, std::max<int64_t>(1, (per_sm + rounds - 1) / rounds)) : max_cpc;
+  const int cpc = want_cpc > 0 ? std::min(want_cpc, max_cpc) : even;
   L.cells_per_cta = cpc;
   L.threads = 32 * G * cpc;
   L.smem = per_cell * cpc;

@@ -16,11 +16,6 @@
 
 namespace chemgpu {
 
-// Resident CTAs per SM the kernels are compiled for.  Groups of one warp serve small mechanisms, whose
-// cells take a few KB of shared memory: there the registers limit the warps per SM, and two CTAs of
-// 128 registers a thread hide more latency than one of 255.
-constexpr int integrate_min_ctas(int G) { return G == 1 ? 2 : 1; }
-
 // Arguments of one integrate launch (all pointers device memory).
 struct IntegrateArgs {
   double p, dt, rtol, atol;
@@ -52,6 +47,19 @@ enum : int { kIntegrateFp64 = 0, kIntegrateSeulex = 1, kIntegrateOptions = 2 };
 inline int integrate_variant(int solver, bool mixed, bool fdjac) {
   return solver != 0 ? kIntegrateSeulex : (mixed || fdjac) ? kIntegrateOptions : kIntegrateFp64;
 }
+
+// Resident CTAs per SM the kernels are compiled for.  Groups of one warp serve small mechanisms, whose
+// cells take a few KB of shared memory: there the registers limit the warps per SM, and two CTAs of
+// 128 registers a thread hide more latency than one of 255.
+constexpr int integrate_min_ctas(int G) { return G == 1 ? 2 : 1; }
+
+// Threads per CTA of a variant: the default's compact plan puts five cells of 53 species on an SM, 10 warps
+// of 2 per cell at 200 registers a thread.
+constexpr int integrate_max_threads(int G, int variant) {
+  return (G == 2 && variant == kIntegrateFp64) ? CHEM_MAX_THREADS_PER_CTA / 4 * 5 : CHEM_MAX_THREADS_PER_CTA;
+}
+// Which plan of a cell (make_plan) a variant works on.
+constexpr int integrate_plan(int variant) { return variant == kIntegrateFp64 ? 1 /* kPlanCompact */ : 0 /* kPlanFull */; }
 
 // The integrate kernel of one group width (G = 1, 2, 4 or 8 warps per cell) and variant, for occupancy
 // queries and attributes; NULL for another G.

@@ -226,9 +226,11 @@ __device__ inline int64_t next_cell(const IntegrateArgs& a, const Grp<G>& g, con
 }
 
 // kAll: with the low-precision factors and the forward-difference Jacobian; without them the default's
-// code and registers are not shared with theirs.
+// code and registers are not shared with theirs, and it runs on the compact plan: the factors overwrite the
+// Jacobian, which the rare rejected attempt (0.6 % on the shear layer) evaluates again.
 template <int G, bool kAll>
-__global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G)) integrate_kernel(DevMech m, Plan plan, IntegrateArgs a) {
+__global__ void __launch_bounds__(integrate_max_threads(G, kAll ? kIntegrateOptions : kIntegrateFp64), integrate_min_ctas(G))
+    integrate_kernel(DevMech m, Plan plan, IntegrateArgs a) {
   extern __shared__ double smem[];
   Grp<G> g;
   g.init(threadIdx.x % Grp<G>::NT, threadIdx.x / Grp<G>::NT);
@@ -271,9 +273,9 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G
         if (kAll && a.fdjac) {
           cell_fd_jacobian(m, g, pc, w);
         } else {
-          const CellScalars s0 = cell_rates(m, g, pc, w.y, w.f0, eval_mem(w), w.A, true);
+          const CellScalars s0 = cell_rates(m, g, pc, w.y, w.f0, eval_mem(w, m.R, true), w.scr, true);
           PHASE_END(0);
-          cell_jacobian(m, g, s0, w.f0, eval_mem(w), w.A, w.B);
+          cell_jacobian(m, g, s0, w.f0, eval_mem(w, m.R, true), w.A, w.scr);
         }
         PHASE_END(1);
         need_jac = false;
@@ -298,9 +300,11 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G
         } else if (lowp == 2) {
           ok = form_and_factor_low<G, FF>(g, w, N, gh, reinterpret_cast<FF*>(w.invdiag));
         } else {
-          for (int e = g.t; e < N * N; e += NT) w.B[e] = w.A[e];
-          g.sync();
-          for (int i = g.t; i < N; i += NT) w.B[i * N + i] += gh;
+          if (kAll) {
+            for (int e = g.t; e < N * N; e += NT) w.B[e] = w.A[e];
+            g.sync();
+          }
+          for (int i = g.t; i < N; i += NT) w.B[i * N + i] += gh;  // (compact plan: B is A)
           g.sync();
           ok = cell_lu_default<G, double>(g, w.B, N, w.piv, w.perm, w.invdiag);
         }
@@ -398,6 +402,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G
         fac = (err == err && err < INFINITY) ? fmax(0.2, 0.9 * p25) : 0.2;
         fac = fmin(fac, 1.0);
         last_rej = true;
+        if (!kAll) need_jac = true;  // the factors have overwritten it
         h_next = h * fac;
       }
       h = fmin(h_next, a.dt - t);
@@ -493,8 +498,8 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G
       if (attempt >= a.max_steps) { status = CHEM_CELL_MAX_STEPS; break; }
       if (H_next < 1e-14 * a.dt) { status = CHEM_CELL_H_UNDERFLOW; break; }
       if (need_jac) {
-        const CellScalars s0 = cell_rates(m, g, pc, w.y, w.f0, eval_mem(w), w.A, true);
-        cell_jacobian(m, g, s0, w.f0, eval_mem(w), w.A, w.B);
+        const CellScalars s0 = cell_rates(m, g, pc, w.y, w.f0, eval_mem(w, m.R, true), w.scr, true);
+        cell_jacobian(m, g, s0, w.f0, eval_mem(w, m.R, true), w.A, w.scr);
         need_jac = false;
       }
       double fac_cur = 0.2, fac_prv = 0.2;  // fac of the last column computed and of the one before
@@ -633,7 +638,7 @@ __global__ void __launch_bounds__(CHEM_MAX_THREADS_PER_CTA, integrate_min_ctas(G
   }                                                                                                \
   void integrate_launch_g##G(int variant, int grid, int threads, size_t smem, cudaStream_t st,     \
                              const DevMech& d, const IntegrateArgs& a) {                           \
-    const Plan plan = make_plan(d.K, d.R, d.n_pd, G);                                              \
+    const Plan plan = make_plan(d.K, d.R, d.n_pd, G, integrate_plan(variant));                     \
     if (variant == kIntegrateSeulex)                                                               \
       seulex_kernel<G><<<grid, threads, smem, st>>>(d, plan, a);                                   \
     else if (variant == kIntegrateFp64)                                                            \

@@ -237,7 +237,8 @@ void build_jacobian_plan(HostMech& m) {
   for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int)i;
   // decreasing list length, so that the threads of a pass get similar work
   std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return ent[a].size() > ent[b].size(); });
-  m.zg_dst = ord;
+  m.zg_dst.clear();
+  for (int e : ord) m.zg_dst.push_back(((e / K + 1) % K) * K + (e % K + 1) % K);
   m.zgb.assign(1, 0);
   m.zgx.clear();
   const size_t longest = ent.empty() ? 0 : ent[ord[0]].size();
