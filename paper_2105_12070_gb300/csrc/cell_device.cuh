@@ -851,10 +851,23 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   s.inv_cp = recip(s.cp);
   s.dcp_dT = dcp * kRu;
   if (G == 1) g.sync();  // (with several warps the reduction's barrier has published C and the thermo)
+  // (the tables of the larger mechanisms, whose groups have several warps, do not fit what the cells leave
+  // of L1: eight loads in flight per thread here and the look-ahead below cover the L2 latency; for a
+  // small mechanism they only add instructions)
   for (int r = g.t; r < npd; r += NT) {
     const double* e = m.eff_t + r;
     S a0 = cst<S>(0.0), a1 = cst<S>(0.0);
     int k = 0;
+    for (; G > 1 && k + 7 < K; k += 8) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = e[(size_t)(k + i) * npd];
+#pragma unroll
+      for (int i = 0; i < 8; i += 2) {
+        a0 = fma(v[i], w.C[k + i], a0);
+        a1 = fma(v[i + 1], w.C[k + i + 1], a1);
+      }
+    }
     for (; k + 1 < K; k += 2) {
       a0 = fma(e[(size_t)k * npd], w.C[k], a0);
       a1 = fma(e[(size_t)(k + 1) * npd], w.C[k + 1], a1);
@@ -868,8 +881,24 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   const int r_first = (split == 0) ? g.t : (g.warp() == 0) ? g.lane() : split + g.t - 32;
   const int r_end = (split == 0 || g.warp() != 0) ? R : split;
   const int r_step = (split == 0) ? NT : (g.warp() == 0) ? 32 : NT - 32;
+  // (the next reaction's table entries are loaded beside the current one's arithmetic)
+  uint32_t slots_n = 0;
+  int64_t kA_n = 0, kb_n = 0, kE_n = 0;
+  if (G > 1 && r_first < r_end) {
+    slots_n = m.rx4[r_first];
+    kA_n = m.fxk[r_first];
+    kb_n = m.fxk[R + r_first];
+    kE_n = m.fxk[2 * R + r_first];
+  }
   for (int r = r_first; r < r_end; r += r_step) {
-    const uint32_t slots = m.rx4[r];
+    const uint32_t slots = G > 1 ? slots_n : m.rx4[r];
+    const int64_t kA = G > 1 ? kA_n : m.fxk[r], kb = G > 1 ? kb_n : m.fxk[R + r], kE = G > 1 ? kE_n : m.fxk[2 * R + r];
+    if (G > 1 && r + r_step < r_end) {
+      slots_n = m.rx4[r + r_step];
+      kA_n = m.fxk[r + r_step];
+      kb_n = m.fxk[R + r + r_step];
+      kE_n = m.fxk[2 * R + r + r_step];
+    }
     const int a0 = slots & 255, a1 = (slots >> 8) & 255, p0 = (slots >> 16) & 255, p1 = slots >> 24;
     const bool two_r = a1 != 255, two_p = p1 != 255;
     const S Ca0 = w.C[a0], Ca1 = two_r ? w.C[a1] : cst<S>(1.0);
@@ -877,7 +906,7 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
     const S pf = Ca0 * Ca1, pr = Cp0 * Cp1;
     // log2 of the forward constant, and of 1/Kc = exp(sum nu g/RT - dnu ln(Patm/(Ru T))); sums that
     // wrap on the way are right modulo 2^64
-    const int64_t Xf = m.fxk[r] + fx_mulhi(m.fxk[R + r], L2s) - fx_mulhi(m.fxk[2 * R + r], iT);
+    const int64_t Xf = kA + fx_mulhi(kb, L2s) - fx_mulhi(kE, iT);
     const int dnu = (int)two_p - (int)two_r;
     uint64_t Xc = (uint64_t)g2[p0] - (uint64_t)g2[a0];
     if (two_p) Xc += (uint64_t)g2[p1];
@@ -970,24 +999,38 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
     S om = cst<S>(0.0);
     const int len = m.sr_ptr[k + 1] - m.sr_ptr[k];
     const uint32_t* e = m.srx + k;
-    if (jac) {
-      // with the species' sums of sum_j dq/dC_j C_j and dq/dT
-      S zc = cst<S>(0.0), dw = cst<S>(0.0);
-      for (int i = 0; i < len; ++i) {
-        const uint32_t v = e[(size_t)i * K];
-        const double nu = __hiloint2double((int)(v & 0xffff0000u), 0);
-        const int r = v & 0xffffu;
-        om = fma(nu, w.q[r], om);
+    // (jac: with the species' sums of sum_j dq/dC_j C_j and dq/dT)
+    S zc = cst<S>(0.0), dw = cst<S>(0.0);
+    auto add = [&](uint32_t v) {
+      const double nu = __hiloint2double((int)(v & 0xffff0000u), 0);
+      const int r = v & 0xffffu;
+      om = fma(nu, w.q[r], om);
+      if (jac) {
         zc = fma(nu, w.DC[r], zc);
         dw = fma(nu, w.dqdT[r], dw);
       }
+    };
+    if constexpr (G == 1) {
+      for (int i = 0; i < len; ++i) add(e[(size_t)i * K]);
+    } else {
+      constexpr int kAhead = 4;
+      uint32_t v[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) v[u] = u < len ? e[(size_t)u * K] : 0u;
+      for (int i = 0; i < len; i += kAhead) {
+        uint32_t nx[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) nx[u] = i + kAhead + u < len ? e[(size_t)(i + kAhead + u) * K] : 0u;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (v[u]) add(v[u]);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) v[u] = nx[u];
+      }
+    }
+    if (jac) {
       w.zc[k] = zc;
       w.dwT[k] = dw;
-    } else {
-      for (int i = 0; i < len; ++i) {
-        const uint32_t v = e[(size_t)i * K];
-        om = fma(__hiloint2double((int)(v & 0xffff0000u), 0), w.q[v & 0xffffu], om);
-      }
     }
     w.omega[k] = om;
     Qp = fma(w.hRT[k], om, Qp);
