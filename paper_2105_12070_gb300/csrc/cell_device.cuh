@@ -359,6 +359,7 @@ struct EvalMem {
   S *zc, *dwT, *rowA, *rowB, *ccol, *wq;  // Jacobian temporaries [K]
   S* pv;                                  // efficiency-pair coefficients [n_pairs]
   S* bc = nullptr;                        // broadcast slot of the cell scalars [5] (or none)
+  bool fxM = false;                       // third-body sums in fixed point (needs bc)
 };
 
 // The solve's evaluation arrays: the Jacobian temporaries reuse the stage vectors, which are
@@ -791,6 +792,7 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   CellScalarsT<S> s;
   s.T = y[0];
   const double T = val(s.T), Td = der(s.T);
+  if (w.fxM && g.t == 0) w.bc[6] = cst<S>(0.0);  // (published by the first reduction)
   S ysum = cst<S>(0.0), yw = cst<S>(0.0);
   for (int k = g.t; k < d; k += NT) {
     const S Yk = y[1 + k];
@@ -798,6 +800,7 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
     yw = fma(Yk, sp[K + k], yw);
   }
   g.sum2(ysum, yw);
+  if (G == 1 && w.fxM) g.sync();
   const S Yd = 1.0 - ysum;
   yw = fma(Yd, sp[K + d], yw);
   // the reciprocals of T, yw and p on three lanes of each warp: one Newton iteration for all three
@@ -816,6 +819,21 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   const int64_t iT = (int64_t)(__shfl_sync(kFull, (unsigned long long)rT, 0) >>
                                ((int)(__double_as_longlong(T) >> 52) - 1029));
   const int64_t L2s = L2 << 7;
+  // Third-body sums in fixed point (w.fxM: the source-term kernel, whose four warps per sub-partition
+  // saturate the FP64 pipe; inside the integrators, with half as many, the sums wait for their tables and
+  // gain nothing): concentrations in units of 2^-60 of the power of two above the total p/(Ru T),
+  // efficiencies normalised per reaction.  The C_k add up to the total, so with no negative one beyond
+  // 1/64 of it (K <= 128) the sums of the 64-bit high products stay below 2^62; a state that breaks
+  // this takes the FP64 sums.  Where a reaction's efficiencies lie within a factor of 16 (the host's
+  // rule) the rounding, 2^-60 of the largest term each, is below that of the FP64 sum, at 20 clocks per
+  // term in place of 64-76: source terms of 53 species x 65536 1.59 -> 1.37 ms.
+  bool fxM = false;
+  int eC = 0;
+  int64_t* Cx = reinterpret_cast<int64_t*>(w.omega);  // (free until the production rates)
+  if constexpr (!kDual) {
+    fxM = w.fxM && m.effx != nullptr;
+    eC = (int)((__double_as_longlong(p * (invT * (1.0 / kRu))) >> 52) & 0x7ff);
+  }
   S cp = cst<S>(0.0), dcp = cst<S>(0.0);
   int64_t* g2 = reinterpret_cast<int64_t*>(w.gRT);  // (g/RT) / ln 2 as fx
   for (int k = g.t; k < K; k += NT) {
@@ -828,7 +846,18 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
     auto cx = [&](int i) { return __double_as_longlong(c(i)); };
     const double gT = T * fma(T, fma(T, fma(T, c(16), c(15)), c(14)), c(13));
     g2[k] = cx(10) + fx_mulhi(cx(11), L2s) + 2 * fx_mulhi(cx(12), iT) + fx_of(gT);
-    w.C[k] = s.rho * yiw;
+    const S Ck = s.rho * yiw;
+    w.C[k] = Ck;
+    if constexpr (!kDual) {
+      if (fxM) {
+        const int64_t cb = __double_as_longlong(Ck);
+        const int sh = (int)((cb >> 52) & 0x7ff) - eC + 8;  // significand (52 bits) << 8 at the total's exponent
+        if (sh > 8 || (cb < 0 && sh > 2)) w.bc[6] = 1.0;    // (not finite: the largest exponent)
+        const int64_t sig = (cb & 0xfffffffffffffLL) | 0x10000000000000LL;
+        const int64_t v = sh >= 0 ? sig << min(sh, 8) : sh > -60 ? ((sig >> (-sh - 1)) + 1) >> 1 : 0;
+        Cx[k] = cb < 0 ? -v : v;
+      }
+    }
     if (kDual || jac) {
       const double dcpv = fma(T, fma(T, fma(T, c(19), c(18)), c(17)), c(1));
       const S dcpR = with_der<S>(dcpv, kDual ? fma(T, fma(3.0 * T, c(19), 2.0 * c(18)), c(17)) * Td : 0.0);
@@ -854,7 +883,24 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   // (the tables of the larger mechanisms, whose groups have several warps, do not fit what the cells leave
   // of L1: eight loads in flight per thread here and the look-ahead below cover the L2 latency; for a
   // small mechanism they only add instructions)
-  for (int r = g.t; r < npd; r += NT) {
+  if constexpr (!kDual) {
+    fxM = fxM && w.bc[6] == 0.0;
+    if (fxM) {
+      for (int r = g.t; r < npd; r += NT) {
+        const int64_t* e = m.effx + r;
+        int64_t a0 = K >> 1, a1 = 0;  // (half a unit per truncated product)
+        int k = 0;
+        for (; k + 1 < K; k += 2) {
+          a0 += fx_mulhi(e[(size_t)k * npd], Cx[k]);
+          a1 += fx_mulhi(e[(size_t)(k + 1) * npd], Cx[k + 1]);
+        }
+        if (k < K) a0 += fx_mulhi(e[(size_t)k * npd], Cx[k]);
+        // units: 2^(eC - 1023 - 60) of the concentrations, 2^(exponent - 62) of the efficiencies
+        w.M[r] = (double)(a0 + a1) * pow2(eC - 1023 - 58 + m.effe[r]);
+      }
+    }
+  }
+  for (int r = fxM ? npd : g.t; r < npd; r += NT) {
     const double* e = m.eff_t + r;
     S a0 = cst<S>(0.0), a1 = cst<S>(0.0);
     int k = 0;

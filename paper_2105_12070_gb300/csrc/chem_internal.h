@@ -63,6 +63,10 @@ struct HostMech {
   std::vector<double> spf;             // [kSpfRows][K]
   std::vector<double> rxd_t;           // [2][R] b, Ea/Rc
   std::vector<double> eff_t;           // [K][n_pd] efficiencies, transposed
+  // the same in fixed point, eff * 2^(62 - effe) with effe[r] the exponent that puts the reaction's largest
+  // below 1; empty unless every reaction's efficiencies are positive and within a factor of 16
+  std::vector<int64_t> effx;           // [K][n_pd]
+  std::vector<int> effe;               // [n_pd]
   // species production lists, entry e of species k at [e * K + k]: reaction index in the low half,
   // the top 16 bits of the net coefficient as a double in the high half (small integers have no others)
   std::vector<uint32_t> srx;
@@ -134,6 +138,8 @@ struct DevMech {
   const double* spf;
   const double* rxd_t;
   const double* eff_t;
+  const int64_t* effx;  // NULL: none
+  const int* effe;
   const uint32_t* srx;
 };
 

@@ -47,7 +47,9 @@ __global__ void __launch_bounds__(kJac && G == 2 ? 320 : 256, kJac ? 1 : 2) rate
   for (int64_t cell = (int64_t)blockIdx.x * groups_per_cta + g.gid; cell < ncells; cell += ngroups) {
     for (int i = g.t; i < N; i += NT) w.y[i] = (i == 0) ? T[cell] : Y[(size_t)(i - 1) * ncells + cell];
     g.sync();
-    CellScalars s = cell_rates(m, g, p, w.y, w.f0, eval_mem(w, m.R, kJac), kJac ? w.scr : nullptr, kJac);
+    EvalMem<double> e = eval_mem(w, m.R, kJac);
+    e.fxM = !kJac;
+    CellScalars s = cell_rates(m, g, p, w.y, w.f0, e, kJac ? w.scr : nullptr, kJac);
     if (kJac) {
       cell_jacobian(m, g, s, w.f0, eval_mem(w, m.R, true), w.A, w.scr);
       double* o = out + (size_t)cell * N * N;
@@ -650,6 +652,8 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   const size_t o_spf = place(h.spf.size() * sizeof(double));
   const size_t o_rdt = place(h.rxd_t.size() * sizeof(double));
   const size_t o_eft = place(h.eff_t.size() * sizeof(double));
+  const size_t o_efx = place(std::max<size_t>(1, h.effx.size()) * sizeof(int64_t));
+  const size_t o_efe = place(h.effe.size() * sizeof(int));
   const size_t o_srx = place(h.srx.size() * sizeof(uint32_t));
   const size_t total = off;
   std::vector<char> img(total, 0);
@@ -684,6 +688,8 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   put(o_spf, h.spf.data(), h.spf.size() * sizeof(double));
   put(o_rdt, h.rxd_t.data(), h.rxd_t.size() * sizeof(double));
   put(o_eft, h.eff_t.data(), h.eff_t.size() * sizeof(double));
+  put(o_efx, h.effx.data(), h.effx.size() * sizeof(int64_t));
+  put(o_efe, h.effe.data(), h.effe.size() * sizeof(int));
   put(o_srx, h.srx.data(), h.srx.size() * sizeof(uint32_t));
   e = cudaMalloc(&m->dbuf, total);
   if (e == cudaSuccess) e = cudaMemcpy(m->dbuf, img.data(), total, cudaMemcpyHostToDevice);
@@ -727,6 +733,8 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   d.spf = reinterpret_cast<const double*>(b + o_spf);
   d.rxd_t = reinterpret_cast<const double*>(b + o_rdt);
   d.eff_t = reinterpret_cast<const double*>(b + o_eft);
+  d.effx = h.effx.empty() ? nullptr : reinterpret_cast<const int64_t*>(b + o_efx);
+  d.effe = reinterpret_cast<const int*>(b + o_efe);
   d.srx = reinterpret_cast<const uint32_t*>(b + o_srx);
   d.n_pairs = (int)h.pr_pd.size();
   d.n_prows = (int)h.pr_rows.size();

@@ -87,6 +87,22 @@ void build_fx_tables(HostMech& m) {
   m.eff_t.assign((size_t)std::max(npd, 1) * K, 0.0);
   for (int r = 0; r < npd; ++r)
     for (int k = 0; k < K; ++k) m.eff_t[(size_t)k * npd + r] = m.eff[(size_t)r * K + k];
+  bool even = npd > 0;
+  for (int r = 0; r < npd && even; ++r) {
+    const auto* e = &m.eff[(size_t)r * K];
+    const double lo = *std::min_element(e, e + K), hi = *std::max_element(e, e + K);
+    even = lo > 0.0 && hi <= 16.0 * lo && hi < 1e9 && lo > 1e-9;
+  }
+  m.effx.clear();
+  m.effe.assign(std::max(npd, 1), 0);
+  if (even) {
+    m.effx.assign((size_t)npd * K, 0);
+    for (int r = 0; r < npd; ++r) {
+      const auto* e = &m.eff[(size_t)r * K];
+      m.effe[r] = std::ilogb(*std::max_element(e, e + K)) + 1;
+      for (int k = 0; k < K; ++k) m.effx[(size_t)k * npd + r] = (int64_t)std::llround(std::ldexp((long double)e[k], 62 - m.effe[r]));
+    }
+  }
   int longest = 0;
   for (int k = 0; k < K; ++k) longest = std::max(longest, m.sr_ptr[k + 1] - m.sr_ptr[k]);
   m.srx.assign((size_t)std::max(longest, 1) * K, 0);

@@ -120,3 +120,36 @@ def test_ln_a_change_moves_the_interval_of_a_captured_launch():
     chem.chem_set_lnA(mech, lnA)
     again = step(opts)
     assert torch.equal(first[0], again[0]) and torch.equal(first[1], again[1])
+
+
+@pytest.mark.parametrize("efficiencies", ["even", "one_hot"])
+def test_third_body_sums_of_unphysical_states(efficiencies):
+    """The source-term kernel's fixed-point third-body sums hand over what they cannot hold: mass
+    fractions far outside [0, 1] (a diverged trial state), and mechanisms with zero efficiencies."""
+    m = copy.deepcopy(synth.mechanism_53())
+    if efficiencies == "one_hot":
+        r = min(m.eff)
+        m.eff[r] = np.eye(m.K)[3]
+    path = m.write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    rng = np.random.default_rng(9)
+    n = 64
+    Y = rng.dirichlet(np.ones(m.K), size=n)
+    for c in range(n):
+        if c % 4 == 1:
+            Y[c, c % m.K] -= 0.9           # one large negative, made up for elsewhere
+            Y[c, (c + 7) % m.K] += 0.9
+        elif c % 4 == 2:
+            Y[c, ::2] += 2.0               # many beyond 1, as many below -1
+            Y[c, 1::2] -= 2.0 * Y[c, ::2].size / Y[c, 1::2].size
+        elif c % 4 == 3:
+            Y[c, c % m.K] -= 0.03          # near the bound of 1/64 of the total
+    T = rng.uniform(800.0, 2000.0, n)
+    Y = np.ascontiguousarray(Y.T)
+    f = torch.empty((mech.N, n), dtype=torch.float64, device="cuda")
+    chem.chem_rates(mech, P, _dev(T), _dev(Y), f)
+    torch.cuda.synchronize()
+    fo, gross = ora.rates(P, T, Y, gross=True)
+    ok = np.isfinite(fo).all(axis=0) & np.isfinite(gross).all(axis=0)
+    assert ok.sum() >= n // 2
+    assert np.all(np.abs(f.cpu().numpy() - fo)[:, ok] <= 1e-11 * gross[:, ok] + 1e-300)
