@@ -343,14 +343,27 @@ int adjoint_enqueue(const DevMech& d, int num_sms, size_t max_smem, double p_cgs
                     int rec_cap, const int32_t* nsteps, const int32_t* status, const double* gT, const double* gY,
                     double* gT0, double* gY0, double* g_lnA, double* g_lnA_cells, double* ws, int* counters,
                     cudaStream_t st, std::string& err) {
-  // launch shape: 8 warps per CTA; two cells of 4 warps when both working sets fit, else one
-  // cell of 8 warps
-  int G = 4, cpc = 2;
-  AdjPlan plan = make_adj_plan(d.K, d.R, d.n_pd, d.n_pairs, G);
-  if ((size_t)plan.total * sizeof(double) * cpc > max_smem) {
+  // Launch shape, 8 warps per CTA at most.  A small mechanism's cell keeps one warp busy: one each, spread
+  // over all SMs (a step of the 10-species mechanism has no loop of more than three passes by 32 lanes,
+  // and a single warp needs no barriers).  Else two cells of 4 warps when both working sets fit and there
+  // is more than one cell per SM, else one of 8 warps.
+  const int64_t per_sm = (ncells + num_sms - 1) / num_sms;
+  int G, cpc;
+  AdjPlan plan;
+  auto bytes = [&](int g) {
+    plan = make_adj_plan(d.K, d.R, d.n_pd, d.n_pairs, g);
+    return (size_t)plan.total * sizeof(double);
+  };
+  if (d.K <= 16 && bytes(1) <= max_smem) {
+    G = 1;
+    cpc = (int)std::min<int64_t>({8, std::max<int64_t>(1, per_sm), (int64_t)(max_smem / bytes(1))});
+  } else if (per_sm > 1 && 2 * bytes(4) <= max_smem) {
+    G = 4;
+    cpc = 2;
+  } else {
     G = 8;
     cpc = 1;
-    plan = make_adj_plan(d.K, d.R, d.n_pd, d.n_pairs, G);
+    bytes(8);
   }
   const size_t smem = (size_t)plan.total * sizeof(double) * cpc;
   if (smem > max_smem) {
@@ -363,7 +376,9 @@ int adjoint_enqueue(const DevMech& d, int num_sms, size_t max_smem, double p_cgs
   };
   cudaError_t e = cudaMemsetAsync(counters, 0, 2 * sizeof(int), st);
   if (e != cudaSuccess) return fail(e, "cudaMemsetAsync");
-  const void* fn = G == 4 ? (const void*)adjoint_kernel<4> : (const void*)adjoint_kernel<8>;
+  const void* fn = G == 1   ? (const void*)adjoint_kernel<1>
+                   : G == 4 ? (const void*)adjoint_kernel<4>
+                            : (const void*)adjoint_kernel<8>;
   const int threads = 32 * G * cpc;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return fail(e, "cudaFuncSetAttribute");
@@ -382,7 +397,8 @@ int adjoint_enqueue(const DevMech& d, int num_sms, size_t max_smem, double p_cgs
   a.queue = counters; a.nfail = counters + 1;
   const int64_t ctas = (ncells + cpc - 1) / cpc;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, (int64_t)num_sms * occ));
-  if (G == 4) adjoint_kernel<4><<<grid, threads, smem, st>>>(d, plan, a);
+  if (G == 1) adjoint_kernel<1><<<grid, threads, smem, st>>>(d, plan, a);
+  else if (G == 4) adjoint_kernel<4><<<grid, threads, smem, st>>>(d, plan, a);
   else adjoint_kernel<8><<<grid, threads, smem, st>>>(d, plan, a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(e, "adjoint kernel launch");

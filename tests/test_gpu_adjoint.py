@@ -222,3 +222,24 @@ def test_autograd_function(small):
     np.testing.assert_array_equal(T0.grad.cpu().numpy(), gT0)
     np.testing.assert_array_equal(Y0.grad.cpu().numpy(), gY0)
     np.testing.assert_array_equal(lnA.grad.cpu().numpy(), gA)
+
+
+@pytest.mark.parametrize("which,dt", [("small", 1e-7), ("igniting", 1e-10)])
+def test_gradients_do_not_depend_on_the_company(which, dt, request):
+    """A few cells alone take another launch shape of the reverse sweep than among many (one warp per
+    small cell; eight instead of four for a large one).  The shapes sum the same terms in other
+    orders: agreement to 1e-10 of the largest component (a few hundred steps of roundings of 1e-16
+    each, amplified by the step's conditioning as in the dot-product test)."""
+    w, mech, _ = request.getfixturevalue(which)
+    many = np.arange(200) % 16
+    few = np.arange(3)
+    rng = np.random.default_rng(3)
+    gT, gY = rng.standard_normal(16), rng.standard_normal((mech.K, 16))
+    out = []
+    for cells in (many, few):
+        _, _, rec, nsteps, status = _record(mech, w, cells, cap=2048, dt=dt)
+        assert torch.all(status == 0)
+        out.append(_adjoint(mech, w, rec, nsteps, status, gT[cells], np.ascontiguousarray(gY[:, cells])))
+    for c in few:
+        for a, b in ((out[0][0][c], out[1][0][c]), (out[0][1][:, c], out[1][1][:, c]), (out[0][3][c], out[1][3][c])):
+            assert np.max(np.abs(a - b)) <= 1e-10 * np.max(np.abs(b))
