@@ -128,18 +128,20 @@ void build_fx_tables(HostMech& m) {
       return (std::fabs(lnA) + std::fabs(E) / lo) * 1.4427 + std::fabs(b) * 13.0 < 1000.0;
     };
     // bound over [lo, hi] of |sum_k c_k (g_k/RT)| / ln 2
-    auto g_bound = [&](const std::vector<std::pair<int, double>>& terms) {
-      std::vector<double> ends = {lo, hi};
-      for (const auto& t : terms) {
-        const double mid = m.spf[(size_t)2 * K + t.first];
-        if (mid > lo && mid < hi) ends.push_back(mid);
+    auto g_bound = [&](const std::pair<int, double>* terms, int n_terms) {
+      double ends[6] = {lo, hi};
+      int n_ends = 2;
+      for (int t = 0; t < n_terms; ++t) {
+        const double mid = m.spf[(size_t)2 * K + terms[t].first];
+        if (mid > lo && mid < hi) ends[n_ends++] = mid;
       }
-      std::sort(ends.begin(), ends.end());
+      std::sort(ends, ends + n_ends);
       double worst = 0.0;
-      for (size_t e = 0; e + 1 < ends.size(); ++e) {
+      for (int e = 0; e + 1 < n_ends; ++e) {
         const double t0 = ends[e], t1 = ends[e + 1], mid = 0.5 * (t0 + t1);
         double c[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (const auto& t : terms) {
+        for (int u = 0; u < n_terms; ++u) {
+          const std::pair<int, double>& t = terms[u];
           const int first = 3 + (mid <= m.spf[(size_t)2 * K + t.first] ? 0 : kSpfRange) + 10;
           for (int i = 0; i < 7; ++i) {
             const double o = m.spf[(size_t)(first + i) * K + t.first];
@@ -154,7 +156,10 @@ void build_fx_tables(HostMech& m) {
       }
       return worst;
     };
-    for (int k = 0; k < K && fits; ++k) fits = g_bound({{k, 1.0}}) < 1000.0;
+    for (int k = 0; k < K && fits; ++k) {
+      const std::pair<int, double> one(k, 1.0);
+      fits = g_bound(&one, 1) < 1000.0;
+    }
     for (int r = 0; r < R && fits; ++r) {
       const double* d = &m.rxd[(size_t)r * kRxDoubles];
       fits = rate_fits(d[0], d[1], d[2]);
@@ -163,10 +168,11 @@ void build_fx_tables(HostMech& m) {
         fits = rate_fits(q[0], q[1], q[2]);
       }
       const int* ii = &m.rxi[(size_t)r * kRxInts];
-      std::vector<std::pair<int, double>> terms;
+      std::pair<int, double> terms[4];
+      int n = 0;
       for (int u = 0; u < 4; ++u)
-        if (ii[u] >= 0) terms.push_back({ii[u], u < 2 ? -1.0 : 1.0});
-      fits = fits && g_bound(terms) < 900.0;
+        if (ii[u] >= 0) terms[n++] = {ii[u], u < 2 ? -1.0 : 1.0};
+      fits = fits && g_bound(terms, n) < 900.0;
     }
     if (fits) {
       m.fx_T = {lo, hi};
@@ -247,20 +253,32 @@ void build_jacobian_plan(HostMech& m) {
       }
     }
   }
-  std::vector<std::vector<Contrib>> ent((size_t)d * K);  // one list per entry of the species rows
-  for (const Contrib& c : cs) ent[c.dst].push_back(c);
-  std::vector<int> ord(ent.size());
-  for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int)i;
-  // decreasing list length, so that the threads of a pass get similar work
-  std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return ent[a].size() > ent[b].size(); });
+  // contributions entry by entry (counting sort), and the entries by decreasing list length, so that the
+  // threads of a pass get similar work
+  std::vector<int> first((size_t)d * K + 1, 0);
+  for (const Contrib& c : cs) first[c.dst + 1]++;
+  size_t longest = 0;
+  for (int e = 0; e < d * K; ++e) {
+    longest = std::max<size_t>(longest, first[e + 1]);
+    first[e + 1] += first[e];
+  }
+  std::vector<Contrib> ent(cs.size());
+  {
+    std::vector<int> at(first.begin(), first.end() - 1);
+    for (const Contrib& c : cs) ent[at[c.dst]++] = c;
+  }
+  std::vector<int> ord, of_length(longest + 2, 0);
+  for (int e = 0; e < d * K; ++e) of_length[longest - (first[e + 1] - first[e]) + 1]++;
+  for (size_t l = 0; l <= longest; ++l) of_length[l + 1] += of_length[l];
+  ord.resize((size_t)d * K);
+  for (int e = 0; e < d * K; ++e) ord[of_length[longest - (first[e + 1] - first[e])]++] = e;
   m.zg_dst.clear();
   for (int e : ord) m.zg_dst.push_back(((e / K + 1) % K) * K + (e % K + 1) % K);
   m.zgb.assign(1, 0);
   m.zgx.clear();
-  const size_t longest = ent.empty() ? 0 : ent[ord[0]].size();
   for (size_t c = 0; c < longest; ++c) {
-    for (size_t i = 0; i < ord.size() && ent[ord[i]].size() > c; ++i) {
-      const Contrib& x = ent[ord[i]][c];
+    for (size_t i = 0; i < ord.size() && first[ord[i]] + (int)c < first[ord[i] + 1]; ++i) {
+      const Contrib& x = ent[first[ord[i]] + c];
       uint64_t b;
       std::memcpy(&b, &x.coef, 8);
       m.zgx.push_back((uint32_t)x.src | (uint32_t)(b >> 48) << 16);
