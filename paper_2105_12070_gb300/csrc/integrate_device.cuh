@@ -193,7 +193,8 @@ __device__ __forceinline__ bool stage_solve_low(const Grp<G>& g, const CellMem& 
   return conv <= CHEM_REFINE_TOL;
 }
 
-// u <- W^-1 rhs: FP64 factors (lowp 0: one solve), FP32 factors (1) or FP32 pairs (2).
+// u <- W^-1 rhs: FP32 factors (lowp 1) or FP32 pairs (2) from w.rhs; FP64 factors (0) in place, the right-hand
+// side in u.
 template <bool kAll, int G>
 __device__ __forceinline__ bool stage_solve(const Grp<G>& g, const CellMem& w, const IntegrateArgs& a, int N, double gh, int lowp,
                             double* u) {
@@ -202,8 +203,6 @@ __device__ __forceinline__ bool stage_solve(const Grp<G>& g, const CellMem& w, c
     if (lowp == 1) return stage_solve_low<G, float>(g, w, a, N, gh, u);
     if (lowp == 2) return stage_solve_low<G, FF>(g, w, a, N, gh, u);
   }
-  for (int i = g.t; i < N; i += NT) u[i] = w.rhs[i];
-  g.sync();
   cell_solve(g, w.B, N, w.perm, w.invdiag, u);
   return true;
 }
@@ -310,65 +309,56 @@ __global__ void __launch_bounds__(integrate_max_threads(G, kAll ? kIntegrateOpti
         }
         PHASE_END(2);
         if (!ok) break;  // exactly singular: reject the attempt
+        // The four stages, then (stage 4 of this loop) the solution and the embedded error, filtered through
+        // (I - gamma h J)^-1 = W^-1 / (gamma h).  One copy of the evaluation and of the substitutions
+        // serves all of them: the loop body is what the instruction cache has to hold.
         bool conv = true;
-        // stage 1
-        for (int i = g.t; i < N; i += NT) w.rhs[i] = w.f0[i];
-        g.sync();
-        conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[0]);
-        PHASE_END(3);
-        // stage 2
-        if (conv) {
-          for (int i = g.t; i < N; i += NT) w.ynew[i] = fma(c_a21, w.u[0][i], w.y[i]);
+        const int n2 = (int)(w.u[1] - w.u[0]);
+        for (int stage = 0; stage < 5; ++stage) {
+          if (stage == 1 || stage == 2) {  // (stage 3 has stage 2's argument)
+            for (int i = g.t; i < N; i += NT)
+              w.ynew[i] = stage == 1 ? fma(c_a21, w.u[0][i], w.y[i]) : w.y[i] + c_a31 * w.u[0][i] + c_a32 * w.u[1][i];
+            g.sync();
+            cell_rates(m, g, pc, w.ynew, w.fs, eval_mem(w), (double*)nullptr, false);
+            PHASE_END(4);
+          }
+          double* x = stage < 4 ? w.u[0] + stage * n2 : w.err;
+          double* rhs = (kAll && lowp) ? w.rhs : x;  // FP64 substitutions work in place
+          for (int i = g.t; i < N; i += NT) {
+            double v;
+            if (stage == 0) {
+              v = w.f0[i];
+            } else if (stage == 1) {
+              v = fma(c_c21 * invh, w.u[0][i], w.fs[i]);
+            } else if (stage == 2) {
+              v = w.fs[i] + invh * (c_c31 * w.u[0][i] + c_c32 * w.u[1][i]);
+            } else if (stage == 3) {
+              v = w.fs[i] + invh * (c_c41 * w.u[0][i] + c_c42 * w.u[1][i] + c_c43 * w.u[2][i]);
+            } else {
+              w.ynew[i] = w.y[i] + c_m[0] * w.u[0][i] + c_m[1] * w.u[1][i] + c_m[2] * w.u[2][i] + c_m[3] * w.u[3][i];
+              v = c_e[0] * w.u[0][i] + c_e[1] * w.u[1][i] + c_e[2] * w.u[2][i] + c_e[3] * w.u[3][i];
+            }
+            rhs[i] = v;
+          }
           g.sync();
-          cell_rates(m, g, pc, w.ynew, w.fs, eval_mem(w), (double*)nullptr, false);
-          PHASE_END(4);
-          for (int i = g.t; i < N; i += NT) w.rhs[i] = fma(c_c21 * invh, w.u[0][i], w.fs[i]);
-          g.sync();
-          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[1]);
+          if (kAll && lowp && stage == 4) {
+            // (the filter only feeds the step-size control, so low-precision factors need no refinement)
+            if (g.warp() == g.lead) {
+              if (lowp == 1) low_solve<float>(w, N, w.invd32, w.rhs, w.err);
+              else low_solve<FF>(w, N, reinterpret_cast<const FF*>(w.invdiag), w.rhs, w.err);
+            }
+            g.sync();
+          } else {
+            conv = stage_solve<kAll>(g, w, a, N, gh, lowp, x);
+            if (!conv) break;
+          }
           PHASE_END(3);
-        }
-        // stage 3
-        if (conv) {
-          for (int i = g.t; i < N; i += NT) w.ynew[i] = w.y[i] + c_a31 * w.u[0][i] + c_a32 * w.u[1][i];
-          g.sync();
-          cell_rates(m, g, pc, w.ynew, w.fs, eval_mem(w), (double*)nullptr, false);
-          PHASE_END(4);
-          for (int i = g.t; i < N; i += NT)
-            w.rhs[i] = w.fs[i] + invh * (c_c31 * w.u[0][i] + c_c32 * w.u[1][i]);
-          g.sync();
-          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[2]);
-        }
-        // stage 4 (same argument as stage 3)
-        if (conv) {
-          for (int i = g.t; i < N; i += NT)
-            w.rhs[i] = w.fs[i] + invh * (c_c41 * w.u[0][i] + c_c42 * w.u[1][i] + c_c43 * w.u[2][i]);
-          g.sync();
-          conv = stage_solve<kAll>(g, w, a, N, gh, lowp, w.u[3]);
         }
         if (!conv) {
           if (g.t == 0) atomicAdd(&a.totals[3], 1ull);
           f64_until = attempt + CHEM_MIXED_FP64_RUN;
           continue;  // redo this attempt with FP64 factors
         }
-        // solution, embedded error, filtered through (I - gamma h J)^-1 = W^-1 / (gamma h)
-        // (the filter only feeds the step-size control, so FP32 factors need no refinement)
-        for (int i = g.t; i < N; i += NT) {
-          w.ynew[i] = w.y[i] + c_m[0] * w.u[0][i] + c_m[1] * w.u[1][i] + c_m[2] * w.u[2][i] + c_m[3] * w.u[3][i];
-          w.rhs[i] = c_e[0] * w.u[0][i] + c_e[1] * w.u[1][i] + c_e[2] * w.u[2][i] + c_e[3] * w.u[3][i];
-        }
-        g.sync();
-        if (lowp == 1) {
-          if (g.warp() == g.lead) low_solve<float>(w, N, w.invd32, w.rhs, w.err);
-          g.sync();
-        } else if (lowp == 2) {
-          if (g.warp() == g.lead) low_solve<FF>(w, N, reinterpret_cast<const FF*>(w.invdiag), w.rhs, w.err);
-          g.sync();
-        } else {
-          for (int i = g.t; i < N; i += NT) w.err[i] = w.rhs[i];
-          g.sync();
-          cell_solve(g, w.B, N, w.perm, w.invdiag, w.err);
-        }
-        PHASE_END(3);
         double e = 0.0;
         for (int i = g.t; i < N; i += NT) {
           const double sc = fma(a.rtol, Grp<G>::max_mag(w.y[i], w.ynew[i]), a.atol);

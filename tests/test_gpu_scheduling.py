@@ -99,3 +99,22 @@ def test_cells_beside_each_other_do_not_matter(solver, dt, max_steps):
         if ref is None:
             ref = got
         assert got[:2] == ref[:2] and torch.equal(T, ref[2]) and torch.equal(Y, ref[3]), cpc
+
+
+@pytest.mark.parametrize("solver", [chem.CHEM_SOLVER_ROSENBROCK, chem.CHEM_SOLVER_SEULEX])
+def test_warps_per_cell_keep_the_bits(solver):
+    """From 32 to 64 species every thread holds at most one component with 2, 4 or 8 warps: the automatic
+    shape may take more warps for a call of few cells without changing a cell's result."""
+    w = synth.workload_shear_layer(16)
+    mech = chem.Mechanism(w["mech"].write_temp())
+    idx = np.arange(0, 256, 37)
+    ref = None
+    for shape in (dict(warps_per_cell=2), dict(warps_per_cell=4), dict(warps_per_cell=8), dict()):
+        T = torch.from_numpy(w["T"][idx].copy()).cuda()
+        Y = torch.from_numpy(np.ascontiguousarray(w["Y"][:, idx])).cuda()
+        chem.chem_integrate(mech, w["p_Pa"], T, Y, 1e-9, w["rtol"], w["atol"],
+                            opts=chem.default_opts(solver=solver, **shape))
+        torch.cuda.synchronize()
+        if ref is None:
+            ref = (T, Y)
+        assert torch.equal(T, ref[0]) and torch.equal(Y, ref[1]), shape
