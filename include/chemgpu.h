@@ -262,8 +262,8 @@ int chem_last_cell_counters(const chem_mech* mech, int32_t* steps, int32_t* reje
  * benchmark reports for the integrate kernel, measured in the same process and clock state. */
 int chem_probe_fp64_peak(double* tflops);
 
-/* Diagnostic for the tests: y[i] = the exponential the rate kernels use (table-driven, Tang
- * 1989) of x[i], n entries, device arrays, asynchronous on `stream`. */
+/* Diagnostic for the tests: y[i] = the exponential of the general rate evaluation (table-driven,
+ * Tang 1989; states outside the fixed-point range use it) of x[i], n entries, device arrays, asynchronous on `stream`. */
 int chem_debug_exp(const double* x, double* y, int64_t n, void* stream);
 
 /* Diagnostic for the tests: factors n dense N x N matrices (A: n x N x N, row-major, FP64,

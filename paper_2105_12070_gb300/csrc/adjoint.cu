@@ -19,7 +19,8 @@
 // Y_3 and Y_2, and four evaluations of J^T v_i in dual numbers along u_i.  The J^T products are
 // matrix-free (cell_jacobian_vjp): weighted column sums of d omega/dC built from the
 // per-reaction data, so only the Jacobian at y_n (for W) is ever formed.  That keeps the working
-// set near 95 KB for 53 species: two cells of 4 warps per CTA, cells from a queue.
+// set near 95 KB for 53 species: two cells of 4 warps per CTA (one of
+// 8 warps when there are no more cells than SMs, one warp per cell up to 16 species), cells from a queue.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -1114,7 +1114,7 @@ __device__ __forceinline__ CellScalarsT<S> cell_rates(const DevMech& m, const Gr
 // rho = p Wbar/(Ru T), Y_K = 1 - sum Y_i, in place on Z: rows k < K-1 hold d omega_k / dC, row K-1
 // d Q / dC (Q = sum_k H_k omega_k).  Z's entry (k, j) is kept at row k + 1 and column j + 1, both modulo K,
 // where the entry of J made from it belongs; Z's last row and column become J's temperature row and column.
-// Bound by FP64 issue; the plans are read as packed 4-byte words in the threads' order (8 KB of the
+// Bound by FP64 issue; the plans are read as packed 4-byte words in the threads' order (28 KB of the
 // SM's L1 is left beside the cells' shared memory for 53 species, so their volume counts).
 template <int G>
 __device__ void cell_jacobian(const DevMech& m, const Grp<G>& g, const CellScalars& s, const double* f,

@@ -10,7 +10,7 @@ timers perturb the kernel a little; compare phases, not absolute speed.
     python -m paper_2105_12070_gb300.phases [--cells 1216] [--dt 1e-8] [--define NAME ...] [--modes 0,2]
 
 --define adds a preprocessor macro to the timer build (e.g. CHEM_LU_VARIANT=0: the LU column by
-column, =2: in 8-column panels; CHEM_LU_RCP_DIVISION: FP64 pivot reciprocals by division).
+column, =2: in 8-column panels).
 """
 from __future__ import annotations
 
