@@ -554,9 +554,9 @@ __device__ inline void troe_fx(const double* fd, int n, S T, S invT, S Pr, S& F,
 }
 
 // Evaluates f(y) into f[0..N).  With jac, also leaves per-reaction derivative data in
-// scr[u * R + r], u = 0..4: {dq/dC through each of the 4 slots (an empty slot's entry is not read),
-// phi (coefficient of the efficiencies; pressure-dependent reactions only)} (rows of R, so that the
-// threads of consecutive reactions store to consecutive words), the species production rates in
+// scr[u * R + r]: for u = 0..3 dq/dC through each of the 4 slots (an empty slot's entry is not read), and
+// for u = 4 and r < n_pd only phi, the coefficient of the efficiencies: 4 R + n_pd entries in all, in rows
+// so that the threads of consecutive reactions store to consecutive words.  The species production rates in
 // w.omega and the species' sums of sum_j dq/dC_j C_j and of dq/dT at fixed C in w.zc and w.dwT.
 // With kP (adjoint use, requires jac) it also writes P[r] = v . d f / d ln A_r for the weight
 // vector v = vP (N): with q'_r = d q_r / d ln A_r (q_r for elementary and third-body
@@ -719,7 +719,7 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
       o[R] = kfm * Ca0;
       o[2 * R] = -krm * Cp1;
       o[3 * R] = -krm * Cp0;
-      o[4 * R] = phi;
+      if (pd) o[4 * R] = phi;  // (the compact plan has this row for the pressure-dependent reactions only)
       w.DC[r] = fma(phi, Mr, ((a1 >= 0) ? Rf + Rf : Rf) - ((p1 >= 0) ? Rr + Rr : Rr));
       w.dqdT[r] = dqdT;
       if (kP) {

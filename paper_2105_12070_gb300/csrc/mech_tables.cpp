@@ -232,9 +232,9 @@ struct FileReaction {
 
 // Gather plan of the Jacobian's mass-action part and the row lists of its efficiency part, for
 // the species rows k < K-1 (the enthalpy row follows from them, see the kernels).
-// Per-reaction scratch layout (see the kernels): 8 rows of R values, scr[u * R + r] with u =
-// 0..3 dq/dC at the distinct slot species, 4 phi, 5 sum_j dq/dC_j C_j, 6 dq/dT, 7 reaction
-// enthalpy (rows, so that the threads of consecutive reactions touch consecutive words).
+// Per-reaction scratch layout (see the kernels): 4 R + n_pd values, scr[u * R + r] with u = 0..3 dq/dC
+// through the four slots, and scr[4 R + r], r < n_pd, phi (rows, so that the threads of consecutive
+// reactions touch consecutive words).
 void build_jacobian_plan(HostMech& m) {
   const int K = m.K, d = K - 1;
   struct Contrib { int dst, src; double coef; };

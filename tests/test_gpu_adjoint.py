@@ -243,3 +243,14 @@ def test_gradients_do_not_depend_on_the_company(which, dt, request):
     for c in few:
         for a, b in ((out[0][0][c], out[1][0][c]), (out[0][1][:, c], out[1][1][:, c]), (out[0][3][c], out[1][3][c])):
             assert np.max(np.abs(a - b)) <= 1e-10 * np.max(np.abs(b))
+
+
+@pytest.mark.parametrize("which,T,dt", [("small", [150.0, 8200.0, 8500.0, 9000.0], 1e-10), ("igniting", [150.0, 200.0, 250.0], 1e-9)])
+def test_adjoint_outside_the_fixed_point_range(which, T, dt, request):
+    """The general rate evaluation in FP64 and in dual numbers: states outside the temperature interval of
+    the fixed-point one."""
+    w, mech, om = request.getfixturevalue(which)
+    cells = np.arange(len(T))
+    Y = np.ascontiguousarray(np.random.default_rng(5).dirichlet(np.ones(mech.K), size=len(T)).T)
+    w = dict(w, T=np.array(T), Y=Y, dt=dt)
+    _dot_test(w, mech, om, cells, seed=4)

@@ -1,8 +1,8 @@
 """The fixed-point rate evaluation at the edges of its range, against the oracle: temperatures on both
 sides of the interval it takes and of Tmid, states with zero, tiny and slightly negative mass
 fractions, a species on both sides of a reaction, mechanisms it must leave to the general form, and a change of ln A that moves the
-interval under a captured launch.  Tolerances as in test_gpu_parity.py (1e-11 of the gross flux,
-1e-12 of the row)."""
+interval under a captured launch; and solves on the general form, against the oracle.  Tolerances as in
+test_gpu_parity.py (1e-11 of the gross flux, 1e-12 of the row; solves rtol/atol-shaped)."""
 import copy
 import os
 
@@ -59,6 +59,61 @@ def test_edges_of_the_range(make):
     _check(mech, ora, T, Y)
 
 
+RTOL, ATOL = 1e-6, 1e-10
+SOLVERS = ((chem.CHEM_SOLVER_ROSENBROCK, "rosenbrock"), (chem.CHEM_SOLVER_SEULEX, "seulex"))
+
+
+def _check_solves(mech, ora, T, Y, dt, p=P, solvers=SOLVERS, **options):
+    for solver, name in solvers:
+        To, Yo, sto, _, _ = ora.integrate(p, T, Y, dt, RTOL, ATOL, nthreads=4, solver=name)
+        assert np.all(sto == 0)
+        Td, Yd = _dev(T), _dev(Y)
+        status = torch.full((T.size,), -1, dtype=torch.int32, device="cuda")
+        chem.chem_integrate(mech, p, Td, Yd, dt, RTOL, ATOL, status=status,
+                            opts=chem.default_opts(solver=solver, **options))
+        torch.cuda.synchronize()
+        assert torch.all(status == 0), (name, status)
+        assert np.all(np.abs(Td.cpu().numpy() - To) <= RTOL * np.abs(To) + ATOL), name
+        assert np.all(np.abs(Yd.cpu().numpy() - Yo) <= RTOL * np.abs(Yo) + ATOL), name
+
+
+COLD, HOT = [100.0, 150.0, 159.0, 200.0, 250.0], [8200.0, 8500.0, 9000.0]
+
+
+@pytest.mark.parametrize("make,T,dt", [(synth.mechanism_small, COLD, 1e-8), (synth.mechanism_small, HOT, 1e-10),
+                                       (synth.mechanism_53, COLD, 1e-8), (synth.mechanism_100, COLD, 1e-10)])
+def test_solves_outside_the_range(make, T, dt):
+    """The solve keeps its state beside the evaluation's scratch: outside the interval the general form must
+    stay inside it.  Changes of two last bits in T and Y (six draws) move the oracle's results by at
+    most 1e-5 of the tolerance here.  (The hot cells cool to 2300-2900 K: they enter the interval on the way.)"""
+    path = make().write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    rng = np.random.default_rng(5)
+    Y = np.ascontiguousarray(rng.dirichlet(np.ones(mech.K), size=len(COLD) + len(HOT)).T)
+    Y = np.ascontiguousarray(Y[:, :len(T)] if T is COLD else Y[:, len(COLD):])
+    _check_solves(mech, ora, np.array(T), Y, dt)
+    _check_solves(mech, ora, np.array(T), Y, dt, solvers=SOLVERS[:1], precision=chem.CHEM_PREC_MIXED_FF)
+
+
+def test_many_reactions_outside_the_range():
+    """More elementary reactions than the cell's vectors hold (R - n_pd > 12 K)."""
+    m = copy.deepcopy(synth.mechanism_small())
+    n_pd, copies = int((m.rtype != 0).sum()), 6
+    assert np.all(m.rtype[n_pd:] == 0)
+    at = np.concatenate([np.arange(n_pd)] + [np.arange(n_pd, m.R)] * copies)
+    rng = np.random.default_rng(2)
+    for name in ("rtype", "reac", "prod", "b", "Ea"):
+        setattr(m, name, getattr(m, name)[at].copy())
+    m.A = m.A[at] * rng.uniform(0.5, 2.0, at.size)
+    assert m.R - n_pd > 12 * m.K
+    path = m.write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    T, Y = _states(mech.K)
+    _check(mech, ora, T, Y)
+    cold = T < 200.0
+    _check_solves(mech, ora, T[cold], np.abs(Y[:, cold]), 1e-10)
+
+
 def test_species_on_both_sides(tmp_path):
     """A + B = 2 B (isomers): one species in three slots of a reaction."""
     text = open(os.path.join(os.path.dirname(__file__), "golden", "isomer_AB.txt")).read()
@@ -71,9 +126,8 @@ def test_species_on_both_sides(tmp_path):
     _check(mech, ora, *_states(mech.K))
 
 
-@pytest.mark.parametrize("change", ["barrier", "exponent", "prefactor"])
-def test_mechanisms_outside_the_limits(change):
-    m = copy.deepcopy(synth.mechanism_small())
+def _outside_the_limits(m, change):
+    m = copy.deepcopy(m)
     if change == "barrier":
         m.Ea[3] = 400e3     # beyond the table's 2^17 K ln 2
     elif change == "exponent":
@@ -81,6 +135,24 @@ def test_mechanisms_outside_the_limits(change):
         m.A[5] = 1e-180
     else:
         m.A[7] = 1e290
+    return m
+
+
+@pytest.mark.parametrize("make,change,dt", [(synth.mechanism_small, "barrier", 1e-10), (synth.mechanism_53, "barrier", 1e-10),
+                                            (synth.mechanism_53, "exponent", 1e-12)])
+def test_solves_without_an_interval(make, change, dt):
+    """Mechanisms that no temperature lets into fixed point, at flame temperatures.  (Two last bits in T and Y
+    move the oracle's results by at most 7e-4 of the tolerance; the pre-factor's case is no solvable
+    problem, nor is the exponent's with 10 species: the oracle itself fails there.)"""
+    path = _outside_the_limits(make(), change).write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    T, Y = synth.cells_uniform(3, mech.K, 4, (1000.0, 1300.0))
+    _check_solves(mech, ora, T, Y, dt)
+
+
+@pytest.mark.parametrize("change", ["barrier", "exponent", "prefactor"])
+def test_mechanisms_outside_the_limits(change):
+    m = _outside_the_limits(synth.mechanism_small(), change)
     path = m.write_temp()
     mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
     T, Y = _states(mech.K)
@@ -98,27 +170,37 @@ def test_mechanisms_outside_the_limits(change):
 def test_ln_a_change_moves_the_interval_of_a_captured_launch():
     w = synth.workload_small()
     path = w["mech"].write_temp()
-    mech = chem.Mechanism(path)
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
     lnA = chem.chem_get_lnA(mech)
     opts = chem.default_opts(use_graph=1)
-    T0, Y0 = _dev(w["T"][:40]), _dev(w["Y"][:, :40])
+    Th, Yh = w["T"][:40], np.ascontiguousarray(w["Y"][:, :40])
+    T0, Y0 = _dev(Th), _dev(Yh)
     T, Y = torch.empty_like(T0), torch.empty_like(Y0)
+    status = torch.empty(40, dtype=torch.int32, device="cuda")
 
-    def step(o):
+    def step(o, oracle):
         T.copy_(T0)
         Y.copy_(Y0)
-        chem.chem_integrate(mech, w["p_Pa"], T, Y, 1e-7, opts=o)
+        status.fill_(-1)
+        chem.chem_integrate(mech, w["p_Pa"], T, Y, 1e-7, RTOL, ATOL, status=status, opts=o)
         torch.cuda.synchronize()
+        assert torch.all(status == 0)
+        To, Yo, _, _, _ = oracle.integrate(w["p_Pa"], Th, Yh, 1e-7, RTOL, ATOL, nthreads=4)
+        assert np.all(np.abs(T.cpu().numpy() - To) <= RTOL * np.abs(To) + ATOL)
+        assert np.all(np.abs(Y.cpu().numpy() - Yo) <= RTOL * np.abs(Yo) + ATOL)
         return T.clone(), Y.clone()
 
-    first = step(opts)
+    first = step(opts, ora)
     far = lnA.copy()
-    far[4] = -1500.0        # a reaction switched off by its pre-factor: outside the fixed-point range
+    far[4] = -700.0         # a reaction switched off by its pre-factor: outside the fixed-point range
     chem.chem_set_lnA(mech, far)
-    replayed, direct = step(opts), step(chem.default_opts())
+    off = copy.deepcopy(w["mech"])
+    off.A[4] = np.exp(-700.0)
+    without = O.OracleMechanism(off.write_temp())
+    replayed, direct = step(opts, without), step(chem.default_opts(), without)
     assert torch.equal(replayed[0], direct[0]) and torch.equal(replayed[1], direct[1])
     chem.chem_set_lnA(mech, lnA)
-    again = step(opts)
+    again = step(opts, ora)
     assert torch.equal(first[0], again[0]) and torch.equal(first[1], again[1])
 
 
