@@ -204,9 +204,7 @@ struct Grp {
   // The larger magnitude, NaN if either is (a NaN error norm must reject the step): the bit patterns
   // with the sign masked are ordered like the values, NaN above infinity, so no FP64 comparison (which
   // takes the FP64 pipe for as long as an addition) is issued.
-  __device__ static unsigned long long mag(double a) {
-    return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffULL;
-  }
+  __device__ static unsigned long long mag(double a) { return fx_mag(a); }
   __device__ static double max_mag(double a, double b) { return __longlong_as_double((long long)max(mag(a), mag(b))); }
   // the largest magnitude in the group
   __device__ double max_nan(double v) const {
@@ -438,7 +436,7 @@ __device__ const double c_exp2_j32[64] = {
 __device__ inline double exp_fast(double x) {
   // |x| < 708 by an integer compare of the bit pattern with the sign masked (monotone for
   // non-negative doubles; NaN compares above), so the range check costs no FP64 instruction
-  if ((__double_as_longlong(x) & 0x7fffffffffffffffLL) >= 0x4086200000000000LL) return exp(x);
+  if (fx_mag(x) >= 0x4086200000000000ULL) return exp(x);
   const double shifter = 0x1.8p52;  // adding it rounds x 32/ln2 to an integer in the low bits
   const double t = fma(x, 0x1.71547652b82fep+5, shifter);
   const int k = (int)__double2loint(t);
@@ -1406,7 +1404,7 @@ __device__ void cell_jacobian_vjp(const DevMech& m, const Grp<G>& g, const CellS
 __device__ inline float f32_of(double v) {
   const long long b = __double_as_longlong(v);
   const unsigned sign = (unsigned)((unsigned long long)b >> 63) << 31;
-  const long long mag = b & 0x7fffffffffffffffLL;
+  const long long mag = (long long)fx_mag(v);
   if (mag >= 0x7ff0000000000000LL) return __uint_as_float(sign | 0x7f800000u | (mag > 0x7ff0000000000000LL));
   const long long r = mag + 0x0fffffffLL + ((mag >> 29) & 1);
   const long long fb = (r >> 29) - ((long long)(1023 - 127) << 23);
@@ -1526,9 +1524,13 @@ __device__ inline FF lu_recip<FF>(double c) {
 
 // |a| as an ordered integer key (bit pattern of a non-negative float / double)
 // (the sign bit masked off in the integer pipe, so that no FP64 instruction is spent on it)
-__device__ inline long long abs_key(double a) { return __double_as_longlong(a) & 0x7fffffffffffffffLL; }
-__device__ inline long long abs_key(float a) { return (long long)__float_as_int(fabsf(a)); }
-__device__ inline long long abs_key(FF a) { return (long long)__float_as_int(fabsf(a.hi)); }
+__device__ inline long long abs_key(double a) { return (long long)fx_mag(a); }
+__device__ inline long long abs_key(float a) {  // (see fx_mag)
+  unsigned b;
+  asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(b) : "r"(__float_as_uint(a)));
+  return (long long)b;
+}
+__device__ inline long long abs_key(FF a) { return abs_key(a.hi); }
 
 // U' = D^-1 U: the strictly upper part of row i times invdiag[i], over the N (N - 1) / 2 entries
 // in row order (each thread walks its entries in increasing order and advances its row as it goes).

@@ -43,6 +43,18 @@ CHEM_FX_FN double fx_from_bits(int64_t b) {
   return v;
 #endif
 }
+// The bits of |v|, ordered like the magnitudes, NaN above infinity.  Not fx_bits(v) & 0x7ff..f: the compiler
+// may make that an fabs, and abs.f64 passes a NaN through with its sign, so that CUDA's own NaN
+// (0xfff8...) compares as a negative integer.
+CHEM_FX_FN uint64_t fx_mag(double v) {
+#ifdef __CUDA_ARCH__
+  unsigned hi;
+  asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(hi) : "r"(__double2hiint(v)));
+  return (uint64_t)hi << 32 | (unsigned)__double2loint(v);
+#else
+  return (uint64_t)fx_bits(v) & 0x7fffffffffffffffULL;
+#endif
+}
 // high 64 bits of the signed product
 CHEM_FX_FN int64_t fx_mulhi(int64_t a, int64_t b) {
 #ifdef __CUDA_ARCH__
@@ -270,8 +282,7 @@ CHEM_FX_FN fx_t fx_log2(double x) {
 
 // 2^v of any double
 CHEM_FX_FN double fx_exp2_of(double v) {
-  const int64_t mag = fx_bits(v) & 0x7fffffffffffffffLL;
-  return mag < 0x408fe00000000000LL ? fx_exp2(fx_of(v)) : fx_exp2_wide(v);  // |v| < 1020
+  return fx_mag(v) < 0x408fe00000000000ULL ? fx_exp2(fx_of(v)) : fx_exp2_wide(v);  // |v| < 1020
 }
 
 // whether fx_log2 takes x: positive and normal

@@ -236,3 +236,26 @@ def test_third_body_sums_of_unphysical_states(efficiencies):
     assert ok.sum() >= n // 2
     # (a negative mean molar mass makes the density, and with it the scale, negative)
     assert np.all(np.abs(f.cpu().numpy() - fo)[:, ok] <= 1e-11 * np.abs(gross[:, ok]) + 1e-300)
+
+
+def test_non_finite_fall_off_factors():
+    """A negative or zero reduced pressure (a diverged trial state, an absent only collider) has no logarithm:
+    the source terms that it enters are NaN, as in the oracle, and not a finite number."""
+    m = copy.deepcopy(synth.mechanism_53())
+    troe = [r for r in range(m.R) if m.rtype[r] == synth.TYPE_TROE]
+    m.eff[troe[3]] = np.eye(m.K)[7]
+    path = m.write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    X = np.ones((4, m.K))
+    X[0] = 1e-3
+    X[0, np.argmax(m.eff[troe[0]])], X[0, np.argmin(m.eff[troe[0]])] = -1.0, 2.0  # [M] < 0 of several reactions
+    X[1, 7], X[2, 7] = 0.0, -1e-3                                                # [M] = 0 and < 0 of one
+    Y = X * m.W
+    Y = np.ascontiguousarray((Y / Y.sum(axis=1, keepdims=True)).T)
+    T = np.full(4, 1100.0)
+    f = torch.empty((mech.N, 4), dtype=torch.float64, device="cuda")
+    chem.chem_rates(mech, P, _dev(T), _dev(Y), f)
+    torch.cuda.synchronize()
+    fo = ora.rates(P, T, Y)
+    assert np.isnan(fo[:, :3]).any(axis=0).all() and np.isfinite(fo[:, 3]).all()
+    np.testing.assert_array_equal(np.isnan(f.cpu().numpy()), np.isnan(fo))

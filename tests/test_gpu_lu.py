@@ -75,3 +75,21 @@ def test_singular_flag():
     for variant in (0, 1, 2):
         *_, S = chem.chem_debug_lu(torch.from_numpy(A).cuda(), chem.CHEM_PREC_FP64, variant=variant)
         assert S.cpu().tolist() == [0, 1]
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("N", [1, 20, 53, 100])
+@pytest.mark.parametrize("variant", [0, 2])
+def test_columns_of_nan(N, prec, variant):
+    """NaN of either sign and any payload (all bits set is memory filled with 0xff) have the largest magnitudes: a
+    column of one pattern still has a pivot row, the lowest."""
+    A = np.random.default_rng(4).normal(size=(5, N, N))
+    for m, bits in ((1, -1), (2, 0x7FFFFFFFFFFFFFFF), (3, -0x8000000000000)):
+        A[m].view(np.int64)[...] = bits
+    A[4][:, N // 2].view(np.int64)[...] = -1
+    F, D, P, S = (t.cpu().numpy() for t in chem.chem_debug_lu(torch.from_numpy(A).cuda(), prec, variant=variant))
+    for m in (1, 2, 3):
+        np.testing.assert_array_equal(P[m], np.arange(N))
+        assert np.isnan(F[m].reshape(N * N, -1)).any(axis=1).all() and np.isnan(D[m].reshape(N, -1)).any(axis=1).all()
+    np.testing.assert_array_equal(np.sort(P[4]), np.arange(N))
+    np.testing.assert_array_equal(S, 0)
