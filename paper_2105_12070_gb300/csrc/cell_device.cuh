@@ -1638,14 +1638,19 @@ __device__ inline S lu_unpack(double c) {
   else return FF(__int_as_float(__double2hiint(c)), __int_as_float(__double2loint(c)));
 }
 
+// Key of a pivot candidate: |a|'s bits plus one, so that 0 is left for no entry.  Unsigned: the magnitude of a
+// NaN with all bits set is the largest signed integer, and its row has to count as an entry.
+template <typename S>
+__device__ inline unsigned long long pivot_key(S a) { return (unsigned long long)abs_key(a) + 1; }
+
 // The warp's pivot candidate: the lane with the largest key (0: no entry), ties to the lowest row, writes
 // (key, row, reciprocal) to out, integers as bits.  Two or three warp reductions (redux.sync) in
 // place of five rounds of five shuffles.
 template <typename S>
-__device__ inline void warp_candidate(long long key, int row, double inv, int none, int lane, double* out) {
+__device__ inline void warp_candidate(unsigned long long key, int row, double inv, int none, int lane, double* out) {
   bool mine = true;
   if (std::is_same<S, double>::value) {
-    const unsigned hi = (unsigned)((unsigned long long)key >> 32);
+    const unsigned hi = (unsigned)(key >> 32);
     const unsigned top = __reduce_max_sync(kFull, hi);
     mine = hi == top;
   }
@@ -1654,7 +1659,7 @@ __device__ inline void warp_candidate(long long key, int row, double inv, int no
   mine = mine && lo == top;
   const int first = __reduce_min_sync(kFull, mine ? row : 0x7fffffff);
   if (first == none ? lane == 0 : mine && row == first) {
-    out[0] = __longlong_as_double(key);
+    out[0] = __longlong_as_double((long long)key);
     out[1] = __longlong_as_double(row);
     out[2] = inv;
   }
@@ -1680,12 +1685,12 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
   bool ok = true;
   // pivot candidates of column 0
   {
-    long long best = 0;
+    unsigned long long best = 0;
     int bi = N;
     S bv = S(1.0f);
     for (int i = g.t; i < N; i += NT) {
       const S a = A[i * N];
-      const long long v = abs_key(a) + 1;
+      const unsigned long long v = pivot_key(a);
       if (v > best) { best = v; bi = i; bv = a; }
     }
     warp_candidate<S>(best, bi, lu_pack_recip(bv), N, g.lane(), cand + 3 * g.warp());
@@ -1693,12 +1698,12 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
   g.sync();
   for (int k = 0; k < N; ++k) {
     const double* cr = cand + (k & 1) * 3 * G;
-    long long best = __double_as_longlong(cr[0]);
+    unsigned long long best = (unsigned long long)__double_as_longlong(cr[0]);
     int bi = (int)__double_as_longlong(cr[1]);
     double bv = cr[2];
 #pragma unroll
     for (int w = 1; w < G; ++w) {
-      const long long ob = __double_as_longlong(cr[3 * w]);
+      const unsigned long long ob = (unsigned long long)__double_as_longlong(cr[3 * w]);
       const int oi = (int)__double_as_longlong(cr[3 * w + 1]);
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; bv = cr[3 * w + 2]; }
     }
@@ -1739,7 +1744,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
     // trailing update: column k+1 first (its entries are the next pivot's candidates, each thread
     // keeping the largest it produced), then the other columns
     const int mm = N - k - 1;
-    long long nb = 0;
+    unsigned long long nb = 0;
     int ni = N;
     S nv = S(1.0f);
     if (mm > 0) {
@@ -1750,7 +1755,7 @@ __device__ bool cell_lu_fused(const Grp<G>& g, S* A, int N, int* piv, int* perm,
       for (int i = g.t; i < mm; i += NT) {
         const S r = fma(-Ak[i * N], u0, T0[i * N]);
         T0[i * N] = r;
-        const long long v = abs_key(r) + 1;
+        const unsigned long long v = pivot_key(r);
         if (v > nb) { nb = v; ni = k + 1 + i; nv = r; }
       }
       warp_candidate<S>(nb, ni, lu_pack_recip(nv), N, g.lane(), cand + ((k + 1) & 1) * 3 * G + 3 * g.warp());
