@@ -381,7 +381,7 @@ int adjoint_enqueue(const DevMech& d, int num_sms, size_t max_smem, double p_cgs
                    : G == 4 ? (const void*)adjoint_kernel<4>
                             : (const void*)adjoint_kernel<8>;
   const int threads = 32 * G * cpc;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);  // (as in pick_launch)
   if (e != cudaSuccess) return fail(e, "cudaFuncSetAttribute");
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem);

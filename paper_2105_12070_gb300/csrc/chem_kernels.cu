@@ -456,7 +456,9 @@ int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, in
                        : variant == kLaunchJacobian ? rates_fn<true>(G)
                                                     : integrate_kernel_fn(G, variant);
   int occ = 0;
-  CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem));
+  // (always the device's limit: the attribute belongs to the function in the whole process, and a handle in
+  // another thread may be between its own setting and launch)
+  CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->max_smem));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, L.threads, L.smem));
   if (occ < 1) return set_err(CHEM_ESIZE, "kernel cannot be resident with the requested shared memory");
   const int cps = want_ctas_per_sm > 0 ? std::min(want_ctas_per_sm, occ) : occ;
@@ -1259,16 +1261,17 @@ int chem_debug_lu(const double* A, int N, int64_t n, int precision, int variant,
   const unsigned grid = (unsigned)std::min<int64_t>(n, 65535);
   const int bytes = precision == CHEM_PREC_MIXED ? 4 : 8;
   const size_t smem = sizeof(double) * (size_t)lu_probe_doubles(N, bytes);
+  const int most = (int)sizeof(double) * lu_probe_doubles(128, bytes);  // (the same for every call, as in pick_launch)
   if (precision == CHEM_PREC_FP64) {
-    CK(cudaFuncSetAttribute(lu_probe_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(lu_probe_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     lu_probe_kernel<double><<<grid, 64, smem, st>>>(A, N, n, variant, static_cast<double*>(factors),
                                                     static_cast<double*>(invdiag), perm, singular);
   } else if (precision == CHEM_PREC_MIXED) {
-    CK(cudaFuncSetAttribute(lu_probe_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(lu_probe_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     lu_probe_kernel<float><<<grid, 64, smem, st>>>(A, N, n, variant, static_cast<float*>(factors),
                                                    static_cast<float*>(invdiag), perm, singular);
   } else {
-    CK(cudaFuncSetAttribute(lu_probe_kernel<FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(lu_probe_kernel<FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     lu_probe_kernel<FF><<<grid, 64, smem, st>>>(A, N, n, variant, static_cast<FF*>(factors),
                                                 static_cast<FF*>(invdiag), perm, singular);
   }

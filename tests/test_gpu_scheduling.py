@@ -1,6 +1,10 @@
 """Scheduling options of chem_integrate (the GPU counterpart of the paper's load balancing,
 Sec. 2.2): results do not depend on how cells are scheduled, and the graph and batch paths give
 the same answer as the plain launch."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -118,3 +122,35 @@ def test_warps_per_cell_keep_the_bits(solver):
         if ref is None:
             ref = (T, Y)
         assert torch.equal(T, ref[0]) and torch.equal(Y, ref[1]), shape
+
+
+class _Side(ctypes.Structure):
+    _fields_ = [("mech", ctypes.c_void_p), ("T", ctypes.c_void_p), ("Y", ctypes.c_void_p), ("n", ctypes.c_int64),
+                ("J", ctypes.c_void_p), ("stream", ctypes.c_void_p)]
+
+
+def test_two_threads_with_their_own_handles(tmp_path):
+    """Two host threads, each with a handle of the same mechanism and a stream of its own, one with five
+    cells on an SM and one with three: the kernel's shared-memory limit, which belongs to the process, has to
+    hold for both."""
+    lib = str(tmp_path / "two_threads.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", lib,
+                    os.path.join(os.path.dirname(os.path.abspath(__file__)), "two_threads.cpp"), "-lpthread"], check=True)
+    fn = ctypes.CDLL(lib).two_threads
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
+    path = synth.mechanism_53().write_temp()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    keep, sides = [], []
+    for n in (5 * sms, 3 * sms):  # (the same kernel: 2 warps per cell)
+        mech, stream = chem.Mechanism(path), torch.cuda.Stream()
+        T, Y = synth.cells_uniform(1, mech.K, n, (1000.0, 1300.0))
+        T, Y = torch.from_numpy(T).cuda(), torch.from_numpy(np.ascontiguousarray(Y)).cuda()
+        J = torch.full((n, mech.N, mech.N), float("nan"), dtype=torch.float64, device="cuda")
+        keep.append((mech, stream, T, Y, J))
+        sides.append(_Side(mech.handle, T.data_ptr(), Y.data_ptr(), n, J.data_ptr(), stream.cuda_stream))
+    torch.cuda.synchronize()
+    jacobian = ctypes.cast(chem.load_library().chem_jacobian, ctypes.c_void_p)
+    failed = fn(jacobian, 1e6, ctypes.addressof(sides[0]), ctypes.addressof(sides[1]), 4000)
+    torch.cuda.synchronize()
+    assert failed == 0
+    assert all(torch.isfinite(k[4]).all() for k in keep)
