@@ -86,32 +86,18 @@ static __device__ __noinline__ double fx_rcp_wide(double a) { return 1.0 / a; }
 inline double fx_rcp_wide(double a) { return 1.0 / a; }
 #endif
 
-// 1/a by Newton's iteration r <- r + r (1 - m r) on the significand m in [1, 2) as integers, from the
-// FP32 approximate reciprocal (rcp.approx, error below 2^-22): two steps reach 2^-62, so the
+// 1/a of a normal a (exponent field 3 .. 2043) by Newton's iteration r <- r + r (1 - m r) on the significand
+// m in [1, 2) as integers: two steps from a seed with an error below 2^-22 reach 2^-62, so the
 // rounded result is within 0.51 units in the last place.  No FP64 instruction (a Newton iteration in
-// FP64 takes four).  Zero, subnormal, very large, infinite and NaN arguments take the division.
-// r: the reciprocal of the significand before rounding, in (1/2, 1], unit 2^-64.
-CHEM_FX_FN double fx_rcp(double a, uint64_t& r) {
+// FP64 takes four).  seed: the bits of a float next to 1/m in [1/2, 1].  r: the reciprocal of the significand
+// before rounding, in (1/2, 1], unit 2^-64.
+CHEM_FX_FN double fx_rcp_from(double a, uint32_t seed, uint64_t& r) {
   const int64_t b = fx_bits(a);
   const int ef = (int)((b >> 52) & 0x7ff);
-  if (ef < 3 || ef > 2043) {
-    r = 0;
-    return fx_rcp_wide(a);
-  }
   const uint64_t m = ((uint64_t)b << 11) | 0x8000000000000000ULL;  // unit 2^-63
-  const uint32_t mf = 0x3f800000u | ((uint32_t)(m >> 40) & 0x7fffffu);
-  uint32_t rf;
-#ifdef __CUDA_ARCH__
-  float s;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint_as_float(mf)));
-  rf = __float_as_uint(s);
-#else
-  float x;
-  std::memcpy(&x, &mf, 4);
-  x = 1.0f / x;
-  std::memcpy(&rf, &x, 4);
-#endif
-  // the seed in (1/2, 1] as a 32-bit fraction (1 itself as 1 - 2^-24, inside its error)
+  // the seed as a 32-bit fraction (1 itself as 1 - 2^-24, inside its error; for m next to 2 it may come out below
+  // 1/2, whose leading bit would then stand for twice its value)
+  const uint32_t rf = seed < 0x3f000000u ? 0x3f000000u : seed;
   const uint32_t r0 = rf >= 0x3f800000u ? 0xffffff00u : ((rf << 8) | 0x80000000u);
   r = (uint64_t)r0 << 32;  // unit 2^-64
   int64_t e = (int64_t)(0x8000000000000000ULL - fx_umulhi(m, r));  // 1 - m r, unit 2^-63, below 2^42
@@ -123,6 +109,30 @@ CHEM_FX_FN double fx_rcp(double a, uint64_t& r) {
   const uint64_t mant = (r >> 11) + ((r >> 10) & 1);
   const int64_t res = (b & 0xfffffffffffffLL) == 0 ? (int64_t)(2046 - ef) << 52 : ((int64_t)(2044 - ef) << 52) + (int64_t)mant;
   return fx_from_bits(res | (b & (int64_t)0x8000000000000000ULL));
+}
+
+// 1/a from the FP32 approximate reciprocal (rcp.approx, documented within one unit in the last place: 2^-23).
+// Zero, subnormal, very large, infinite and NaN arguments take the division (r = 0).
+CHEM_FX_FN double fx_rcp(double a, uint64_t& r) {
+  const int64_t b = fx_bits(a);
+  const int ef = (int)((b >> 52) & 0x7ff);
+  if (ef < 3 || ef > 2043) {
+    r = 0;
+    return fx_rcp_wide(a);
+  }
+  const uint32_t mf = 0x3f800000u | ((uint32_t)(b >> 29) & 0x7fffffu);
+  uint32_t rf;
+#ifdef __CUDA_ARCH__
+  float s;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint_as_float(mf)));
+  rf = __float_as_uint(s);
+#else
+  float x;
+  std::memcpy(&x, &mf, 4);
+  x = 1.0f / x;
+  std::memcpy(&rf, &x, 4);
+#endif
+  return fx_rcp_from(a, rf, r);
 }
 CHEM_FX_FN double fx_rcp(double a) {
   uint64_t r;

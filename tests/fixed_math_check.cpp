@@ -1,6 +1,6 @@
 // Host check of csrc/fixed_math.cuh against long double (64 or more significand bits): prints the
 // largest errors of fx_exp2 (units of the last place), fx_log2 and fx_of (units of 2^-52) and fx_rcp (units
-// of the last place; the host takes its FP32 seed from a division).
+// of the last place; the host takes its FP32 seed from a division, and from its neighbours up to two floats away).
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -23,7 +23,15 @@ int main(int argc, char** argv) {
   long double we = 0, wl = 0, wf = 0, wr = 0;
   auto check_exp = [&](fx_t x) { we = std::fmax(we, ulps(fx_exp2(x), std::exp2((long double)x / one))); };
   auto check_log = [&](double x) { wl = std::fmax(wl, std::fabs((long double)fx_log2(x) - std::log2((long double)x) * one)); };
-  auto check_rcp = [&](double a) { wr = std::fmax(wr, ulps(fx_rcp(a), 1.0L / a)); };
+  auto check_rcp = [&](double a) {
+    wr = std::fmax(wr, ulps(fx_rcp(a), 1.0L / a));
+    uint64_t m = ((uint64_t)fx_bits(a) & 0xfffffffffffffULL) | 0x3ff0000000000000ULL, r;
+    float x = 1.0f / (float)std::fmin(fx_from_bits((int64_t)m), 2.0 - std::ldexp(1.0, -23));
+    uint32_t rf;
+    std::memcpy(&rf, &x, 4);
+    // (the floats next to 1/2 from below are half as far apart: one more)
+    for (int s = -3; s <= 2; ++s) wr = std::fmax(wr, ulps(fx_rcp_from(a, rf + (uint32_t)s, r), 1.0L / a));
+  };
   for (int i = 0; i < 200000; ++i) {
     const double v = span * U(g);
     check_exp(fx_of(v));
@@ -43,6 +51,7 @@ int main(int argc, char** argv) {
     check_log(std::nextafter(x, 4.0));
     check_rcp(x);
     check_rcp(std::nextafter(x, 0.0));
+    check_rcp(x * (1.0 - std::ldexp(1.0, -24)));
     check_rcp(std::ldexp(std::nextafter(x, 4.0), i * 15 - 960));
   }
   // outside the normal range the reciprocal is the division's
