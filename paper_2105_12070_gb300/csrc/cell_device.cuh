@@ -829,8 +829,9 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   int eC = 0;
   int64_t* Cx = reinterpret_cast<int64_t*>(w.omega);  // (free until the production rates)
   if constexpr (!kDual) {
-    fxM = w.fxM && m.effx != nullptr;
     eC = (int)((__double_as_longlong(p * (invT * (1.0 / kRu))) >> 52) & 0x7ff);
+    // (a total of 2^-895 to infinity, so that the sums' unit below is a normal number)
+    fxM = w.fxM && m.effx != nullptr && (unsigned)(eC - 128) < 2047u - 128u;
   }
   S cp = cst<S>(0.0), dcp = cst<S>(0.0);
   int64_t* g2 = reinterpret_cast<int64_t*>(w.gRT);  // (g/RT) / ln 2 as fx

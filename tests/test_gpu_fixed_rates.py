@@ -259,3 +259,18 @@ def test_non_finite_fall_off_factors():
     fo = ora.rates(P, T, Y)
     assert np.isnan(fo[:, :3]).any(axis=0).all() and np.isfinite(fo[:, 3]).all()
     np.testing.assert_array_equal(np.isnan(f.cpu().numpy()), np.isnan(fo))
+
+
+@pytest.mark.parametrize("p", [1e-292, 1e-285, 1e-265, 1e-3])
+def test_third_body_sums_at_tiny_pressures(p):
+    """Concentrations next to the smallest normal number: the fixed-point sums hand over where their unit
+    would be below it."""
+    path = synth.mechanism_53().write_temp()
+    mech, ora = chem.Mechanism(path), O.OracleMechanism(path)
+    T, Y = synth.cells_uniform(8, mech.K, 16, (800.0, 2000.0))
+    f = torch.empty((mech.N, 16), dtype=torch.float64, device="cuda")
+    chem.chem_rates(mech, p, _dev(T), _dev(Y), f)
+    torch.cuda.synchronize()
+    fo, gross = ora.rates(p, T, Y, gross=True)
+    assert np.isfinite(fo).all() and np.isfinite(gross).all() and (gross > 0).any(axis=0).all()
+    assert np.all(np.abs(f.cpu().numpy() - fo) <= 1e-11 * gross + 1e-300)
