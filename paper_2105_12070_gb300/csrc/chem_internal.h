@@ -1,6 +1,7 @@
 // Internal layout shared by the host table builder (mech_tables.cpp) and the kernels
 // (chem_kernels.cu).  Not part of the public ABI.
 #pragma once
+#include <array>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -39,6 +40,8 @@ constexpr int kSpDoubles = 17;
 constexpr int kSpfRange = 20;
 constexpr int kSpfRows = 3 + 2 * kSpfRange;
 
+constexpr int kFxIntervalCount = 7;  // temperature intervals tried for fx_T
+
 struct HostMech {
   int K = 0, R = 0, E = 0;
   int n_elem = 0, n_tb = 0, n_fo = 0;  // counts in device order
@@ -56,6 +59,9 @@ struct HostMech {
   // Tables of the fixed-point rate evaluation (build_fx_tables).  Logarithms base 2.
   std::vector<double> fx_T;            // {lo, hi}: it takes temperatures inside (equal: none), chosen
                                        // so that every exponent stays inside the fixed-point range
+  bool fx_ok = false;                  // every table value but ln A fits its fixed-point format
+  // per candidate of fx_T: whether the exponents that do not depend on ln A keep their bounds (-1: not asked yet)
+  std::array<int8_t, kFxIntervalCount> fx_thermo_fits;
   std::vector<uint32_t> rx4;           // [R] slot species, one byte each (255 = empty)
   std::vector<int64_t> fxk;            // [3][R] log2 A * 2^52, b * 2^57, Ea/(Rc ln 2) * 2^46
   std::vector<int64_t> fxo;            // [3][n_fo] the same of the low-pressure limit
@@ -93,8 +99,10 @@ struct HostMech {
   std::vector<int> cl_rx;
 };
 
-// (Re)build the tables of the fixed-point rate evaluation from the others (after a change of ln A too).
+// Build the tables of the fixed-point rate evaluation from the others.
 void build_fx_tables(HostMech& m);
+// After a change of ln A: the first row of fxk and fx_T, all that depends on it.
+void update_fx_lnA(HostMech& m);
 
 // Parse the mechanism text file; false + message on error.
 bool parse_mechanism(const char* path, HostMech& m, std::string& err);

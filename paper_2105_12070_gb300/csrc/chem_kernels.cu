@@ -1119,12 +1119,12 @@ int chem_set_lnA(chem_mech* m, const double* lnA) {
   for (int r = 0; r < h.R; ++r)
     if (!std::isfinite(lnA[r])) return set_err(CHEM_EINVAL, "chem_set_lnA: non-finite value");
   for (int dr = 0; dr < h.R; ++dr) h.rxd[(size_t)dr * kRxDoubles] = lnA[h.order[dr]];
-  build_fx_tables(h);
+  update_fx_lnA(h);
   // the device tables are read by kernels in flight on any stream: wait for them first
   CK(cudaDeviceSynchronize());
   CK(cudaMemcpy(const_cast<double*>(m->dev.rxd), h.rxd.data(), h.rxd.size() * sizeof(double),
                 cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(const_cast<int64_t*>(m->dev.fxk), h.fxk.data(), h.fxk.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(const_cast<int64_t*>(m->dev.fxk), h.fxk.data(), (size_t)h.R * sizeof(int64_t), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(const_cast<double*>(m->dev.fx_T), h.fx_T.data(), h.fx_T.size() * sizeof(double), cudaMemcpyHostToDevice));
   return CHEM_OK;
 }

@@ -45,7 +45,6 @@ void build_fx_tables(HostMech& m) {
     for (int u = 0; u < 4; ++u) v |= (uint32_t)(ii[u] < 0 ? 255 : ii[u] & 255) << (8 * u);
     m.rx4[r] = v;
     const double* d = &m.rxd[(size_t)r * kRxDoubles];
-    m.fxk[r] = to_fixed(d[0] * log2e, 52, ok);
     m.rxd_t[r] = d[1];
     m.rxd_t[R + r] = d[2];
     m.fxk[R + r] = to_fixed(d[1], 57, ok);
@@ -112,69 +111,84 @@ void build_fx_tables(HostMech& m) {
       std::memcpy(&b, &m.sr_nu[e], 8);
       m.srx[(size_t)(e - m.sr_ptr[k]) * K + k] = (uint32_t)(m.sr_idx[e] & 0xffff) | (uint32_t)(b >> 48) << 16;
     }
-  // The temperature interval in which no exponent can leave its range.  Within an interval where
-  // every species stays in one of its two ranges, each term's magnitude is largest at an end, so
-  // bounds taken there hold inside: |log2 k| < 1000 for each rate constant and < 900 for the
-  // equilibrium exponent of a reaction (the sums of two rate exponents and of one with the
-  // equilibrium exponent stay below 2048), and |g/RT|/ln 2 < 1000 for each species (the range of the
-  // conversion).  lo > 128 keeps 1/T * 2^70 inside 63 bits, hi <= 8192 keeps log2 T below 13.
-  m.fx_T = {0.0, 0.0};
-  const double candidates[][2] = {{160.0, 8192.0}, {256.0, 8192.0}, {512.0, 8192.0}, {160.0, 4096.0}, {256.0, 4096.0},
-                                  {512.0, 4096.0}, {1024.0, 4096.0}};
-  for (const auto& cand : candidates) {
-    const double lo = cand[0], hi = cand[1];
-    bool fits = ok;
-    auto rate_fits = [&](double lnA, double b, double E) {
-      return (std::fabs(lnA) + std::fabs(E) / lo) * 1.4427 + std::fabs(b) * 13.0 < 1000.0;
-    };
-    // bound over [lo, hi] of |sum_k c_k (g_k/RT)| / ln 2
-    auto g_bound = [&](const std::pair<int, double>* terms, int n_terms) {
-      double ends[6] = {lo, hi};
-      int n_ends = 2;
-      for (int t = 0; t < n_terms; ++t) {
-        const double mid = m.spf[(size_t)2 * K + terms[t].first];
-        if (mid > lo && mid < hi) ends[n_ends++] = mid;
-      }
-      std::sort(ends, ends + n_ends);
-      double worst = 0.0;
-      for (int e = 0; e + 1 < n_ends; ++e) {
-        const double t0 = ends[e], t1 = ends[e + 1], mid = 0.5 * (t0 + t1);
-        double c[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int u = 0; u < n_terms; ++u) {
-          const std::pair<int, double>& t = terms[u];
-          const int first = 3 + (mid <= m.spf[(size_t)2 * K + t.first] ? 0 : kSpfRange) + 10;
-          for (int i = 0; i < 7; ++i) {
-            const double o = m.spf[(size_t)(first + i) * K + t.first];
-            int64_t x;
-            std::memcpy(&x, &o, 8);
-            c[i] += t.second * (i > 2 ? o : std::ldexp((double)x, i == 0 ? -52 : i == 1 ? -57 : -45));
-          }
+  m.fx_ok = ok;
+  m.fx_thermo_fits.fill(-1);
+  update_fx_lnA(m);
+}
+
+// The temperature interval in which no exponent can leave its range.  Within an interval where
+// every species stays in one of its two ranges, each term's magnitude is largest at an end, so
+// bounds taken there hold inside: |log2 k| < 1000 for each rate constant and < 900 for the
+// equilibrium exponent of a reaction (the sums of two rate exponents and of one with the
+// equilibrium exponent stay below 2048), and |g/RT|/ln 2 < 1000 for each species (the range of the
+// conversion).  lo > 128 keeps 1/T * 2^70 inside 63 bits, hi <= 8192 keeps log2 T below 13.
+static const double kFxIntervals[kFxIntervalCount][2] = {{160.0, 8192.0}, {256.0, 8192.0}, {512.0, 8192.0}, {160.0, 4096.0},
+                                                         {256.0, 4096.0}, {512.0, 4096.0}, {1024.0, 4096.0}};
+
+// Whether the species' and the equilibrium exponents keep their bounds over [lo, hi].
+static bool fx_thermo_fits(const HostMech& m, double lo, double hi) {
+  const int K = m.K;
+  // bound over [lo, hi] of |sum_k c_k (g_k/RT)| / ln 2
+  auto g_bound = [&](const std::pair<int, double>* terms, int n_terms) {
+    double ends[6] = {lo, hi};
+    int n_ends = 2;
+    for (int t = 0; t < n_terms; ++t) {
+      const double mid = m.spf[(size_t)2 * K + terms[t].first];
+      if (mid > lo && mid < hi) ends[n_ends++] = mid;
+    }
+    std::sort(ends, ends + n_ends);
+    double worst = 0.0;
+    for (int e = 0; e + 1 < n_ends; ++e) {
+      const double t0 = ends[e], t1 = ends[e + 1], mid = 0.5 * (t0 + t1);
+      double c[7] = {0, 0, 0, 0, 0, 0, 0};
+      for (int u = 0; u < n_terms; ++u) {
+        const std::pair<int, double>& t = terms[u];
+        const int first = 3 + (mid <= m.spf[(size_t)2 * K + t.first] ? 0 : kSpfRange) + 10;
+        for (int i = 0; i < 7; ++i) {
+          const double o = m.spf[(size_t)(first + i) * K + t.first];
+          int64_t x;
+          std::memcpy(&x, &o, 8);
+          c[i] += t.second * (i > 2 ? o : std::ldexp((double)x, i == 0 ? -52 : i == 1 ? -57 : -45));
         }
-        const double v = std::fabs(c[0]) + 13.0 * std::fabs(c[1]) + std::fabs(c[2]) / t0 +
-                         t1 * (std::fabs(c[3]) + t1 * (std::fabs(c[4]) + t1 * (std::fabs(c[5]) + t1 * std::fabs(c[6]))));
-        worst = std::max(worst, v);
       }
-      return worst;
+      const double v = std::fabs(c[0]) + 13.0 * std::fabs(c[1]) + std::fabs(c[2]) / t0 +
+                       t1 * (std::fabs(c[3]) + t1 * (std::fabs(c[4]) + t1 * (std::fabs(c[5]) + t1 * std::fabs(c[6]))));
+      worst = std::max(worst, v);
+    }
+    return worst;
+  };
+  for (int k = 0; k < K; ++k) {
+    const std::pair<int, double> one(k, 1.0);
+    if (!(g_bound(&one, 1) < 1000.0)) return false;
+  }
+  for (int r = 0; r < m.R; ++r) {
+    const int* ii = &m.rxi[(size_t)r * kRxInts];
+    std::pair<int, double> terms[4];
+    int n = 0;
+    for (int u = 0; u < 4; ++u)
+      if (ii[u] >= 0) terms[n++] = {ii[u], u < 2 ? -1.0 : 1.0};
+    if (!(g_bound(terms, n) < 900.0)) return false;
+  }
+  return true;
+}
+
+void update_fx_lnA(HostMech& m) {
+  const int R = m.R, nf = m.n_fo;
+  const long double log2e = 1.0L / std::log(2.0L);
+  bool ok = m.fx_ok;
+  for (int r = 0; r < R; ++r) m.fxk[r] = to_fixed(m.rxd[(size_t)r * kRxDoubles] * log2e, 52, ok);
+  m.fx_T = {0.0, 0.0};
+  for (int c = 0; ok && c < kFxIntervalCount; ++c) {
+    const double lo = kFxIntervals[c][0], hi = kFxIntervals[c][1];
+    auto rate_fits = [&](const double* d) {
+      return (std::fabs(d[0]) + std::fabs(d[2]) / lo) * 1.4427 + std::fabs(d[1]) * 13.0 < 1000.0;
     };
-    for (int k = 0; k < K && fits; ++k) {
-      const std::pair<int, double> one(k, 1.0);
-      fits = g_bound(&one, 1) < 1000.0;
-    }
-    for (int r = 0; r < R && fits; ++r) {
-      const double* d = &m.rxd[(size_t)r * kRxDoubles];
-      fits = rate_fits(d[0], d[1], d[2]);
-      if (fits && r < nf) {
-        const double* q = &m.fo[(size_t)r * kFoDoubles];
-        fits = rate_fits(q[0], q[1], q[2]);
-      }
-      const int* ii = &m.rxi[(size_t)r * kRxInts];
-      std::pair<int, double> terms[4];
-      int n = 0;
-      for (int u = 0; u < 4; ++u)
-        if (ii[u] >= 0) terms[n++] = {ii[u], u < 2 ? -1.0 : 1.0};
-      fits = fits && g_bound(terms, n) < 900.0;
-    }
-    if (fits) {
+    bool fits = true;
+    for (int r = 0; r < R && fits; ++r)
+      fits = rate_fits(&m.rxd[(size_t)r * kRxDoubles]) && (r >= nf || rate_fits(&m.fo[(size_t)r * kFoDoubles]));
+    if (!fits) continue;
+    if (m.fx_thermo_fits[c] < 0) m.fx_thermo_fits[c] = fx_thermo_fits(m, lo, hi);
+    if (m.fx_thermo_fits[c]) {
       m.fx_T = {lo, hi};
       break;
     }
