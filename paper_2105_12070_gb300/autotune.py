@@ -26,10 +26,13 @@ def _key(mech, precision: int, solver: int) -> str:
     return f"K{mech.K}-R{mech.R}-pd{mech.n_pd}-solver{solver}-prec{precision}-{name}"
 
 
-def candidates():
+def candidates(precision: int = chem.CHEM_PREC_FP64, solver: int = chem.CHEM_SOLVER_ROSENBROCK):
+    """(warps per cell, cells per CTA): 8 warps per CTA at most, and 10 of 2 per cell for the FP64 Rosenbrock
+    solve, whose smaller plan the library compiles for five cells (integrate_max_threads)."""
     out = []
     for G in (1, 2, 4, 8):
-        for cpc in range(1, 8 // G + 1):
+        warps = 10 if G == 2 and precision == chem.CHEM_PREC_FP64 and solver == chem.CHEM_SOLVER_ROSENBROCK else 8
+        for cpc in range(1, warps // G + 1):
             out.append((G, cpc))
     return out
 
@@ -58,7 +61,7 @@ def autotune(mech: chem.Mechanism, p_Pa: float, T, Y, dt: float, rtol: float = 1
     Y0 = Y[:, idx].contiguous().cuda()
     results = []
     stream = torch.cuda.current_stream()
-    for G, cpc in candidates():
+    for G, cpc in candidates(precision, solver):
         opts = chem.default_opts(precision=precision, solver=solver, warps_per_cell=G, cells_per_cta=cpc)
         try:
             Tt, Yt = T0.clone(), Y0.clone()
