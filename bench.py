@@ -47,20 +47,21 @@ METRIC = "cells/s per CFD Δt (53 sp, rtol 1e-6), batched/mixed vs plain FP64; %
 L2_BYTES = 129 * 2 ** 20
 OPCOUNT_FILE = os.path.join(ROOT, "tests", "golden", "opcount_mech53.json")
 # FLOPs per operation.  Unit weights: add, mul, div, exp and log count one each (the conservative
-# count, `roofline.frac`).  Weighted: an exp or log counts its cost in FMA flops, the measured FP64
-# pipe throughput of the library exp and log relative to DFMA on GB300 (17 and 31 DFMA),
-# reported beside it as `roofline.frac_weighted`.
+# count, `roofline.frac`).  Weighted: an exp or log counts as many flops as CUDA's exp and log take on
+# the FP64 pipe of GB300 (17 and 31 DFMA), reported beside it as `roofline.frac_weighted`: the method's
+# work in FP64 units.  It is no fraction of a roofline, as the kernels evaluate their exponentials
+# and logarithms on the integer pipe.
 UNIT_WEIGHTS = {"add": 1, "mul": 1, "div": 1, "exp": 1, "log": 1}
 FLOP_WEIGHTS = {"add": 1, "mul": 1, "div": 1, "exp": 2 * 17, "log": 2 * 31}
 # DRAM bytes (read + write) of the integrate kernel as a function of the cells of a launch,
 # fitted to two ncu captures (dram__bytes_read.sum + dram__bytes_write.sum, the timed launch of
 # `bench.py --cells n --dt 1e-9 --warmup 1 --steps 1`) of the current kernel on evenly spaced
-# slices of the shear-layer field: 1 566 720 B read / 0 B written at 608 cells and 3 371 264 B /
-# 0 B at 4864 cells, i.e. fixed bytes (mechanism tables, the CTAs' first touches) plus bytes per
+# slices of the shear-layer field: 1 960 960 B read and 32 256 B written at 608 cells, 3 684 096 B and
+# 122 368 B at 4864 cells, i.e. fixed bytes (mechanism tables, the CTAs' first touches) plus bytes per
 # cell (its state; the rest of the state is read from L2, where the library's staging copy in
 # the same call left it, and the results stay in L2 until the copy back).
-TRAFFIC_FIT = {"fixed": 1566720 - 608 * (3371264 - 1566720) / (4864 - 608),
-               "per_cell": (3371264 - 1566720) / (4864 - 608), "cells": (608, 4864)}
+TRAFFIC_FIT = {"fixed": 1993216 - 608 * (3806464 - 1993216) / (4864 - 608),
+               "per_cell": (3806464 - 1993216) / (4864 - 608), "cells": (608, 4864)}
 
 
 def parse_args(argv=None):
@@ -333,7 +334,9 @@ def roofline_block(steps_np, rej_np, kern_ms_per_launch, peak, rosen, n_cells, t
             "achieved_weighted": a_w if ok else None,
             "frac_weighted": a_w / peak["tflops"] if ok else None,
             "frac_weighted_of_measured": a_w / peak["measured_tflops"] if ok else None,
-            "weights_weighted": "exp 34 and log 62 flops (17 and 31 DFMA of FP64 pipe time)",
+            "weights_weighted": "exp 34 and log 62 flops (17 and 31 DFMA, the cost of CUDA's FP64 exp and log; the "
+                                "kernels evaluate them on the integer pipe, so the weighted fields are no "
+                                "roofline fraction)",
             "flops_per_attempt": per_unit["per_attempt"], "flops_per_accepted_step": per_unit["per_accepted"],
             "flops_per_attempt_weighted": per_w["per_attempt"],
             "flops_per_accepted_step_weighted": per_w["per_accepted"]}

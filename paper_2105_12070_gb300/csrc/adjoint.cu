@@ -50,7 +50,8 @@ AdjPlan make_adj_plan(int K, int R, int n_pd, int n_pairs, int G) {
   p.nAB2 = round2(2 * R + 2 * n_pd);
   // matrix region, reused by the phases of a step: the Jacobian at y_n (-J, then W and its LU in
   // place) with the per-reaction scratch of the evaluations behind it; the dual-number per-reaction
-  // scratch
+  // scratch.  (SA + K K, what the assembly took before it worked in place, keeps the limit on the
+  // mechanism's size where it was.)
   p.off_M = 0;
   const int msize = round2(std::max({p.SA + K * K, K * K + 8 * R, 16 * R}));
   // 18 vectors: y f ys rhs u0..u3 ub0..ub3 (v_i overwrite ub_i) ybar lam invdiag wv (+2 spare)
@@ -347,7 +348,10 @@ int adjoint_enqueue(const DevMech& d, int num_sms, size_t max_smem, double p_cgs
   // Launch shape, 8 warps per CTA at most.  A small mechanism's cell keeps one warp busy: one each, spread
   // over all SMs (a step of the 10-species mechanism has no loop of more than three passes by 32 lanes,
   // and a single warp needs no barriers).  Else two cells of 4 warps when both working sets fit and there
-  // is more than one cell per SM, else one of 8 warps.
+  // is more than one cell per SM, else one of 8 warps.  The line lies where calls of few cells begin to
+  // lose; sweeps of 100 / 300 / 1000 cells in ms, one warp against four or eight: 10 species / 30 reactions
+  // 77 93 119 against 102 105 225; 12 / 60 473 549 646 against 559 564 1186; 16 / 80 192 222 271 against
+  // 207 207 324; 20 / 100 262 267 369 against 244 241 542; 31 / 150 710 724 1096 against 639 596 1371.
   const int64_t per_sm = (ncells + num_sms - 1) / num_sms;
   int G, cpc;
   AdjPlan plan;

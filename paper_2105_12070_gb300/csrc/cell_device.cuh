@@ -773,7 +773,7 @@ __device__ CellScalarsT<S> cell_rates_any(const DevMech& m, const Grp<G>& g, dou
 // logarithms of the rate and equilibrium constants are summed in 64-bit fixed point and the
 // exponentials and logarithms evaluated there (fixed_math.cuh), from tables with the constant
 // factors multiplied in.  Bound by FP64 issue (64 clocks per warp instruction and sub-partition):
-// a plain reaction takes 5 FP64 instructions here against 39 in the general form, a species' thermo
+// a plain reaction takes 4 FP64 instructions here against 39 in the general form, a species' thermo
 // 17 against about 45.
 // The tables are laid out so that consecutive threads read consecutive words: at this pace the
 // strided records of the general form would be bound by L1 wavefronts.
@@ -819,12 +819,17 @@ __device__ CellScalarsT<S> cell_rates_fx(const DevMech& m, const Grp<G>& g, doub
   const int64_t L2s = L2 << 7;
   // Third-body sums in fixed point (w.fxM: the source-term kernel, whose four warps per sub-partition
   // saturate the FP64 pipe; inside the integrators, with half as many, the sums wait for their tables and
-  // gain nothing): concentrations in units of 2^-60 of the power of two above the total p/(Ru T),
-  // efficiencies normalised per reaction.  The C_k add up to the total, so with no negative one beyond
-  // 1/64 of it (K <= 128) the sums of the 64-bit high products stay below 2^62; a state that breaks
-  // this takes the FP64 sums.  Where a reaction's efficiencies lie within a factor of 16 (the host's
-  // rule) the rounding, 2^-60 of the largest term each, is below that of the FP64 sum, at 20 clocks per
-  // term in place of 64-76: source terms of 53 species x 65536 1.59 -> 1.37 ms.
+  // gain nothing): concentrations in units of 2^-60 of the power of two 2^e at or below the total p/(Ru T),
+  // efficiencies normalised per reaction to a largest one in [1/2, 1).  The C_k add up to the total, so with
+  // no negative one of 2^(e-5) or more (K <= 128: negatives below 4 2^e, positives below 6 2^e) the sums
+  // of the 64-bit high products, unit 2^-58, stay below 2^62; a state that breaks this takes the FP64 sums.
+  // A concentration is rounded to 1/8 of a product's unit and every product truncated to one, half of which is
+  // added back.  The host's rule keeps a reaction's efficiencies within a factor of 16, so that [M] is at
+  // least 2^53 units: 5 K / 8 units are 2^-48 of it at worst for 53 species, as is the bound of the FP64 sum's
+  // two chains.  Typical states have 2^56 units and more, and the source terms' error against quadruple
+  // precision did not change (4e-16 and 1.2e-15 of the 2-norm).
+  // At 20 clocks per term in place of 64-76: source terms of 53 species x 65536 1.59 -> 1.37 ms.  One
+  // reaction outside the rule (a zero efficiency, say) leaves the whole mechanism to the FP64 sums.
   bool fxM = false;
   int eC = 0;
   int64_t* Cx = reinterpret_cast<int64_t*>(w.omega);  // (free until the production rates)
@@ -1390,7 +1395,6 @@ __device__ void cell_jacobian_vjp(const DevMech& m, const Grp<G>& g, const CellS
   g.sync();
 }
 
-// ------------------------------------------------------------------------------------------
 // ------------------------------------------------------------------------------------------
 // FP32 pairs ("float-float"): a value hi + lo with |lo| <= ulp(hi) / 2 carries about 48
 // significand bits in FP32 arithmetic (Dekker 1971; Knuth's two-sum and the FMA two-product),

@@ -90,7 +90,6 @@ struct HostMech {
   std::vector<int> pr_ptr;             // [K + 1]
   std::vector<int> pr_pd;
   std::vector<double> pr_nu;
-  std::vector<int> pr_row;             // row of each (row, reaction) pair
   std::vector<int> pr_rows;            // rows with pairs, shortest lists first
   // Column lists (products with J^T): for species column j, the per-reaction scratch indices
   // of dq/dC_j and their reactions
@@ -127,7 +126,6 @@ struct DevMech {
   const int* pr_ptr;
   const int* pr_pd;
   const double* pr_nu;
-  const int* pr_row;
   const int* pr_rows;
   int n_pairs, n_prows;
   // reaction split of the rate evaluation for groups of 2, 4 and 8 warps (index 1, 2, 3; index 0

@@ -408,8 +408,8 @@ void launch_integrate(const Launch& L, cudaStream_t st, const DevMech& d, Integr
 // The kernels of pick_launch: one of the integrate variants (integrate.h), or the one-shot ones.
 enum : int { kLaunchRates = 100, kLaunchJacobian = 101 };
 
-// Launch shape: G warps per cell, as many cells per CTA as the shared memory allows (at most 8
-// warps per CTA, 15 named barriers), one persistent CTA wave.
+// Launch shape: G warps per cell, as many cells per CTA as the shared memory allows (at most 8 warps per
+// CTA, 10 for the FP64 solve and Jacobians with 2 warps per cell; 15 named barriers), one persistent CTA wave.
 int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, int want_ctas_per_sm, int variant,
                 Launch& L) {
   const int kind = variant == kLaunchRates ? kPlanRates : variant == kLaunchJacobian ? kPlanCompact : integrate_plan(variant);
@@ -418,7 +418,8 @@ int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, in
   int G = want_G;
   if (G <= 0) {
     // automatic: about 8 warps per SM -- G = 8 / (cells that fit), a power of two in 1..8, and
-    // at least 2 warps per cell from 32 species up
+    // at least 2 warps per cell from 32 species up.  (The cells are counted with the full plan for every
+    // variant.)
     const size_t per_cell2 = (size_t)make_plan(m->host.K, m->host.R, m->dev.n_pd, 2).total * sizeof(double);
     const int fit = (int)std::max<size_t>(1, m->max_smem / per_cell2);
     G = 1;
@@ -428,6 +429,10 @@ int pick_launch(const chem_mech* m, int64_t ncells, int want_G, int want_cpc, in
     // A call with few cells per SM gives each of them the warps that would stand idle.  Only where
     // every thread of the group holds at most one species either way: the reductions then add the
     // same numbers in the same order, so that a cell's result does not depend on its company.
+    // From 64 reactions: with two passes of a warp or fewer there is nothing to share.  Solves of 152 cells,
+    // ms with 1, 2, 4 and 8 warps per cell: 10 species / 30 reactions 66.2 68.5 69.9 78.3; 16 / 48 29.5 28.2
+    // 28.4 31.5; 16 / 80 70.1 65.9 66.4 73.0; 20 / 100 103 94.8 93.4 102; 31 / 150 327 265 257 273; 53 / 325 with 2, 4
+    // and 8: 515 430 427, and 304 cells 539 462 870.  (Below 32 species 4 would be better than the 8 taken here.)
     if (32 * G >= m->host.K && m->host.R >= 64)
       while (G < CHEM_FEW_CELLS_MAX_G && 2 * G * per_sm <= 8) G *= 2;
   }
@@ -640,7 +645,6 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   const size_t o_prp = place(h.pr_ptr.size() * sizeof(int));
   const size_t o_prd = place(std::max<size_t>(1, h.pr_pd.size()) * sizeof(int));
   const size_t o_prn = place(std::max<size_t>(1, h.pr_nu.size()) * sizeof(double));
-  const size_t o_prr = place(std::max<size_t>(1, h.pr_row.size()) * sizeof(int));
   const size_t o_prs = place(std::max<size_t>(1, h.pr_rows.size()) * sizeof(int));
   const size_t o_ord = place(h.order.size() * sizeof(int));
   const size_t o_clp = place(h.cl_ptr.size() * sizeof(int));
@@ -676,7 +680,6 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   put(o_prp, h.pr_ptr.data(), h.pr_ptr.size() * sizeof(int));
   put(o_prd, h.pr_pd.data(), h.pr_pd.size() * sizeof(int));
   put(o_prn, h.pr_nu.data(), h.pr_nu.size() * sizeof(double));
-  put(o_prr, h.pr_row.data(), h.pr_row.size() * sizeof(int));
   put(o_prs, h.pr_rows.data(), h.pr_rows.size() * sizeof(int));
   put(o_ord, h.order.data(), h.order.size() * sizeof(int));
   put(o_clp, h.cl_ptr.data(), h.cl_ptr.size() * sizeof(int));
@@ -721,7 +724,6 @@ int chem_load_mechanism(const char* path, chem_mech** out) {
   d.pr_ptr = reinterpret_cast<const int*>(b + o_prp);
   d.pr_pd = reinterpret_cast<const int*>(b + o_prd);
   d.pr_nu = reinterpret_cast<const double*>(b + o_prn);
-  d.pr_row = reinterpret_cast<const int*>(b + o_prr);
   d.pr_rows = reinterpret_cast<const int*>(b + o_prs);
   d.order = reinterpret_cast<const int*>(b + o_ord);
   d.cl_ptr = reinterpret_cast<const int*>(b + o_clp);

@@ -55,7 +55,10 @@ constexpr int integrate_min_ctas(int G) { return G == 1 ? 2 : 1; }
 
 // Threads per CTA of a variant: the default's compact plan puts five cells of 53 species on an SM, 10 warps
 // of 2 per cell at 168 registers a thread (three warps on two of the four sub-partitions).
-// Shear layer of 6080 cells: 2454 -> 2784 cells/s against four cells at 244 registers.
+// Shear layer of 6080 cells: 2454 -> 2784 cells/s against four cells at 244 registers.  2432 cells, ms with 320
+// and with 256 threads: 40 species / 200 reactions 167 and 180, 53 / 325 415 and 463; where only four cells
+// fit an SM the smaller register budget costs nothing: 58 / 330 904 and 905, 60 / 360 1409 and 1405, 62 / 390
+// 890 and 893.
 constexpr int integrate_max_threads(int G, int variant) {
   return (G == 2 && variant == kIntegrateFp64) ? CHEM_MAX_THREADS_PER_CTA / 4 * 5 : CHEM_MAX_THREADS_PER_CTA;
 }

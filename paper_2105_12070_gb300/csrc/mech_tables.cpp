@@ -317,10 +317,8 @@ void build_jacobian_plan(HostMech& m) {
     }
   }
   m.pr_ptr[K] = (int)m.pr_pd.size();
-  m.pr_row.assign(m.pr_pd.size(), 0);
   m.pr_rows.clear();
   for (int k = 0; k < K; ++k) {
-    for (int c = m.pr_ptr[k]; c < m.pr_ptr[k + 1]; ++c) m.pr_row[c] = k;
     if (m.pr_ptr[k + 1] > m.pr_ptr[k]) m.pr_rows.push_back(k);
   }
   std::stable_sort(m.pr_rows.begin(), m.pr_rows.end(), [&](int a, int b) {

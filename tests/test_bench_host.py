@@ -96,7 +96,7 @@ def test_budget_guard(bench):
 
 
 def test_budget_projection(bench):
-    """The driver's run: 20 steps of 83.3 s after ~25 s of start-up and CPU legs fit in 1740 s
+    """A run of 20 steps of 83.3 s after ~25 s of start-up and CPU legs fit in 1740 s
     with the 20 s reserve; at 85.2 s per step only 19 do."""
     b = bench.Budget(1740.0, t0=0.0)
     pj = b.projection(1, 20, 83.3, 20.0, now=25.0 + 83.3)
