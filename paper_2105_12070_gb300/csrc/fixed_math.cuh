@@ -97,10 +97,9 @@ CHEM_FX_FN double fx_rcp_from(double a, uint32_t seed, uint64_t& r) {
   const int64_t b = fx_bits(a);
   const int ef = (int)((b >> 52) & 0x7ff);
   const uint64_t m = ((uint64_t)b << 11) | 0x8000000000000000ULL;  // unit 2^-63
-  // the seed as a 32-bit fraction (1 itself as 1 - 2^-24, inside its error; for m next to 2 it may come out below
-  // 1/2, whose leading bit would then stand for twice its value)
-  const uint32_t rf = seed < 0x3f000000u ? 0x3f000000u : seed;
-  const uint32_t r0 = rf >= 0x3f800000u ? 0xffffff00u : ((rf << 8) | 0x80000000u);
+  // the seed as a 32-bit fraction (1 itself as 1 - 2^-24, inside its error).  Its leading bit is added, not set: for
+  // m next to 2 the seed may come out below 1/2, as 0x3effffff, whose shifted bits carry out and leave 2^31 - 2^8
+  const uint32_t r0 = seed >= 0x3f800000u ? 0xffffff00u : (seed << 8) + 0x80000000u;
   r = (uint64_t)r0 << 32;  // unit 2^-64
   int64_t e = (int64_t)(0x8000000000000000ULL - fx_umulhi(m, r));  // 1 - m r, unit 2^-63, below 2^42
   r += (uint64_t)((int64_t)((uint64_t)fx_mulhi((int64_t)(r >> 1), e << 21)) >> 19);
