@@ -5,9 +5,9 @@
 // evaluation, most of its FP64 instructions, run on the integer pipe.  Logarithms are base 2 and
 // kept as int64 with 52 fraction bits ("fx", range +-2048): ln k = ln A + b ln T - E/T is a sum
 // of terms of size 10-100, whose FP64 rounding errors are 2^-50..2^-47 absolute.  In fx, in units of 2^-52:
-// log2 A is rounded (1/2), the products with b and 1/T are truncated (below 1 each), and the error of
-// log2 T (below 0.9) counts |b| times, as does, for g/RT, a_1's, whose a_6/T is doubled after its
-// truncation (below 2).  For |b| <= 2 the sum is within 4.5 units, 2^-50, of the exact one.
+// log2 A is rounded (1/2), the products with b and with 1/T are truncated (below 1 each), and the error of
+// log2 T (below 0.9) counts |b| times: for |b| <= 2 the sum is within 4.5 units, 2^-49.8, of the exact
+// one.  In a species' g/RT the term a_6/T is doubled after its truncation (below 2).
 // Everything here also compiles for the host.
 #pragma once
 #include <cstdint>
